@@ -10,6 +10,7 @@
 #include <new>
 #include <vector>
 
+#include "fixed.cuh"
 #include "qcd_handles.h"
 
 namespace qcd {
@@ -103,10 +104,13 @@ qcd_status check_cuda(cudaError_t e, const char *what)
 
 // ----------------------------------------------------------------- sizes
 
-int spinor_planes(int prec) { return (prec == QCD_PREC_F64 || prec == QCD_PREC_DF64) ? 12 : prec == QCD_PREC_F32 ? 6 : 3; }
+int spinor_planes(int prec) { return (prec == QCD_PREC_F64 || prec == QCD_PREC_DF64 || prec == kPrecFix) ? 12 : prec == QCD_PREC_F32 ? 6 : 3; }
 size_t spinor_plane_elem_bytes(int) { return 16; }
 size_t spinor_half_bytes(int prec, int stride) { return (size_t)spinor_planes(prec) * 16 * stride; }
-size_t spinor_half_norm_bytes(int prec, int stride) { return prec == QCD_PREC_F16 ? (size_t)4 * stride : 0; }
+size_t spinor_half_norm_bytes(int prec, int stride)
+{
+    return prec == QCD_PREC_F16 || prec == kPrecFix ? (size_t)4 * stride : 0;
+}
 
 int gauge_planes(int prec, int recon)
 {
@@ -296,6 +300,11 @@ FieldView view_of(const qcd_spinor *s)
     return f;
 }
 
+static std::string ws_name(const std::string &name, int prec, int rhs_log2)
+{
+    return name + "/p" + std::to_string(prec) + "/n" + std::to_string(rhs_log2);
+}
+
 FieldView ws_field(const qcd_lattice *lat, const std::string &name, int nh, int prec, int rhs_log2)
 {
     // fits an int: lattice creation demands h * Lmax < 2^32 with Lmax >=
@@ -304,7 +313,7 @@ FieldView ws_field(const qcd_lattice *lat, const std::string &name, int nh, int 
     const int stride = rhs_log2 == 0 ? lat->stride : (ne + 63) / 64 * 64;
     const size_t db = spinor_half_bytes(prec, stride), nb = spinor_half_norm_bytes(prec, stride);
     char *base = static_cast<char *>(
-        workspace(lat, name + "/p" + std::to_string(prec) + "/n" + std::to_string(rhs_log2), nh * (db + nb)));
+        workspace(lat, ws_name(name, prec, rhs_log2), nh * (db + nb)));
     FieldView f;
     f.nh = nh;
     f.h = ne;
@@ -331,17 +340,18 @@ cudaError_t zero_now(void *p, size_t n)
     return e == cudaSuccess ? cudaStreamSynchronize(cudaStreamLegacy) : e;
 }
 
+static std::mutex derived_mu;  // concurrent solves may share one gauge field
+
 GaugeView gauge_view(const qcd_gauge *g, int prec, int recon, cudaStream_t s, qcd_status *st)
 {
     *st = QCD_OK;
     const int stride = g->lat->stride;
-    if (prec == g->prec && recon == g->recon) return GaugeView{g->data, stride};
+    if (prec == g->prec && recon == g->recon) return GaugeView{g->data, stride, nullptr};
     const int key = prec * 100 + recon;
     auto *gm = const_cast<qcd_gauge *>(g);
-    static std::mutex derived_mu;  // concurrent solves may share one gauge field
     std::lock_guard<std::mutex> lk(derived_mu);
     auto it = gm->derived.find(key);
-    if (it != gm->derived.end()) return GaugeView{it->second.first, stride};
+    if (it != gm->derived.end()) return GaugeView{it->second.first, stride, nullptr};
     // The copy is converted on `s` and then published to every stream, so
     // the conversion must be complete first: it is built outside stream
     // capture and the stream is synchronised before the pointer is stored.
@@ -350,7 +360,7 @@ GaugeView gauge_view(const qcd_gauge *g, int prec, int recon, cudaStream_t s, qc
         cudaGetLastError();
         *st = fail(QCD_ERR_INVALID_ARG, "gauge copy: a copy in a new precision is built outside stream capture "
                                         "(call qcd_gauge_prepare first)");
-        return GaugeView{nullptr, stride};
+        return GaugeView{nullptr, stride, nullptr};
     }
     const size_t bytes = gauge_bytes(prec, recon, stride);
     void *p = nullptr;
@@ -358,30 +368,66 @@ GaugeView gauge_view(const qcd_gauge *g, int prec, int recon, cudaStream_t s, qc
     if (cudaMalloc(&p, bytes) != cudaSuccess) {
         cudaGetLastError();
         *st = fail(QCD_ERR_OOM, "gauge copy: cudaMalloc(%zu) failed", bytes);
-        return GaugeView{nullptr, stride};
+        return GaugeView{nullptr, stride, nullptr};
     }
-    const GaugeView dst{p, stride}, src{g->data, stride};
+    const GaugeView dst{p, stride, nullptr}, src{g->data, stride, nullptr};
     cudaError_t e = launch_gauge_convert(dst, prec, recon, src, g->prec, g->recon, g->lat->geom, s);
     if (e != cudaSuccess) {
         cudaFree(p);
         *st = check_cuda(e, "gauge copy");
-        return GaugeView{nullptr, stride};
+        return GaugeView{nullptr, stride, nullptr};
     }
     if (recon == 8) {
         *st = check_recon8(dst, prec, nullptr, src, g->prec, g->recon, g->lat->geom, s, "gauge copy");
         if (*st != QCD_OK) {
             cudaFree(p);
-            return GaugeView{nullptr, stride};
+            return GaugeView{nullptr, stride, nullptr};
         }
     }
     e = cudaStreamSynchronize(s);  // other streams may use the copy as soon as it is stored
     if (e != cudaSuccess) {
         cudaFree(p);
         *st = check_cuda(e, "gauge copy");
-        return GaugeView{nullptr, stride};
+        return GaugeView{nullptr, stride, nullptr};
     }
     gm->derived[key] = {p, bytes};
     return dst;
+}
+
+GaugeView hop_links(const qcd_gauge *g, int prec, int recon, cudaStream_t s, qcd_status *st)
+{
+    GaugeView v = gauge_view(g, prec, recon, s, st);
+    if (*st != QCD_OK || prec != QCD_PREC_F64 || g->prec != prec || g->recon != recon) return v;
+    auto *gm = const_cast<qcd_gauge *>(g);
+    std::lock_guard<std::mutex> lk(derived_mu);
+    if (g->fix_state == qcd_gauge::FIX_STALE) {
+        // as for a derived copy: complete before any stream may read it
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+            cudaGetLastError();
+            return v;
+        }
+        DeviceLock dl(device_mutex());
+        if (!gm->fix && cudaMalloc(&gm->fix, gauge_bytes(QCD_PREC_F64, 18, g->lat->stride)) != cudaSuccess) {
+            cudaGetLastError();
+            gm->fix = nullptr;
+            gm->fix_state = qcd_gauge::FIX_UNFIT;  // not asked for again before the next upload
+            return v;
+        }
+        bool fits = false;
+        const cudaError_t e = gauge_to_fix(static_cast<int4 *>(gm->fix), v, recon, g->lat->geom, s, &fits);
+        if (e != cudaSuccess) {
+            *st = check_cuda(e, "fixed-point links");
+            return v;
+        }
+        gm->fix_state = fits ? qcd_gauge::FIX_READY : qcd_gauge::FIX_UNFIT;
+        if (!fits) {
+            cudaFree(gm->fix);
+            gm->fix = nullptr;
+        }
+    }
+    if (g->fix_state == qcd_gauge::FIX_READY) v.fix = static_cast<const int4 *>(g->fix);
+    return v;
 }
 
 // ----------------------------------------------------------------- hop
@@ -423,13 +469,17 @@ cudaError_t launch_dslash_f64(int recon, const DslashLaunch &a, cudaStream_t s);
 cudaError_t launch_dslash_f32(int recon, const DslashLaunch &a, cudaStream_t s);
 cudaError_t launch_dslash_f16(int recon, const DslashLaunch &a, cudaStream_t s);
 cudaError_t launch_dslash_bf16(int recon, const DslashLaunch &a, cudaStream_t s);
+cudaError_t launch_dslash_fix_d0(const DslashLaunch &a, cudaStream_t s);
+cudaError_t launch_dslash_fix_d1(const DslashLaunch &a, cudaStream_t s);
 cudaError_t launch_dslash_df64_d0(int recon, const DslashLaunch &a, cudaStream_t s);
 cudaError_t launch_dslash_df64_d1(int recon, const DslashLaunch &a, cudaStream_t s);
 
 cudaError_t launch_dslash(int prec, int recon, const DslashLaunch &a, cudaStream_t s)
 {
     switch (prec) {
-    case QCD_PREC_F64: return launch_dslash_f64(recon, a, s);
+    case QCD_PREC_F64:
+        if (a.U.fix && a.split != 8) return a.dagger ? launch_dslash_fix_d1(a, s) : launch_dslash_fix_d0(a, s);
+        return launch_dslash_f64(recon, a, s);
     case QCD_PREC_F32: return launch_dslash_f32(recon, a, s);
     case QCD_PREC_F16: return launch_dslash_f16(recon, a, s);
     case QCD_PREC_BF16: return launch_dslash_bf16(recon, a, s);
@@ -490,10 +540,10 @@ static void tune_store(const std::string &key, int v)
     fclose(f);
 }
 
-static std::string tune_key(const qcd_lattice *lat, int prec, int recon, int L, bool both)
+static std::string tune_key(const qcd_lattice *lat, int prec, int recon, int L, bool both, bool fix)
 {
     char k[160];
-    snprintf(k, sizeof(k), "dslash:p%d:r%d:n%d:b%d:%dx%dx%dx%d", prec, recon, L, both ? 1 : 0, lat->dims[0], lat->dims[1],
+    snprintf(k, sizeof(k), "dslash%s:p%d:r%d:n%d:b%d:%dx%dx%dx%d", fix ? "fix" : "", prec, recon, L, both ? 1 : 0, lat->dims[0], lat->dims[1],
              lat->dims[2], lat->dims[3]);
     return k;
 }
@@ -519,7 +569,7 @@ int tuned_tpb(const qcd_lattice *lat, const GaugeView &U, int prec, int recon, i
     const int force = g_force_tps.load();
     if (lanes8_ok && force == 8) return kLanes8;
     if (lanes8_ok && force == 1) return 64;
-    const std::string key = tune_key(lat, prec, recon, L, both);
+    const std::string key = tune_key(lat, prec, recon, L, both, lanes8_ok && U.fix);
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
         tune_load();
@@ -532,16 +582,16 @@ int tuned_tpb(const qcd_lattice *lat, const GaugeView &U, int prec, int recon, i
     const FieldView ti = ws_field(lat, "tune_in", both ? 2 : 1, prec, L);
     const FieldView to = ws_field(lat, "tune_out", both ? 2 : 1, prec, L);
     if (!ti.hv[0].data || !to.hv[0].data || launch_zero(ti, s) != cudaSuccess) return fallback;
+    // the fixed-point kernel with the pass that brings its input into that form
+    const FieldView tf = lanes8_ok && U.fix ? ws_field(lat, "hop_in", both ? 2 : 1, kPrecFix, L) : FieldView{};
+    const bool fix = tf.hv[0].data != nullptr;
     DslashLaunch a;
     memset(&a, 0, sizeof(a));
     a.g = lat->geom;
     a.both = both ? 1 : 0;
     a.rhs_log2 = L;
     a.U = U;
-    for (int p = 0; p < 2; ++p) {
-        a.out[p] = to.hv[both ? p : 0];
-        a.in[p] = ti.hv[both ? 1 - p : 0];
-    }
+    for (int p = 0; p < 2; ++p) a.out[p] = to.hv[both ? p : 0];
     a.epi = EPI_PLAIN;
     a.state = lat->state;
     cudaEvent_t e0, e1;
@@ -554,11 +604,19 @@ int tuned_tpb(const qcd_lattice *lat, const GaugeView &U, int prec, int recon, i
         a.tpb = v & 0xffff;
         a.split = (v >> 16) == 8 ? 8 : 1;
         a.tmap = tmap_of(lat, prec, L, a.tpb, a.split);
-        bool ok = launch_dslash(prec, recon, a, s) == cudaSuccess;  // warm-up
+        const bool vfix = fix && a.split != 8;
+        a.U.fix = vfix ? U.fix : nullptr;
+        const FieldView &in = vfix ? tf : ti;
+        for (int p = 0; p < 2; ++p) a.in[p] = in.hv[both ? 1 - p : 0];
+        auto launch = [&] {
+            if (vfix && launch_convert(tf, ti, s) != cudaSuccess) return false;
+            return launch_dslash(prec, recon, a, s) == cudaSuccess;
+        };
+        bool ok = launch();  // warm-up
         float ms_min = 1e30f;
         for (int r = 0; r < 3 && ok; ++r) {
             cudaEventRecord(e0, s);
-            ok = launch_dslash(prec, recon, a, s) == cudaSuccess;
+            ok = launch();
             cudaEventRecord(e1, s);
             float ms = 0.f;
             if (ok && cudaEventSynchronize(e1) == cudaSuccess && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess)
@@ -578,8 +636,43 @@ int tuned_tpb(const qcd_lattice *lat, const GaugeView &U, int prec, int recon, i
     return best;
 }
 
+bool fixed_hops(const qcd_lattice *lat, const GaugeView &U, int prec, int recon, int L, bool both, cudaStream_t s)
+{
+    return prec == QCD_PREC_F64 && U.fix && (tuned_tpb(lat, U, prec, recon, L, both, s) >> 16) != 8;
+}
+
+// Whether the fixed-point kernel can take a launch: with its input to be
+// brought into that form, `in` becomes that workspace field (not allocated
+// under stream capture, where a launch without it stays with FP64).
+static bool fix_input(const qcd_lattice *lat, const FieldView *&in, FieldView &ws, cudaStream_t s)
+{
+    if (in->prec == kPrecFix) return true;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    const auto it = lat->ws.find(ws_name("hop_in", kPrecFix, in->rhs_log2));
+    const size_t have = it == lat->ws.end() ? 0 : it->second.second;
+    const int stride = in->hv[0].stride;
+    const size_t need = in->nh * (spinor_half_bytes(kPrecFix, stride) + spinor_half_norm_bytes(kPrecFix, stride));
+    if (have < need && (cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone)) {
+        cudaGetLastError();
+        return false;
+    }
+    ws = ws_field(lat, "hop_in", in->nh, kPrecFix, in->rhs_log2);
+    if (!ws.hv[0].data) return false;
+    if (launch_convert(ws, *in, s) != cudaSuccess) return false;
+    in = &ws;
+    return true;
+}
+
 cudaError_t hop(const qcd_lattice *lat, const GaugeView &U, int recon, const HopArgs &h, cudaStream_t s)
 {
+    // fields in fixed point are FP64 fields as far as the launch shape goes
+    const int prec = h.out->prec == kPrecFix ? (int)QCD_PREC_F64 : h.out->prec;
+    const bool fix_fields = h.in->prec == kPrecFix || h.out->prec == kPrecFix || (h.y && h.y->prec == kPrecFix);
+    const int cfg = fix_fields ? 64 : tuned_tpb(lat, U, prec, recon, h.out->rhs_log2, h.both, s);
+    const FieldView *in = h.in;
+    FieldView in_ws;
+    const bool fix = prec == QCD_PREC_F64 && U.fix && (cfg >> 16) != 8 && fix_input(lat, in, in_ws, s);
+    if (!fix && fix_fields) return cudaErrorInvalidValue;
     DslashLaunch a;
     memset(&a, 0, sizeof(a));
     a.g = lat->geom;
@@ -588,16 +681,19 @@ cudaError_t hop(const qcd_lattice *lat, const GaugeView &U, int recon, const Hop
     a.rhs_log2 = h.out->rhs_log2;
     a.dagger = h.dagger;
     a.U = U;
+    if (!fix) a.U.fix = nullptr;
+    a.out_fix = h.out->prec == kPrecFix;
+    a.y_fix = h.y && h.y->prec == kPrecFix;
     if (h.both) {
         for (int p = 0; p < 2; ++p) {
             a.out[p] = h.out->hv[p];
-            a.in[p] = h.in->hv[1 - p];
+            a.in[p] = in->hv[1 - p];
             if (h.y) a.y[p] = h.y->hv[p];
         }
     } else {
         const int p = h.out_parity;
         a.out[p] = h.out->hv[0];
-        a.in[p] = h.in->hv[0];
+        a.in[p] = in->hv[0];
         if (h.y) a.y[p] = h.y->hv[0];
     }
     memcpy(a.cy, h.cy.c, sizeof(a.cy));
@@ -616,10 +712,9 @@ cudaError_t hop(const qcd_lattice *lat, const GaugeView &U, int recon, const Hop
         a.epi = EPI_CPLX_D;  // out = cd .* D in (real coefficients are the im = 0 case)
     else
         a.epi = h.twisted ? EPI_CPLX_YD : EPI_REAL_YD;
-    const int cfg = tuned_tpb(lat, U, h.out->prec, recon, h.out->rhs_log2, h.both, s);
     a.tpb = cfg & 0xffff;
     a.split = (cfg >> 16) == 8 ? 8 : 1;
-    a.tmap = tmap_of(lat, h.out->prec, h.out->rhs_log2, a.tpb, a.split);
+    a.tmap = tmap_of(lat, prec, h.out->rhs_log2, a.tpb, a.split);
     a.reduce = h.reduce;
     a.red = h.red ? *h.red : reduction_of(lat);
     if (h.reduce) {
@@ -636,20 +731,20 @@ cudaError_t hop(const qcd_lattice *lat, const GaugeView &U, int recon, const Hop
     const bool prof = g_prof_on;
     if (!prof) {
         note_launches();
-        return launch_dslash(h.out->prec, recon, a, s);
+        return launch_dslash(prec, recon, a, s);
     }
     std::lock_guard<std::mutex> lk(g_prof_mu);
     ProfRec r;
     r.e0 = pool_event();
     r.e1 = pool_event();
-    r.prec = h.out->prec;
+    r.prec = prec;
     r.sites = (double)(lat->h << h.out->rhs_log2) * (h.both ? 2 : 1);  // site x rhs elements
-    r.bytes = (double)lat->h * (h.both ? 2 : 1) * 8 * link_bytes(h.out->prec, recon) +
-              r.sites * (h.y ? 3 : 2) * spinor_site_bytes(h.out->prec);
+    r.bytes = (double)lat->h * (h.both ? 2 : 1) * 8 * link_bytes(prec, recon) +
+              r.sites * (h.y ? 3 : 2) * spinor_site_bytes(prec);
     r.flops = r.sites * 1320.0;
     cudaEventRecord(r.e0, s);
     note_launches();
-    cudaError_t e = launch_dslash(h.out->prec, recon, a, s);
+    cudaError_t e = launch_dslash(prec, recon, a, s);
     cudaEventRecord(r.e1, s);
     g_prof.push_back(r);
     return e;
@@ -903,6 +998,7 @@ qcd_status qcd_gauge_upload(qcd_gauge *g, const double *host, void *stream)
     if (!g || !host) return fail(QCD_ERR_INVALID_ARG, "gauge_upload: NULL argument");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const size_t bytes = (size_t)g->lat->h * 2 * 4 * 9 * 16;
+    g->fix_state = qcd_gauge::FIX_STALE;
     if (!g->derived.empty()) {
         cudaStreamSynchronize(s);
         DeviceLock dl(device_mutex());
@@ -912,7 +1008,7 @@ qcd_status qcd_gauge_upload(qcd_gauge *g, const double *host, void *stream)
     cudaError_t e = cudaMallocAsync(&stage, bytes, s);
     if (e != cudaSuccess) return check_cuda(e, "gauge_upload: staging");
     e = cudaMemcpyAsync(stage, host, bytes, cudaMemcpyHostToDevice, s);
-    const GaugeView dst{g->data, g->lat->stride};
+    const GaugeView dst{g->data, g->lat->stride, nullptr};
     if (e == cudaSuccess)
         e = launch_gauge_pack(dst, g->prec, g->recon, static_cast<const double2 *>(stage), g->lat->geom, s);
     qcd_status st = QCD_OK;
@@ -930,7 +1026,7 @@ qcd_status qcd_gauge_prepare(qcd_gauge *g, qcd_prec prec, qcd_recon recon, void 
     if (!g) return fail(QCD_ERR_INVALID_ARG, "gauge_prepare: NULL argument");
     if (!valid_prec(prec) || !valid_recon(recon)) return fail(QCD_ERR_INVALID_ARG, "gauge_prepare: bad prec/recon");
     qcd_status st;
-    gauge_view(g, prec, recon, static_cast<cudaStream_t>(stream), &st);
+    hop_links(g, prec, recon, static_cast<cudaStream_t>(stream), &st);
     return st;
 }
 
@@ -942,6 +1038,7 @@ void qcd_gauge_destroy(qcd_gauge *g)
         DeviceLock dl(device_mutex());
         cudaDeviceSynchronize();
         drop_derived(g);
+        cudaFree(g->fix);
         cudaFree(g->data);
         delete g;
     }
@@ -1180,7 +1277,7 @@ qcd_status qcd_apply_dslash(const qcd_gauge *g, qcd_spinor *out, const qcd_spino
         return fail(QCD_ERR_INVALID_ARG, "apply_dslash: parities must be (EVEN, ODD), (ODD, EVEN) or (FULL, FULL)");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     qcd_status st;
-    GaugeView U = gauge_view(g, out->prec, g->recon, s, &st);
+    GaugeView U = hop_links(g, out->prec, g->recon, s, &st);
     if (st != QCD_OK) return st;
     const FieldView fo = view_of(out), fi = view_of(in);
     HopArgs h{};
@@ -1214,12 +1311,13 @@ qcd_status qcd_apply_dslash_multi(const qcd_gauge *g, qcd_spinor *const *out, co
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const qcd_lattice *lat = g->lat;
     qcd_status st;
-    GaugeView U = gauge_view(g, in[0]->prec, g->recon, s, &st);
+    GaugeView U = hop_links(g, in[0]->prec, g->recon, s, &st);
     if (st != QCD_OK) return st;
     int L = 0;
     while ((1 << L) < nrhs) ++L;
     const int nh = both ? 2 : 1, prec = in[0]->prec;
-    const FieldView bi = ws_field(lat, "dm_in", nh, prec, L), bo = ws_field(lat, "dm_out", nh, prec, L);
+    const bool fix = fixed_hops(lat, U, prec, g->recon, L, both, s);
+    const FieldView bi = ws_field(lat, "dm_in", nh, fix ? kPrecFix : prec, L), bo = ws_field(lat, "dm_out", nh, prec, L);
     if (!bi.hv[0].data || !bo.hv[0].data) return fail(QCD_ERR_OOM, "apply_dslash_multi: workspace");
     cudaError_t e = launch_zero(bi, s);
     FieldView pv[kMaxRhs];
@@ -1254,7 +1352,7 @@ qcd_status qcd_apply_M(const qcd_gauge *g, qcd_spinor *out, const qcd_spinor *in
         return fail(QCD_ERR_INVALID_ARG, "apply_M: eo = 0 needs FULL fields");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     qcd_status st;
-    GaugeView U = gauge_view(g, out->prec, g->recon, s, &st);
+    GaugeView U = hop_links(g, out->prec, g->recon, s, &st);
     if (st != QCD_OK) return st;
     const double a = 2.0 * kappa * mu, b = dagger ? -a : a;
     const bool tw = a != 0.0;
@@ -1272,7 +1370,8 @@ qcd_status qcd_apply_M(const qcd_gauge *g, qcd_spinor *out, const qcd_spinor *in
         h.twisted = tw;
         return check_cuda(hop(g->lat, U, g->recon, h, s), "apply_M");
     }
-    const FieldView t = ws_field(g->lat, "applyM_t", 1, out->prec);
+    const bool fix = fixed_hops(g->lat, U, out->prec, g->recon, 0, false, s);
+    const FieldView t = ws_field(g->lat, "applyM_t", 1, fix ? kPrecFix : out->prec);
     if (!t.hv[0].data) return fail(QCD_ERR_OOM, "apply_M: workspace");
     h.out = &t;
     h.in = &fi;

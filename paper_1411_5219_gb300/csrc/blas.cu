@@ -5,6 +5,7 @@
 // such "algebraic operations like saxpy" next to the fermion matrices
 // (CL2QCD, arXiv:1411.5219, Sec. 4); here each one is a single pass over
 // the fields with FP64 reductions of fixed summation order.
+#include "fixed.cuh"
 #include "qcd_ops.h"
 
 namespace qcd {
@@ -75,7 +76,7 @@ __global__ void __launch_bounds__(kThreads) zero_kernel(const FieldView f)
     if (k < nsites(f)) st<SF>(f, k, zero_spinor<typename SF::R>());
 }
 
-template <typename SF>
+template <typename SO, typename SF>
 __global__ void __launch_bounds__(kThreads) twist_kernel(const FieldView out, const FieldView in, const double cr0,
                                                          const double ci0, const double cr1, const double ci1,
                                                          const double *table, const int stride)
@@ -94,7 +95,7 @@ __global__ void __launch_bounds__(kThreads) twist_kernel(const FieldView out, co
     for (int s = 0; s < 4; ++s)
 #pragma unroll
         for (int cc = 0; cc < 3; ++cc) a.c[s][cc] = cmul(c[s >> 1], a.c[s][cc]);
-    st<SF>(out, k, a);
+    st<SO>(out, k, a);
 }
 
 template <typename SF>
@@ -165,7 +166,7 @@ __global__ void cg_ctrl_loop_kernel(CgState *st, cudaGraphConditionalHandle h)
 }
 
 // r = rhs, p = r (both in the CG precision), x = 0, xs = 0; |rhs|^2.
-template <typename SR, typename SX, typename SS>
+template <typename SR, typename SX, typename SS, typename SP = SR>
 __global__ void __launch_bounds__(kThreads) cg_setup_kernel(const FieldView rhs, const FieldView r, const FieldView p,
                                                             const FieldView x, const FieldView xs, const bool has_xs,
                                                             const Reduction red, CgState *stt)
@@ -176,7 +177,7 @@ __global__ void __launch_bounds__(kThreads) cg_setup_kernel(const FieldView rhs,
         const Spinor<double> b = ld<SpF64>(rhs, k);
         const Spinor<typename SR::R> bc = cvt<typename SR::R>(b);
         st<SR>(r, k, bc);
-        st<SR>(p, k, bc);
+        st<SP>(p, k, bc);
         st<SX>(x, k, zero_spinor<typename SX::R>());
         if (has_xs) st<SS>(xs, k, zero_spinor<typename SS::R>());
         v[0] = norm2(b);
@@ -185,7 +186,7 @@ __global__ void __launch_bounds__(kThreads) cg_setup_kernel(const FieldView rhs,
 }
 
 // x += alpha p; r -= alpha q; |r|^2.
-template <typename SX, typename SF>
+template <typename SX, typename SF, typename SP = SF>
 __global__ void __launch_bounds__(kThreads) cg_xr_kernel(const FieldView x, const FieldView p, const FieldView r,
                                                          const FieldView q, const Reduction red, CgState *stt)
 {
@@ -197,7 +198,7 @@ __global__ void __launch_bounds__(kThreads) cg_xr_kernel(const FieldView x, cons
     RedT v[1] = {RedT(0)};
     if (k < nsites(x)) {
         const double alpha = stt->r[k & ((1 << x.rhs_log2) - 1)].alpha;
-        const Spinor<R> pp = ld<SF>(p, k), qq = ld<SF>(q, k);
+        const Spinor<R> pp = ld<SP>(p, k), qq = ld<SF>(q, k);
         Spinor<R> rr = ld<SF>(r, k);
         Spinor<RX> xx = ld<SX>(x, k);
         const RX ax = (RX)alpha;
@@ -219,7 +220,7 @@ __global__ void __launch_bounds__(kThreads) cg_xr_kernel(const FieldView x, cons
 }
 
 // p = r + beta p
-template <typename SF>
+template <typename SF, typename SP = SF>
 __global__ void __launch_bounds__(kThreads) cg_p_kernel(const FieldView p, const FieldView r, const CgState *stt)
 {
     if (stt->status != CG_RUNNING) return;
@@ -227,7 +228,7 @@ __global__ void __launch_bounds__(kThreads) cg_p_kernel(const FieldView p, const
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= nsites(p)) return;
     const R beta = (R)stt->r[k & ((1 << p.rhs_log2) - 1)].beta;
-    Spinor<R> pp = ld<SF>(p, k);
+    Spinor<R> pp = ld<SP>(p, k);
     const Spinor<R> rr = ld<SF>(r, k);
 #pragma unroll
     for (int s = 0; s < 4; ++s)
@@ -236,7 +237,7 @@ __global__ void __launch_bounds__(kThreads) cg_p_kernel(const FieldView p, const
             pp.c[s][c].re = fma(beta, pp.c[s][c].re, rr.c[s][c].re);
             pp.c[s][c].im = fma(beta, pp.c[s][c].im, rr.c[s][c].im);
         }
-    st<SF>(p, k, pp);
+    st<SP>(p, k, pp);
 }
 
 // xhi += xs; xs = 0
@@ -308,7 +309,7 @@ __global__ void __launch_bounds__(kThreads) cg_verify_kernel(const FieldView f, 
 // batched[(i << L) | rhs] <-> plain[rhs][i] for rhs < n, over both halves,
 // one thread per batched element: a warp reads (or writes) consecutive
 // batched elements, and the same few sites of each plain field.
-template <typename SF>
+template <typename SF, typename SB = SF>
 __global__ void __launch_bounds__(kThreads) batch_copy_kernel(const FieldView b, const PlainSet pl, const int n,
                                                               const int to_batch)
 {
@@ -318,9 +319,9 @@ __global__ void __launch_bounds__(kThreads) batch_copy_kernel(const FieldView b,
     const int rhs = e & ((1 << b.rhs_log2) - 1), i = e >> b.rhs_log2;
     if (rhs >= n) return;
     if (to_batch)
-        SF::store(b.hv[hh], e, SF::load(pl.f[rhs].hv[hh], i));
+        SB::store(b.hv[hh], e, SF::load(pl.f[rhs].hv[hh], i));
     else
-        SF::store(pl.f[rhs].hv[hh], i, SF::load(b.hv[hh], e));
+        SF::store(pl.f[rhs].hv[hh], i, SB::load(b.hv[hh], e));
 }
 
 }  // namespace
@@ -357,6 +358,12 @@ static dim3 grid_of(const FieldView &f) { return dim3(site_blocks(nsites(f))); }
 
 cudaError_t launch_convert(const FieldView &dst, const FieldView &src, cudaStream_t s)
 {
+    if (dst.prec == kPrecFix) {
+        if (src.prec != QCD_PREC_F64) return cudaErrorInvalidValue;
+        convert_kernel<SpFix, SpF64><<<grid_of(dst), kThreads, 0, s>>>(dst, src);
+        note_launches();
+        return cudaGetLastError();
+    }
     QCD_SP_CASES(dst.prec, SO, QCD_SP_CASES(src.prec, SI, convert_kernel<SO, SI><<<grid_of(dst), kThreads, 0, s>>>(dst, src)));
     note_launches();
     return cudaGetLastError();
@@ -366,20 +373,27 @@ cudaError_t launch_batch_copy(const FieldView &batched, const FieldView *plain, 
 {
     if (n < 1 || n > kMaxRhs || n > (1 << batched.rhs_log2)) return cudaErrorInvalidValue;
     PlainSet pl;
+    const bool fix = batched.prec == kPrecFix;
     for (int k = 0; k < n; ++k) {
-        if (batched.prec != plain[k].prec || batched.nh != plain[k].nh || plain[k].h << batched.rhs_log2 != batched.h)
+        if ((batched.prec != plain[k].prec && !(fix && plain[k].prec == QCD_PREC_F64)) || batched.nh != plain[k].nh || plain[k].h << batched.rhs_log2 != batched.h)
             return cudaErrorInvalidValue;
         pl.f[k] = plain[k];
     }
-    QCD_SP_CASES(batched.prec, SF,
-                 batch_copy_kernel<SF><<<grid_of(batched), kThreads, 0, s>>>(batched, pl, n, to_batch));
+    if (fix)
+        batch_copy_kernel<SpF64, SpFix><<<grid_of(batched), kThreads, 0, s>>>(batched, pl, n, to_batch);
+    else
+        QCD_SP_CASES(batched.prec, SF,
+                     batch_copy_kernel<SF><<<grid_of(batched), kThreads, 0, s>>>(batched, pl, n, to_batch));
     note_launches();
     return cudaGetLastError();
 }
 
 cudaError_t launch_zero(const FieldView &f, cudaStream_t s)
 {
-    QCD_SP_CASES(f.prec, SF, zero_kernel<SF><<<grid_of(f), kThreads, 0, s>>>(f));
+    if (f.prec == kPrecFix)
+        zero_kernel<SpFix><<<grid_of(f), kThreads, 0, s>>>(f);
+    else
+        QCD_SP_CASES(f.prec, SF, zero_kernel<SF><<<grid_of(f), kThreads, 0, s>>>(f));
     note_launches();
     return cudaGetLastError();
 }
@@ -387,8 +401,13 @@ cudaError_t launch_zero(const FieldView &f, cudaStream_t s)
 cudaError_t launch_twist(const FieldView &out, const FieldView &in, const double c[2][2], cudaStream_t s,
                          const double *table, int stride)
 {
-    if (out.prec != in.prec) return cudaErrorInvalidValue;
-    QCD_SP_CASES(out.prec, SF, twist_kernel<SF><<<grid_of(out), kThreads, 0, s>>>(out, in, c[0][0], c[0][1], c[1][0], c[1][1],
+    const bool fix = out.prec == kPrecFix && in.prec == QCD_PREC_F64;
+    if (out.prec != in.prec && !fix) return cudaErrorInvalidValue;
+    if (fix)
+        twist_kernel<SpFix, SpF64><<<grid_of(out), kThreads, 0, s>>>(out, in, c[0][0], c[0][1], c[1][0], c[1][1], table,
+                                                                     stride);
+    else
+        QCD_SP_CASES(out.prec, SF, twist_kernel<SF, SF><<<grid_of(out), kThreads, 0, s>>>(out, in, c[0][0], c[0][1], c[1][0], c[1][1],
                                                                                  table, stride));
     note_launches();
     return cudaGetLastError();
@@ -441,7 +460,9 @@ cudaError_t launch_cg_setup(const FieldView &rhs, const FieldView &r, const Fiel
     const FieldView xsv = xs ? *xs : x;
     const bool has = xs != nullptr;
     if (!reduction_fits(red, 1, rhs.rhs_log2, grid_of(rhs).x)) return cudaErrorInvalidValue;
-    if (x.prec == QCD_PREC_F64 && r.prec == QCD_PREC_F64 && !has) {
+    if (x.prec == QCD_PREC_F64 && r.prec == QCD_PREC_F64 && !has && p.prec == kPrecFix) {
+        cg_setup_kernel<SpF64, SpF64, SpF32, SpFix><<<grid_of(rhs), kThreads, 0, s>>>(rhs, r, p, x, xsv, false, red, stt);
+    } else if (x.prec == QCD_PREC_F64 && r.prec == QCD_PREC_F64 && !has) {
         cg_setup_kernel<SpF64, SpF64, SpF32><<<grid_of(rhs), kThreads, 0, s>>>(rhs, r, p, x, xsv, false, red, stt);
     } else if (x.prec == QCD_PREC_F64 && has && xs->prec == QCD_PREC_DF64 && r.prec == QCD_PREC_DF64) {
         cg_setup_kernel<SpDF64, SpF64, SpDF64><<<grid_of(rhs), kThreads, 0, s>>>(rhs, r, p, x, xsv, true, red, stt);
@@ -459,7 +480,9 @@ cudaError_t launch_cg_xr(const FieldView &x, const FieldView &p, const FieldView
                          const Reduction &red, CgState *stt, cudaStream_t s)
 {
     if (!reduction_fits(red, 1, x.rhs_log2, grid_of(x).x)) return cudaErrorInvalidValue;
-    if (x.prec == QCD_PREC_F64 && p.prec == QCD_PREC_F64) {
+    if (x.prec == QCD_PREC_F64 && p.prec == kPrecFix) {
+        cg_xr_kernel<SpF64, SpF64, SpFix><<<grid_of(x), kThreads, 0, s>>>(x, p, r, q, red, stt);
+    } else if (x.prec == QCD_PREC_F64 && p.prec == QCD_PREC_F64) {
         cg_xr_kernel<SpF64, SpF64><<<grid_of(x), kThreads, 0, s>>>(x, p, r, q, red, stt);
     } else if (x.prec == QCD_PREC_DF64 && p.prec == QCD_PREC_DF64) {
         cg_xr_kernel<SpDF64, SpDF64><<<grid_of(x), kThreads, 0, s>>>(x, p, r, q, red, stt);
@@ -474,7 +497,10 @@ cudaError_t launch_cg_xr(const FieldView &x, const FieldView &p, const FieldView
 
 cudaError_t launch_cg_p(const FieldView &p, const FieldView &r, CgState *stt, cudaStream_t s)
 {
-    QCD_SP_CASES(p.prec, SF, cg_p_kernel<SF><<<grid_of(p), kThreads, 0, s>>>(p, r, stt));
+    if (p.prec == kPrecFix)
+        cg_p_kernel<SpF64, SpFix><<<grid_of(p), kThreads, 0, s>>>(p, r, stt);
+    else
+        QCD_SP_CASES(p.prec, SF, cg_p_kernel<SF><<<grid_of(p), kThreads, 0, s>>>(p, r, stt));
     note_launches();
     return cudaGetLastError();
 }

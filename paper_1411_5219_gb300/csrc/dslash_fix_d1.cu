@@ -1,0 +1,9 @@
+// Instantiation of the fixed-point FP64 hopping kernel, dagger = 1 (one
+// translation unit per dagger value, so that they compile in parallel).
+#include "dslash_fix.cuh"
+
+namespace qcd {
+
+cudaError_t launch_dslash_fix_d1(const DslashLaunch &a, cudaStream_t s) { return launch_dslash_fix_dag<1>(a, s); }
+
+}  // namespace qcd

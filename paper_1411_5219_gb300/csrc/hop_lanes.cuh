@@ -44,13 +44,12 @@ __device__ __forceinline__ cx<double> unit_mul(cx<double> z, bool imag, bool neg
 
 // The 24 doubles (12 complex, index 3 spin + colour) that hop k of site i
 // (parity p of the output) contributes to (D psi)(x): k = 2 mu + (backward).
-// U: FP64 reconstruct-18 links, block (parity * 4 + mu) of 9 double2
-// planes; in: the 12 double2 planes of the input half field.  kCoherent:
-// the input was written earlier in the same kernel launch (read through
-// L2, not the non-coherent read-only path).
-template <bool kCoherent>
-__device__ __forceinline__ void hop_lane8(const Geom &g, const double2 *U, int ustride, const double2 *ind,
-                                          int instride, int p, int i, int k, bool dagger, cx<double> (&acc)[12])
+// link(plane, i): entry plane % 9 of the link of half-site i in block
+// (parity * 4 + mu) = plane / 9; load(a, nb): component a of the input at
+// half-site nb.
+template <typename LinkLoad, typename Load>
+__device__ __forceinline__ void hop_lane(const Geom &g, const LinkLoad &link, const Load &load, int p, int i, int k,
+                                         bool dagger, cx<double> (&acc)[12])
 {
     const SiteCoords c = site_coords(g, i, p);
     const int mu = k >> 1;
@@ -72,19 +71,18 @@ __device__ __forceinline__ void hop_lane8(const Geom &g, const double2 *U, int u
     cx<double> psi[12];
 #pragma unroll
     for (int a = 0; a < 12; ++a) {
-        const double2 v = kCoherent ? __ldcg(ind + (size_t)a * instride + nb) : __ldg(ind + (size_t)a * instride + nb);
+        const double2 v = load(a, nb);
         psi[a] = mk(v.x, v.y);
     }
     // the link: forward U_mu(x) (block (p, mu), this site), backward
     // U_mu(x - mu)^dagger (block (1 - p, mu), the neighbour)
     const int blk = (bwd ? 1 - p : p) * 4 + mu, li = bwd ? nb : i;
-    const double2 *up = U + (size_t)blk * 9 * ustride + li;
     cx<double> m[3][3];
 #pragma unroll
     for (int a = 0; a < 3; ++a)
 #pragma unroll
         for (int b = 0; b < 3; ++b) {
-            const double2 v = __ldg(up + (size_t)(bwd ? 3 * b + a : 3 * a + b) * ustride);
+            const double2 v = link(blk * 9 + (bwd ? 3 * b + a : 3 * a + b), li);
             m[a][b] = bwd ? mk(v.x, -v.y) : mk(v.x, v.y);
         }
     // projector sign: (1 - S gamma) forward, (1 + S gamma) backward; S = -1
@@ -136,6 +134,22 @@ __device__ __forceinline__ void hop_lane8(const Geom &g, const double2 *U, int u
             acc[3 * (2 + t) + a] = z;
         }
     }
+}
+
+// hop_lane from FP64 reconstruct-18 links (blocks of 9 double2 planes) and
+// the 12 double2 planes of an input half field.  kCoherent:
+// the input was written earlier in the same kernel launch (read through
+// L2, not the non-coherent read-only path).
+template <bool kCoherent>
+__device__ __forceinline__ void hop_lane8(const Geom &g, const double2 *U, int ustride, const double2 *ind,
+                                          int instride, int p, int i, int k, bool dagger, cx<double> (&acc)[12])
+{
+    hop_lane(g, [&](int plane, int li) { return __ldg(U + (size_t)plane * ustride + li); },
+             [&](int a, int nb) {
+                 const double2 *q = ind + (size_t)a * instride + nb;
+                 return kCoherent ? __ldcg(q) : __ldg(q);
+             },
+             p, i, k, dagger, acc);
 }
 
 // Sum of the eight lanes' partial spinors of a site: afterwards the lanes

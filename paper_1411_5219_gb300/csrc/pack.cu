@@ -5,6 +5,7 @@
 // conversion of a gauge field between device formats.
 #include <cstring>
 
+#include "fixed.cuh"
 #include "qcd_ops.h"
 
 namespace qcd {
@@ -61,6 +62,37 @@ __global__ void gauge_convert_kernel(const GaugeView dst, const GaugeView src, c
     const int b = blockIdx.y;
     if (i >= h) return;
     GO::store64(dst, b, i, cvt_link<double>(GI::load(src, b, i)));
+}
+
+// One part of a link entry in fixed point: u 2^60 rounded, in signed limbs
+// of 30 bits.
+__device__ __forceinline__ void link_fix(double u, int &hi, int &lo)
+{
+    const long long v = __double2ll_rn(u * 0x1p60);
+    const long long h = (v + (1ll << (kFixRadix - 1))) >> kFixRadix;
+    hi = (int)h;
+    lo = (int)(v - (h << kFixRadix));
+}
+
+template <typename GI>
+__global__ void gauge_fix_kernel(int4 *dst, const GaugeView src, const int h, unsigned *unfit)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= h) return;
+    const Link<double> u = GI::load(src, blockIdx.y, i);
+    int4 *p = dst + (size_t)blockIdx.y * 9 * src.stride + i;
+    bool fits = true;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        const cx<double> c = u.m[k / 3][k % 3];
+        int4 v;
+        link_fix(c.re, v.x, v.y);
+        link_fix(c.im, v.z, v.w);
+        p[(size_t)k * src.stride] = v;
+        // (the limbs leave room for links that are unitary to rounding only)
+        fits = fits && fabs(c.re) <= 1.0 + 0x1p-20 && fabs(c.im) <= 1.0 + 0x1p-20 && fabs(c.re) + fabs(c.im) < 1.99;
+    }
+    if (!fits) *unfit = 1u;
 }
 
 // Largest |entry error| of the links stored in format GF against the FP64
@@ -254,6 +286,31 @@ cudaError_t launch_gauge_convert(const GaugeView &dst, int dprec, int drecon, co
                 QCD_G_CASES(sprec, srecon, GI, gauge_convert_kernel<GO, GI><<<grid, 128, 0, s>>>(dst, src, g.h)));
     note_launches();
     return cudaGetLastError();
+}
+
+cudaError_t gauge_to_fix(int4 *dst, const GaugeView &src, int srecon, const Geom &g, cudaStream_t s, bool *fits)
+{
+    unsigned *d = nullptr, unfit = 1;
+    cudaError_t e = cudaMallocAsync(&d, sizeof(*d), s);
+    if (e != cudaSuccess) return e;
+    e = cudaMemsetAsync(d, 0, sizeof(*d), s);
+    if (e == cudaSuccess) {
+        const dim3 grid((g.h + 127) / 128, 8);
+        if (srecon == 18)
+            gauge_fix_kernel<GF64<18>><<<grid, 128, 0, s>>>(dst, src, g.h, d);
+        else if (srecon == 12)
+            gauge_fix_kernel<GF64<12>><<<grid, 128, 0, s>>>(dst, src, g.h, d);
+        else
+            gauge_fix_kernel<GF64<8>><<<grid, 128, 0, s>>>(dst, src, g.h, d);
+        note_launches();
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&unfit, d, sizeof(unfit), cudaMemcpyDeviceToHost, s);
+    cudaError_t e2 = cudaFreeAsync(d, s);
+    if (e == cudaSuccess) e = e2;
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    *fits = unfit == 0;
+    return e;
 }
 
 // Largest entry error of a reconstruct-8 field `dst` against its FP64

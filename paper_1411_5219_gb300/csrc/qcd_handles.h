@@ -62,6 +62,10 @@ struct qcd_gauge {
     size_t bytes = 0;
     // Copies in other (prec, recon) formats, keyed by prec * 100 + recon.
     std::map<int, std::pair<void *, size_t>> derived;
+    // F64 links in fixed point (fixed.cuh) for the FP64 hopping kernels, made on first use: the buffer outlives an upload,
+    // which only marks its contents out of date.
+    void *fix = nullptr;
+    enum FixState { FIX_STALE, FIX_READY, FIX_UNFIT } fix_state = FIX_STALE;  // UNFIT: an entry above 1 or non-finite
 };
 
 struct qcd_spinor {
@@ -111,6 +115,11 @@ FieldView view_of(const qcd_spinor *s);
 FieldView view_half(const qcd_spinor *s, int half);  // half of a FULL field
 FieldView ws_field(const qcd_lattice *lat, const std::string &name, int nh, int prec, int rhs_log2 = 0);
 GaugeView gauge_view(const qcd_gauge *g, int prec, int recon, cudaStream_t s, qcd_status *st);
+// gauge_view for the Wilson hopping term: an F64 field's view carries
+// its fixed-point copy where there is one (built here on first use;
+// left out under stream capture, without memory for it and for links that
+// do not fit, which the FP64 kernels take).
+GaugeView hop_links(const qcd_gauge *g, int prec, int recon, cudaStream_t s, qcd_status *st);
 Reduction reduction_of(const qcd_lattice *lat);
 
 cudaError_t launch_dslash(int prec, int recon, const DslashLaunch &a, cudaStream_t s);
@@ -144,6 +153,11 @@ struct HopArgs {
     int run_status;        // with check_status: run only under this CG status (default CG_RUNNING = 0)
 };
 cudaError_t hop(const qcd_lattice *lat, const GaugeView &U, int recon, const HopArgs &h, cudaStream_t s);
+
+// True when hop() runs such launches in fixed point: their temporaries may
+// then be fields of precision kPrecFix (fixed.cuh).
+bool fixed_hops(const qcd_lattice *lat, const GaugeView &U, int prec, int recon, int rhs_log2, bool both,
+                cudaStream_t s);
 
 // The CG solve behind qcd_solve_cg / qcd_solve_cg_multi, with an optional
 // context lattice (scratch, state, graphs) other than the gauge field's.

@@ -107,6 +107,7 @@ struct SpinorView {
 struct GaugeView {
     void *data;      // block (parity, mu) = parity*4 + mu, planes inside each block
     int stride;      // sites per plane (padded)
+    const int4 *fix; // FP64 links in fixed point (fixed.cuh): nine int4 planes per block, or nullptr
 };
 
 // Spinor storage formats.  load() returns the full 4x3 spinor of site i in
@@ -1190,6 +1191,7 @@ struct DslashLaunch {
     int dagger;
     GaugeView U;
     SpinorView in[2], out[2], y[2];
+    bool out_fix, y_fix; // fixed-point kernel: out, y in fixed point (its input always is)
     double cy[2][2], cd[2][2];  // [chirality][re, im]
     float cyf[2][2], cdf[2][2]; // the same rounded to float (FP32 and 16-bit kernels)
     const double *coef;         // if set: cy, cd read from this device table (8 doubles) instead

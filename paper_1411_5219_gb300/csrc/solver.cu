@@ -26,6 +26,7 @@
 #include <cstring>
 #include <vector>
 
+#include "fixed.cuh"
 #include "qcd_handles.h"
 
 namespace qcd {
@@ -371,8 +372,8 @@ qcd_status cg_graph(const qcd_lattice *lat, const CgFields &f, cudaGraphExec_t *
              f.rs.hv[0].data, f.ps.hv[0].data, f.qs.hv[0].data, f.ts.hv[0].data, f.ss.hv[0].data, f.xs.hv[0].data,
              (void *)f.state, f.rs.prec, f.rhs.nh);
     const size_t used = strlen(key);
-    snprintf(key + used, sizeof(key) - used, "|%p|%d|%d|%p|%d|%p|%p", (void *)f.red.partials, f.rs.rhs_log2,
-             (int)f.split, f.rhs0.hv[0].data, (int)f.mid, f.Um.data, f.r_m.hv[0].data);
+    snprintf(key + used, sizeof(key) - used, "|%p|%d|%d|%p|%d|%p|%p|%p", (void *)f.red.partials, f.rs.rhs_log2,
+             (int)f.split, f.rhs0.hv[0].data, (int)f.mid, f.Um.data, f.r_m.hv[0].data, (const void *)f.Uh.fix);
     auto it = lat->graphs.find(key);
     if (it != lat->graphs.end()) {
         it->second.last_use = ++lat->graph_clock;
@@ -537,7 +538,7 @@ qcd_status qcd::solve_impl(const qcd_gauge *g, qcd_spinor *const *x, const qcd_s
     // arithmetic costs more than the bytes it saves)
     const int srecon = !mixed ? g->recon : (sp == QCD_PREC_DF64 ? 18 : prm->inner_recon);
     qcd_status st;
-    const GaugeView Uh = gauge_view(g, QCD_PREC_F64, g->recon, s, &st);
+    const GaugeView Uh = hop_links(g, QCD_PREC_F64, g->recon, s, &st);
     if (st != QCD_OK) return st;
     const GaugeView Us = mixed ? gauge_view(g, sp, srecon, s, &st) : Uh;
     if (st != QCD_OK) return st;
@@ -600,14 +601,20 @@ qcd_status qcd::solve_impl(const qcd_gauge *g, qcd_spinor *const *x, const qcd_s
                 "solve_cg: coefficients");
     }
 
+    // fixed-point FP64 hops keep the fields that only hops (and p, which the
+    // vector updates) read in that form
+    const bool fix = fixed_hops(lat, Uh, QCD_PREC_F64, g->recon, L, !c.eo, s);
+    const int hp = fix ? kPrecFix : (int)QCD_PREC_F64;
+    if (fix && !ws_field(lat, "hop_in", 2, kPrecFix, L).hv[0].data) return fail(QCD_ERR_OOM, "solve_cg: workspace");
+
     // FP64 fields
     FieldView rhs = c.eo ? ws_field(lat, "cg_rhs", 1, QCD_PREC_F64, L) : bf;
     const FieldView xh = c.eo ? half_of(xf, 0) : xf;
     const FieldView rh = ws_field(lat, "cg_r", nh, QCD_PREC_F64, L);
-    const FieldView ph = ws_field(lat, "cg_p", nh, QCD_PREC_F64, L);
+    const FieldView ph = ws_field(lat, "cg_p", nh, hp, L);
     const FieldView qh = ws_field(lat, "cg_q", nh, QCD_PREC_F64, L);
-    const FieldView th = ws_field(lat, "cg_t", 1, QCD_PREC_F64, L);
-    const FieldView sh = ws_field(lat, "cg_s", nh, QCD_PREC_F64, L);
+    const FieldView th = ws_field(lat, "cg_t", 1, hp, L);
+    const FieldView sh = ws_field(lat, "cg_s", nh, mixed ? (int)QCD_PREC_F64 : hp, L);  // (a defect is formed from the mixed one)
     if (!rhs.hv[0].data || !rh.hv[0].data || !ph.hv[0].data || !qh.hv[0].data || !th.hv[0].data || !sh.hv[0].data)
         return fail(QCD_ERR_OOM, "solve_cg: workspace");
     // inner fields
