@@ -471,6 +471,7 @@ cudaError_t launch_dslash_f16(int recon, const DslashLaunch &a, cudaStream_t s);
 cudaError_t launch_dslash_bf16(int recon, const DslashLaunch &a, cudaStream_t s);
 cudaError_t launch_dslash_fix_d0(const DslashLaunch &a, cudaStream_t s);
 cudaError_t launch_dslash_fix_d1(const DslashLaunch &a, cudaStream_t s);
+cudaError_t launch_dslash_fix_lanes(const DslashLaunch &a, cudaStream_t s);
 cudaError_t launch_dslash_df64_d0(int recon, const DslashLaunch &a, cudaStream_t s);
 cudaError_t launch_dslash_df64_d1(int recon, const DslashLaunch &a, cudaStream_t s);
 
@@ -478,7 +479,8 @@ cudaError_t launch_dslash(int prec, int recon, const DslashLaunch &a, cudaStream
 {
     switch (prec) {
     case QCD_PREC_F64:
-        if (a.U.fix && a.split != 8) return a.dagger ? launch_dslash_fix_d1(a, s) : launch_dslash_fix_d0(a, s);
+        if (a.U.fix && a.split == 16) return launch_dslash_fix_lanes(a, s);
+        if (a.U.fix) return a.dagger ? launch_dslash_fix_d1(a, s) : launch_dslash_fix_d0(a, s);
         return launch_dslash_f64(recon, a, s);
     case QCD_PREC_F32: return launch_dslash_f32(recon, a, s);
     case QCD_PREC_F16: return launch_dslash_f16(recon, a, s);
@@ -497,10 +499,10 @@ cudaError_t launch_dslash(int prec, int recon, const DslashLaunch &a, cudaStream
 // configuration outside stream capture times the FP32/16-bit kernel with 64,
 // 128 and 256 threads per block (CUDA events, three launches each on
 // scratch fields) and keeps the fastest.  FP64 reconstruct-18 launches with
-// one right-hand side choose between one thread per site (64-thread blocks)
-// and the eight-lane kernel (one hop per thread, 128-thread blocks), the
-// latter winning on small lattices; a choice is stored as
-// tpb | (threads per site << 16).  With QCD_TUNE_CACHE=<file> the choices
+// one right-hand side choose between the kernel of large lattices (64 elements
+// per block; in fixed point timed with the pass that converts its input) and
+// the lane kernel (one hop per thread, 128-thread blocks), the latter winning
+// on small lattices; a choice is stored as tpb | (lanes << 16).  With QCD_TUNE_CACHE=<file> the choices
 // are read from and appended to that file, so later processes skip the
 // timing.
 static std::mutex g_tune_mu;
@@ -550,6 +552,10 @@ static std::string tune_key(const qcd_lattice *lat, int prec, int recon, int L, 
 
 constexpr int kLanes8 = 128 | (8 << 16);
 
+// Threads per output site of a choice: the lane kernels take eight in FP64,
+// sixteen in fixed point.
+static int split_of(int cfg, const GaugeView &U) { return (cfg >> 16) != 8 ? 1 : U.fix ? 16 : 8; }
+
 // Batched fields: blocks run in t-major order (DslashLaunch::tmap) when they
 // tile the time slices; the one-thread kernels' block size is 64 for FP64
 // and DF64, else tpb.  Measured on a 16-rhs FP32 launch at 32^3x8 in site
@@ -564,7 +570,7 @@ static int tmap_of(const qcd_lattice *lat, int prec, int rhs_log2, int tpb, int 
 
 int tuned_tpb(const qcd_lattice *lat, const GaugeView &U, int prec, int recon, int L, bool both, cudaStream_t s)
 {
-    const bool lanes8_ok = prec == QCD_PREC_F64 && recon == 18 && L == 0;
+    const bool lanes8_ok = prec == QCD_PREC_F64 && (recon == 18 || U.fix) && L == 0;
     if ((prec == QCD_PREC_F64 && !lanes8_ok) || prec == QCD_PREC_DF64) return 64;
     const int force = g_force_tps.load();
     if (lanes8_ok && force == 8) return kLanes8;
@@ -602,10 +608,10 @@ int tuned_tpb(const qcd_lattice *lat, const GaugeView &U, int prec, int recon, i
     const std::vector<int> cand = lanes8_ok ? std::vector<int>{64, kLanes8} : std::vector<int>{128, 64, 256};
     for (int v : cand) {
         a.tpb = v & 0xffff;
-        a.split = (v >> 16) == 8 ? 8 : 1;
+        a.split = split_of(v, U);
         a.tmap = tmap_of(lat, prec, L, a.tpb, a.split);
-        const bool vfix = fix && a.split != 8;
-        a.U.fix = vfix ? U.fix : nullptr;
+        const bool vfix = fix && a.split == 1;
+        a.U.fix = vfix || a.split == 16 ? U.fix : nullptr;
         const FieldView &in = vfix ? tf : ti;
         for (int p = 0; p < 2; ++p) a.in[p] = in.hv[both ? 1 - p : 0];
         auto launch = [&] {
@@ -681,7 +687,9 @@ cudaError_t hop(const qcd_lattice *lat, const GaugeView &U, int recon, const Hop
     a.rhs_log2 = h.out->rhs_log2;
     a.dagger = h.dagger;
     a.U = U;
-    if (!fix) a.U.fix = nullptr;
+    a.tpb = cfg & 0xffff;
+    a.split = split_of(cfg, U);
+    if (!fix && a.split == 1) a.U.fix = nullptr;
     a.out_fix = h.out->prec == kPrecFix;
     a.y_fix = h.y && h.y->prec == kPrecFix;
     if (h.both) {
@@ -712,8 +720,6 @@ cudaError_t hop(const qcd_lattice *lat, const GaugeView &U, int recon, const Hop
         a.epi = EPI_CPLX_D;  // out = cd .* D in (real coefficients are the im = 0 case)
     else
         a.epi = h.twisted ? EPI_CPLX_YD : EPI_REAL_YD;
-    a.tpb = cfg & 0xffff;
-    a.split = (cfg >> 16) == 8 ? 8 : 1;
     a.tmap = tmap_of(lat, prec, h.out->rhs_log2, a.tpb, a.split);
     a.reduce = h.reduce;
     a.red = h.red ? *h.red : reduction_of(lat);
@@ -880,9 +886,9 @@ qcd_status qcd_lattice_create(const int dims[4], int t_bc, qcd_lattice **out)
     g.tbc = (double)t_bc;
     lat->h = (int)h;
     lat->stride = (int)((h + 63) / 64 * 64);
-    // partials of the largest grid: 128-thread blocks over eight work items
-    // per site of all V sites (the eight-lane FP64 kernel), two values each
-    const size_t bmax = ((size_t)V + 15) / 16;
+    // partials of the largest grid: 128-thread blocks over sixteen work items
+    // per site of all V sites (the lane kernel in fixed point), two values each
+    const size_t bmax = ((size_t)V + 7) / 8;
     lat->red_cap = std::max(red_partials_needed(2, bmax), red_partials_needed(1, bmax));
     // tickets: one per group of the largest grid that shares them (64-thread
     // blocks over a batch of kMaxRhs full fields), and the final one

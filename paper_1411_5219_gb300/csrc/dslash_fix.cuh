@@ -3,37 +3,9 @@
 // fixed point and y and the output in either form.
 #pragma once
 
-#include "fixed.cuh"
-#include "hop_lanes.cuh"
+#include "fix_lanes.cuh"
 
 namespace qcd {
-
-// D psi of one element in FP64, hop after hop: next to sites that fixed point
-// does not hold.
-static __device__ __noinline__ void hop_site_f64(const DslashLaunch &a, int p, int i, int rhs, bool dagger, double *out)
-{
-    const SpinorView &in = a.in[p];
-    for (int k = 0; k < 24; ++k) out[k] = 0.0;
-#pragma unroll 1
-    for (int k = 0; k < 8; ++k) {
-        cx<double> v[12];
-        hop_lane(a.g,
-                 [&](int plane, int li) {
-                     const int4 q = __ldg(a.U.fix + (size_t)plane * a.U.stride + li);
-                     return make_double2(0x1p-60 * (double)of_limbs(q.x, q.y), 0x1p-60 * (double)of_limbs(q.z, q.w));
-                 },
-                 [&](int c, int nb) {
-                     const int e = (nb << a.rhs_log2) | rhs;
-                     return fix_load(__ldg(static_cast<const int4 *>(in.data) + (size_t)c * in.stride + e),
-                                     SpFix::exponent(in, e));
-                 },
-                 p, i, k, dagger, v);
-        for (int c = 0; c < 12; ++c) {
-            out[2 * c] += v[c].re;
-            out[2 * c + 1] += v[c].im;
-        }
-    }
-}
 
 constexpr int kFixThreads = 128;  // two threads per element
 constexpr int kFixElems = kFixThreads / 2;
@@ -171,12 +143,13 @@ __global__ void __launch_bounds__(kFixThreads, 4) dslash_fix_kernel(const Dslash
         d[6 + k] = fix_value(acc.la[k], Em);
     }
     if (raw) {
-        double t[24];
-        hop_site_f64(a, p, i, rhs, kDagger != 0, t);
+        double2 t[12];
+        hop_site_f64(g, a.U.fix, a.U.stride, FixLoad{a.in[p], L, rhs}, p, i, kDagger != 0, t);
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
-            d[k] = t[6 * spin + k];
-            d[6 + k] = t[12 + 6 * spin + k];
+            const double2 v = t[(k < 3 ? 0 : 3) + 3 * spin + k];
+            d[2 * k] = v.x;
+            d[2 * k + 1] = v.y;
         }
     }
     // epilogue, with coefficients from the kernel parameters or the device table of a CG
@@ -236,6 +209,68 @@ __global__ void __launch_bounds__(kFixThreads, 4) dslash_fix_kernel(const Dslash
         }
         grid_reduce_rhs<1>(red, a.rhs_log2, a.red, a.fin, a.state, a.red_out);
     }
+}
+
+// The hop of small lattices, sixteen threads per site (fix_lanes.cuh), FP64
+// fields in and out.
+template <int kEpi, bool kReduce>
+__global__ void __launch_bounds__(128) dslash_fix16_kernel(const DslashLaunch a)
+{
+    if (a.check_status && a.state->status != a.run_status) return;
+    const int items = a.g.h * 16;
+    const int nbp = (items + 127) / 128;
+    const int p = a.both ? (int)(blockIdx.x >= (unsigned)nbp) : a.out_parity;
+    const int w = (blockIdx.x - (a.both ? p * nbp : 0)) * 128 + threadIdx.x;
+    const bool act = w < items;
+    const int i = (act ? w : items - 1) >> 4, lane = w & 15;
+    const PlaneLoad<false> load{static_cast<const double2 *>(a.in[p].data), a.in[p].stride};
+    int E;
+    i64 re, im;
+    hop_fix16(a.g, a.U.fix, a.U.stride, load, p, i, lane, a.dagger != 0, E, re, im);
+    double red[1] = {0.0};
+    if (act && (lane & 3) < 3) {
+        const int chi = (lane >> 2) & 1, plane = 6 * chi + 3 * (lane >> 3) + (lane & 3);
+        cx<double> v = mk(fix_value(re, E), fix_value(im, E));
+        if (E == kFixRaw) {
+            double2 t[12];
+            hop_site_f64(a.g, a.U.fix, a.U.stride, load, p, i, a.dagger != 0, t);
+            v = mk(t[plane].x, t[plane].y);
+        }
+        const double *cf = a.coef;
+        const cx<double> d = mk(cf ? __ldg(cf + 4 + 2 * chi) : a.cd[chi][0], cf ? __ldg(cf + 5 + 2 * chi) : a.cd[chi][1]);
+        const cx<double> cy = mk(cf ? __ldg(cf + 2 * chi) : a.cy[chi][0], cf ? __ldg(cf + 1 + 2 * chi) : a.cy[chi][1]);
+        if (kEpi == EPI_CPLX_D) {
+            v = cmul(d, v);
+        } else if (kEpi == EPI_REAL_YD || kEpi == EPI_CPLX_YD) {
+            const double2 y = __ldg(static_cast<const double2 *>(a.y[p].data) + (size_t)plane * a.y[p].stride + i);
+            if (kEpi == EPI_REAL_YD)
+                v = mk(fma(d.re, v.re, cy.re * y.x), fma(d.re, v.im, cy.re * y.y));
+            else
+                v = cmac(cmul(cy, mk(y.x, y.y)), d, v);
+        }
+        static_cast<double2 *>(a.out[p].data)[(size_t)plane * a.out[p].stride + i] = make_double2(v.re, v.im);
+        red[0] = fma(v.re, v.re, v.im * v.im);
+    }
+    if (kReduce) grid_reduce_rhs<1>(red, 0, a.red, a.fin, a.state, a.red_out);
+}
+
+inline cudaError_t launch_dslash_fix16(const DslashLaunch &a, cudaStream_t s)
+{
+    if (a.rhs_log2 != 0) return cudaErrorInvalidValue;
+    const dim3 grid((16 * a.g.h + 127) / 128 * (a.both ? 2 : 1)), block(128);
+#define QCD_DSF16(E, RD)                                         \
+    if (a.epi == E && a.reduce == RD) {                          \
+        dslash_fix16_kernel<E, RD><<<grid, block, 0, s>>>(a);    \
+        return cudaGetLastError();                               \
+    }
+    QCD_DSF16(EPI_PLAIN, false)
+    QCD_DSF16(EPI_CPLX_D, false)
+    QCD_DSF16(EPI_REAL_YD, false)
+    QCD_DSF16(EPI_REAL_YD, true)
+    QCD_DSF16(EPI_CPLX_YD, false)
+    QCD_DSF16(EPI_CPLX_YD, true)
+#undef QCD_DSF16
+    return cudaErrorInvalidValue;
 }
 
 template <int D>

@@ -9,20 +9,21 @@
 // the time, not bandwidth.  Here a cooperative grid stays resident for the
 // whole solve of every system: source preparation, the CG iterations on
 // Mhat^dag Mhat x_e = Mhat^dag b'_e, the FP64 true-residual check, the odd-
-// site reconstruction and the full-system residual, with grid-wide barriers
-// between the phases instead of kernel launches.
+// site reconstruction and the full-system residual, with barriers over a
+// system's blocks between its phases instead of kernel launches.
 //
 // * Blocks are divided among the systems in proportion to their site
 //   counts (at least one each).  Reductions are summed per fixed chunk of
 //   work items and the chunks in a fixed order, so every sum -- and every
 //   result -- is bitwise the same alone and in any batch.
-// * Hopping phases use eight threads per site, one hop each (forward and
-//   backward of the four directions): the FP64 work of one thread is an
-//   eighth of a site's, which is what bounds the latency of a small
-//   lattice on GB300 (an FP64 warp instruction occupies a sub-partition's
-//   FP64 unit for 64 cycles).  The eight partial spinors are summed with
-//   warp shuffles; the spin projection and the lower-spin rebuild are
-//   table-driven (sign and lane selections, no branches on the direction).
+// * Hopping phases use sixteen threads per site, one hop and one spin each,
+//   in fixed point (fix_lanes.cuh); where the links do not fit that form,
+//   eight threads per site in FP64 (hop_lanes.cuh).  Bound by latency: at
+//   8^3 x 4 an iteration takes 42 us for six phases of one pass each.  Twelve
+//   systems of 432 to 5184 sites per parity: 17.4 ms with FP64 phases, one
+//   barrier over all blocks and its last block adding up every system in
+//   turn; 10.8 ms with the fixed-point phases; 7.8 ms with a barrier per
+//   system, whose last block sums that system alone.
 // * Every barrier wait is bounded by a clock64 budget.  When it runs out the
 //   kernel records QCD_ERR_TIMEOUT and every block returns; the call then
 //   fails with that status and the context stays usable.
@@ -37,7 +38,7 @@
 #include <vector>
 
 #include "qcd_handles.h"
-#include "hop_lanes.cuh"
+#include "fix_lanes.cuh"
 
 namespace qcd {
 namespace {
@@ -79,6 +80,7 @@ struct ManySys {
     Geom g;
     const double2 *U;   // FP64 reconstruct-18 links: block (parity*4 + mu), 9 planes each
     int ustride;
+    const int4 *fix;    // the links in fixed point (fixed.cuh), or nullptr
     HV be, bo, xe, xo;  // the caller's b and x
     HV bp, rhs, r, p, q, t, s;
     double tw_inv[2][2];    // A^-1 per chirality (source preparation)
@@ -90,29 +92,27 @@ struct ManySys {
 
 enum ManyStatus : int { MS_RUNNING = 0, MS_CONVERGED = 1, MS_DONE = 2, MS_BREAKDOWN = 3, MS_MAXITER = 4 };
 
-struct ManySysState {
-    double b2, rr, rr_new, pAp, alpha, beta, rr_stop, rr_true, full_r2, full_b2;
-    int status, iter_done;
+struct alignas(128) ManySysState {
+    double b2, rr, pAp, alpha, beta, rr_stop, rr_true, full_r2, full_b2;
+    int status;
+    int iter;              // CG iterations
+    int reliable;          // true-residual passes
+    unsigned arrive;       // arrivals at this system's barrier (zero at launch)
+    unsigned gen;          // generation of that barrier
 };
 
 struct ManyState {
     ManySysState s[kManyMax];
-    int n;
-    int iter, maxiter;
-    int reliable;          // true-residual passes
+    int maxiter;
     int error;             // QCD_ERR_TIMEOUT when a barrier wait ran out
-    unsigned arrive;       // barrier arrivals (zero at launch)
-    unsigned gen;          // barrier generation
     int timeout_where;     // phase index of the first timeout
 };
 
-// hop_lane8 and reduce_lanes8 (hop_lanes.cuh) compute the hops, eight
-// threads per site.
-// ---- grid barrier with a finaliser run by the last block to arrive
+// ---- a system's barrier with a finaliser run by its last block to arrive
 //
 // Reductions are summed per chunk of kManyThreads consecutive work items of
 // a system (whichever block processes the chunk writes its partial), and
-// the finaliser adds a system's chunks with the whole block in a fixed
+// the finaliser adds the system's chunks with the whole block in a fixed
 // order.  The result therefore depends neither on how many blocks a system
 // gets nor on what else is in the batch.
 
@@ -120,8 +120,6 @@ struct Ctx {
     const ManySys *sys;
     ManyState *st;
     double *part;          // [slot][chunk] partials
-    const int *block_sys;  // system of each block
-    int n, nblk;
     int nchunk;            // chunks per slot (all systems)
     long long budget;      // clock64 cycles a barrier wait may take
 };
@@ -147,21 +145,23 @@ __device__ __forceinline__ double chunk_sum(const Ctx &x, int slot, int k, int i
     return block_total(a);
 }
 
-// A grid-wide barrier.  Before it, each block has written its chunk
-// partials for this phase; the last block to arrive runs `fin` with all its
-// threads (sums, CG decisions by thread 0), then releases the others.
-// Returns false when the wait ran out (the kernel must return).
+// A barrier over the blocks of system k (the systems do not wait for one
+// another).  Before it, each block has written its chunk partials for this
+// phase; the last block to arrive runs `fin` with all its threads (sums, CG
+// decisions by thread 0), then releases the others.  Returns false when the
+// wait ran out, here or in another system (the kernel must return).
 template <typename Fin>
-__device__ bool grid_barrier(const Ctx &x, int where, Fin fin)
+__device__ bool sys_barrier(const Ctx &x, int k, int where, Fin fin)
 {
     __shared__ int ok, last;
     __shared__ unsigned my_gen;
+    ManySysState &q = x.st->s[k];
     __syncthreads();
     if (threadIdx.x == 0) {
         ok = 1;
-        my_gen = *(volatile unsigned *)&x.st->gen;
+        my_gen = *(volatile unsigned *)&q.gen;
         __threadfence();
-        last = atomicAdd(&x.st->arrive, 1u) == (unsigned)x.nblk - 1;
+        last = atomicAdd(&q.arrive, 1u) == (unsigned)x.sys[k].nblocks - 1;
     }
     __syncthreads();
     if (last) {
@@ -169,12 +169,12 @@ __device__ bool grid_barrier(const Ctx &x, int where, Fin fin)
         fin();
         __syncthreads();
         if (threadIdx.x == 0) {
-            x.st->arrive = 0;
+            q.arrive = 0;
             __threadfence();
-            atomicAdd(&x.st->gen, 1u);
+            atomicAdd(&q.gen, 1u);
         }
     } else if (threadIdx.x == 0) {
-        volatile unsigned *genp = &x.st->gen;
+        volatile unsigned *genp = &q.gen;
         const long long t0 = clock64();
         while (*genp == my_gen) {
             if (*(volatile int *)&x.st->error != 0 || clock64() - t0 > x.budget) {
@@ -192,59 +192,89 @@ __device__ bool grid_barrier(const Ctx &x, int where, Fin fin)
 
 // ---- phases
 
+// One complex component v of the output of a hopping phase: epilogue, store
+// (or, without `out`, the difference from b), and what it adds to the sum.
+__device__ __forceinline__ double hop_out(const ManySys &S, const PhaseCoef &pc, HV ManySys::*y, HV ManySys::*out, int p,
+                                          int plane, int i, cx<double> v, bool norm)
+{
+    const int chi = plane / 6;
+    v = cmul(mk(pc.cd[chi][0], pc.cd[chi][1]), v);
+    if (y) {
+        const double2 yy = __ldcg((S.*y).d + (size_t)plane * (S.*y).stride + i);
+        v = cmac(v, mk(pc.cy[chi][0], pc.cy[chi][1]), mk(yy.x, yy.y));
+    }
+    if (!out) {
+        // full residual: |b - M x|^2 (b of this parity)
+        const HV &bh = p == 0 ? S.be : S.bo;
+        const double2 bb = __ldg(bh.d + (size_t)plane * bh.stride + i);
+        const double dr = bb.x - v.re, di = bb.y - v.im;
+        return dr * dr + di * di;
+    }
+    const HV &o = S.*out;
+    o.d[(size_t)plane * o.stride + i] = make_double2(v.re, v.im);
+    return norm ? v.re * v.re + v.im * v.im : 0.0;
+}
+
+// Threads per site of a system's hopping phases.
+__device__ __forceinline__ int hop_threads(const ManySys &S) { return S.fix ? 16 : 8; }
+
 // A hopping phase: for every system, out (parity p) = cy y + cd D in on the
-// system's blocks, eight threads per site; optionally |out|^2 -> slot.
-// With `full` both parities are done and only |b - out|^2, |b|^2 are
-// reduced (slots 0 and 1), nothing is stored.
+// system's blocks, sixteen threads per site in fixed point, eight in FP64;
+// optionally |out|^2 -> slot.  Without `out`, |b - that|^2 is reduced and
+// nothing is stored.
 __device__ void hop_phase(const Ctx &x, int k, int lb, int coef, int p, bool dagger, HV ManySys::*in, HV ManySys::*y,
                           HV ManySys::*out, int red_slot, bool skip_done)
 {
     const ManySys &S = x.sys[k];
     const PhaseCoef &pc = S.pc[coef];
     const int run = __ldcg(&x.st->s[k].status);
-    if (!(skip_done && run != MS_RUNNING)) {
-        const int items = S.g.h * 8;
-        for (int base = lb * blockDim.x; base < items; base += S.nblocks * blockDim.x) {
-            const int w = base + threadIdx.x;
-            const bool act = w < items;
-            double red = 0.0;
+    if (skip_done && run != MS_RUNNING) return;
+    // (copies: a store through a field would have the compiler load the
+    // descriptor again in every pass of the loop)
+    const Geom g = S.g;
+    const int4 *const fix = S.fix;
+    const int us = S.ustride, nblocks = S.nblocks, chunk0 = S.chunk0;
+    const PlaneLoad<true> load{(S.*in).d, (S.*in).stride};
+    const int items = g.h * (fix ? 16 : 8);
+    for (int base = lb * kManyThreads; base < items; base += nblocks * kManyThreads) {
+        const int w = base + threadIdx.x;
+        const bool act = w < items;
+        double red = 0.0;
+        if (fix) {
+            const int i = (act ? w : items - 1) >> 4, lane = w & 15;
+            int E;
+            i64 re, im;
+            hop_fix16(g, fix, us, load, p, i, lane, dagger, E, re, im);
+            if (act && (lane & 3) < 3) {
+                const int plane = 6 * ((lane >> 2) & 1) + 3 * (lane >> 3) + (lane & 3);
+                cx<double> v = mk(fix_value(re, E), fix_value(im, E));
+                if (E == kFixRaw) {
+                    double2 t[12];
+                    hop_site_f64(g, fix, us, load, p, i, dagger, t);
+                    v = mk(t[plane].x, t[plane].y);
+                }
+                red = hop_out(S, pc, y, out, p, plane, i, v, red_slot >= 0);
+            }
+        } else {
             const int i = w >> 3, lane = w & 7;
             cx<double> acc[12];
             if (act) {
-                hop_lane8<true>(S.g, S.U, S.ustride, (S.*in).d, (S.*in).stride, p, i, lane, dagger, acc);
+                hop_lane8<true>(g, S.U, us, load.d, load.stride, p, i, lane, dagger, acc);
             } else {
 #pragma unroll
                 for (int a = 0; a < 12; ++a) acc[a] = mk(0.0, 0.0);
             }
             reduce_lanes8(acc, lane);
             if (act && !(lane & 1)) {
-                const int spin = ((lane >> 2) << 1) | ((lane >> 1) & 1), chi = spin >> 1;
-                const cx<double> cd = mk(pc.cd[chi][0], pc.cd[chi][1]), cy = mk(pc.cy[chi][0], pc.cy[chi][1]);
+                const int spin = ((lane >> 2) << 1) | ((lane >> 1) & 1);
 #pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    const int plane = 3 * spin + a;
-                    cx<double> v = cmul(cd, acc[a]);
-                    if (y) {
-                        const double2 yy = __ldcg((S.*y).d + (size_t)plane * (S.*y).stride + i);
-                        v = cmac(v, cy, mk(yy.x, yy.y));
-                    }
-                    if (!out) {
-                        // full residual: |b - M x|^2 and |b|^2 (b of this parity)
-                        const HV &bh = p == 0 ? S.be : S.bo;
-                        const double2 bb = __ldg(bh.d + (size_t)plane * bh.stride + i);
-                        const double dr = bb.x - v.re, di = bb.y - v.im;
-                        red += dr * dr + di * di;
-                    } else {
-                        const HV &o = S.*out;
-                        o.d[(size_t)plane * o.stride + i] = make_double2(v.re, v.im);
-                        if (red_slot >= 0) red += v.re * v.re + v.im * v.im;
-                    }
-                }
+                for (int a = 0; a < 3; ++a)
+                    red += hop_out(S, pc, y, out, p, 3 * spin + a, i, acc[a], red_slot >= 0);
             }
-            if (red_slot >= 0) {
-                const double t = block_total(red);
-                if (threadIdx.x == 0) x.part[(size_t)red_slot * x.nchunk + S.chunk0 + base / blockDim.x] = t;
-            }
+        }
+        if (red_slot >= 0) {
+            const double t = block_total(red);
+            if (threadIdx.x == 0) x.part[(size_t)red_slot * x.nchunk + chunk0 + base / kManyThreads] = t;
         }
     }
 }
@@ -338,15 +368,17 @@ __device__ void vec_phase(const Ctx &x, int k, int lb, VecOp op, int red_slot)
 
 // ---- the persistent kernel
 
-__global__ void __launch_bounds__(kManyThreads) many_cg_kernel(const ManySys *sys, ManyState *st, double *part,
-                                                              const int *block_sys, int n, int nchunk, long long budget)
+__global__ void __launch_bounds__(kManyThreads, 3) many_cg_kernel(const ManySys *sys, ManyState *st, double *part,
+                                                                 const int *block_sys, int nchunk, long long budget)
 {
-    const Ctx x{sys, st, part, block_sys, n, (int)gridDim.x, nchunk, budget};
+    const Ctx x{sys, st, part, nchunk, budget};
     const int k = block_sys[blockIdx.x];
     const int lb = blockIdx.x - sys[k].block0;
+    const int ht = hop_threads(sys[k]);
+    ManySysState &q = st->s[k];
     int where = 0;
-#define QCD_SYNC(FIN)                                      \
-    if (!grid_barrier(x, where++, [&]() { FIN; })) return;
+#define QCD_SYNC(FIN)                                        \
+    if (!sys_barrier(x, k, where++, [&]() { FIN; })) return;
     // ---- source: t = A^-1 b_o ; b' = b_e + kappa D_eo t ; t = A^-dag D_oe^dag b' ;
     //      rhs = A^dag b' - kappa^2 D_eo^dag t (|rhs|^2) ; r = p = rhs, x_e = 0
     vec_phase(x, k, lb, V_TWIST_BO, -1);
@@ -357,42 +389,29 @@ __global__ void __launch_bounds__(kManyThreads) many_cg_kernel(const ManySys *sy
     QCD_SYNC(;)
     hop_phase(x, k, lb, MC_SRC_R, 0, true, &ManySys::t, &ManySys::bp, &ManySys::rhs, 0, false);
     QCD_SYNC({
-        for (int j = 0; j < x.n; ++j) {
-            const double b2 = chunk_sum(x, 0, j, 8);
-            if (threadIdx.x == 0) {
-                ManySysState &q = x.st->s[j];
-                q.b2 = q.rr = q.rr_true = b2;
-                q.rr_stop = x.sys[j].tol2 * b2;
-                q.alpha = q.beta = q.pAp = 0.0;
-                q.iter_done = 0;
-                q.status = b2 == 0.0 ? MS_DONE : (isfinite(b2) ? MS_RUNNING : MS_BREAKDOWN);
-            }
-        }
+        const double b2 = chunk_sum(x, 0, k, ht);
         if (threadIdx.x == 0) {
-            x.st->iter = 0;
-            x.st->reliable = 0;
+            q.b2 = q.rr = q.rr_true = b2;
+            q.rr_stop = x.sys[k].tol2 * b2;
+            q.alpha = q.beta = q.pAp = 0.0;
+            q.status = b2 == 0.0 ? MS_DONE : (isfinite(b2) ? MS_RUNNING : MS_BREAKDOWN);
+            q.iter = 0;
+            q.reliable = 0;
         }
     })
     vec_phase(x, k, lb, V_SETUP, -1);
     QCD_SYNC(;)
     for (;;) {
         // the loop decision is read by every block after the same barrier
-        bool any_run = false, any_conv = false;
-        for (int j = 0; j < n; ++j) {
-            const int sj = __ldcg(&st->s[j].status);
-            any_run = any_run || sj == MS_RUNNING;
-            any_conv = any_conv || sj == MS_CONVERGED;
-        }
-        if (any_run && __ldcg(&st->iter) < st->maxiter) {
-            // ---- one CG iteration on the running systems
+        const int status = __ldcg(&q.status);
+        if (status == MS_RUNNING && __ldcg(&q.iter) < st->maxiter) {
+            // ---- one CG iteration
             hop_phase(x, k, lb, MC_OP1, 1, false, &ManySys::p, nullptr, &ManySys::t, -1, true);
             QCD_SYNC(;)
             hop_phase(x, k, lb, MC_OP2, 0, false, &ManySys::t, &ManySys::p, &ManySys::s, 0, true);
             QCD_SYNC({
-                for (int j = 0; j < x.n; ++j) {
-                    const double pAp = chunk_sum(x, 0, j, 8);
-                    ManySysState &q = x.st->s[j];
-                    if (threadIdx.x != 0 || q.status != MS_RUNNING) continue;
+                const double pAp = chunk_sum(x, 0, k, ht);
+                if (threadIdx.x == 0) {
                     q.pAp = pAp;
                     if (!(pAp > 0.0) || !isfinite(pAp)) {
                         q.status = MS_BREAKDOWN;
@@ -408,29 +427,25 @@ __global__ void __launch_bounds__(kManyThreads) many_cg_kernel(const ManySys *sy
             QCD_SYNC(;)
             vec_phase(x, k, lb, V_XR, 0);
             QCD_SYNC({
-                if (threadIdx.x == 0) x.st->iter += 1;
-                for (int j = 0; j < x.n; ++j) {
-                    const double rn = chunk_sum(x, 0, j, 12);
-                    ManySysState &q = x.st->s[j];
-                    if (threadIdx.x != 0 || q.status != MS_RUNNING) continue;
-                    if (!isfinite(rn)) {
-                        q.status = MS_BREAKDOWN;
-                        continue;
-                    }
-                    q.beta = rn / q.rr;
-                    q.rr = rn;
-                    if (rn <= q.rr_stop) {
-                        q.status = MS_CONVERGED;
-                        q.iter_done = x.st->iter;
+                const double rn = chunk_sum(x, 0, k, 12);
+                if (threadIdx.x == 0) {
+                    q.iter += 1;
+                    if (q.status == MS_RUNNING) {
+                        if (!isfinite(rn)) {
+                            q.status = MS_BREAKDOWN;
+                        } else {
+                            q.beta = rn / q.rr;
+                            q.rr = rn;
+                            if (rn <= q.rr_stop) q.status = MS_CONVERGED;
+                        }
                     }
                 }
             })
             vec_phase(x, k, lb, V_P, -1);
             QCD_SYNC(;)
-        } else if (any_conv) {
-            // ---- FP64 true residual of the converged systems: q = Mhat^dag Mhat x_e
-            //      (into q via s, t), r = rhs - q; DONE if it meets the target,
-            //      else CG restarts from it
+        } else if (status == MS_CONVERGED) {
+            // ---- FP64 true residual: q = Mhat^dag Mhat x_e (via s, t), r = rhs - q;
+            //      DONE if it meets the target, else CG restarts from it
             hop_phase(x, k, lb, MC_OP1, 1, false, &ManySys::xe, nullptr, &ManySys::t, -1, false);
             QCD_SYNC(;)
             hop_phase(x, k, lb, MC_OP2, 0, false, &ManySys::t, &ManySys::xe, &ManySys::s, -1, false);
@@ -441,11 +456,9 @@ __global__ void __launch_bounds__(kManyThreads) many_cg_kernel(const ManySys *sy
             QCD_SYNC(;)
             vec_phase(x, k, lb, V_TRUE, 0);
             QCD_SYNC({
-                if (threadIdx.x == 0) x.st->reliable += 1;
-                for (int j = 0; j < x.n; ++j) {
-                    const double rt = chunk_sum(x, 0, j, 12);
-                    ManySysState &q = x.st->s[j];
-                    if (threadIdx.x != 0 || q.status != MS_CONVERGED) continue;
+                const double rt = chunk_sum(x, 0, k, 12);
+                if (threadIdx.x == 0) {
+                    q.reliable += 1;
                     q.rr_true = rt;
                     if (!isfinite(rt)) {
                         q.status = MS_BREAKDOWN;
@@ -460,9 +473,7 @@ __global__ void __launch_bounds__(kManyThreads) many_cg_kernel(const ManySys *sy
             })
             vec_phase(x, k, lb, V_RESTART, -1);
             QCD_SYNC({
-                if (threadIdx.x == 0)
-                    for (int j = 0; j < x.n; ++j)
-                        if (x.st->s[j].status == MS_CONVERGED) x.st->s[j].status = MS_RUNNING;
+                if (threadIdx.x == 0 && q.status == MS_CONVERGED) q.status = MS_RUNNING;
             })
         } else {
             break;
@@ -476,12 +487,10 @@ __global__ void __launch_bounds__(kManyThreads) many_cg_kernel(const ManySys *sy
     hop_phase(x, k, lb, MC_FULL, 1, false, &ManySys::xe, &ManySys::xo, nullptr, 1, false);
     bnorm_phase(x, k, lb, 2);
     QCD_SYNC({
-        for (int j = 0; j < x.n; ++j) {
-            const double r0 = chunk_sum(x, 0, j, 8);
-            const double r1 = chunk_sum(x, 1, j, 8);
-            const double b2 = chunk_sum(x, 2, j, 24);
-            if (threadIdx.x != 0) continue;
-            ManySysState &q = x.st->s[j];
+        const double r0 = chunk_sum(x, 0, k, ht);
+        const double r1 = chunk_sum(x, 1, k, ht);
+        const double b2 = chunk_sum(x, 2, k, 24);
+        if (threadIdx.x == 0) {
             q.full_r2 = r0 + r1;
             q.full_b2 = b2;
             if (q.status == MS_RUNNING || q.status == MS_CONVERGED) q.status = MS_MAXITER;
@@ -547,7 +556,7 @@ extern "C" qcd_status qcd_solve_cg_many(int n, const qcd_gauge *const *gauges, q
     if (per_sm < 1) return fail(QCD_ERR_CUDA, "solve_cg_many: the kernel does not fit an SM");
     // blocks: every block resident (cooperative launch), divided among the
     // systems in proportion to their sites, at least one each, and no more
-    // than a system can use (8 threads per site)
+    // than a system can use (16 threads per site)
     long long total_h = 0;
     for (int k = 0; k < n; ++k) total_h += x[k]->lat->h;
     // every block resident at once; a caller sharing the GPU with other work
@@ -558,7 +567,7 @@ extern "C" qcd_status qcd_solve_cg_many(int n, const qcd_gauge *const *gauges, q
     int used = 0;
     for (int k = 0; k < n; ++k) {
         const int h = x[k]->lat->h;
-        const int useful = std::max(1, (8 * h + kManyThreads - 1) / kManyThreads);
+        const int useful = std::max(1, (16 * h + kManyThreads - 1) / kManyThreads);
         nb[k] = std::max(1, std::min(useful, (int)((long long)(grid_cap - n) * h / total_h)));
         used += nb[k];
     }
@@ -571,13 +580,16 @@ extern "C" qcd_status qcd_solve_cg_many(int n, const qcd_gauge *const *gauges, q
         const qcd_gauge *g = gauges[k];
         const qcd_lattice *lat = x[k]->lat;
         qcd_status st = QCD_OK;
-        const GaugeView U = gauge_view(g, QCD_PREC_F64, 18, s, &st);
+        GaugeView U = hop_links(g, QCD_PREC_F64, g->recon, s, &st);
+        if (st != QCD_OK) return st;
+        if (!U.fix && g->recon != 18) U = gauge_view(g, QCD_PREC_F64, 18, s, &st);  // (the FP64 phases read all nine entries)
         if (st != QCD_OK) return st;
         ManySys &S = hs[k];
         memset(&S, 0, sizeof(S));
         S.g = lat->geom;
         S.U = static_cast<const double2 *>(U.data);
         S.ustride = U.stride;
+        S.fix = U.fix;
         auto half = [&](const qcd_spinor *f, int h) {
             return HV{reinterpret_cast<double2 *>(static_cast<char *>(f->data) + h * f->half_data_bytes), lat->stride};
         };
@@ -626,14 +638,13 @@ extern "C" qcd_status qcd_solve_cg_many(int n, const qcd_gauge *const *gauges, q
     double *d_part = reinterpret_cast<double *>(ws + align(desc_bytes) + align(bs_bytes) + align(st_bytes));
     ManyState h_st;
     memset(&h_st, 0, sizeof(h_st));
-    h_st.n = n;
     h_st.maxiter = prm[0].maxiter;
     QCD_CHECK_CUDA(cudaMemcpyAsync(d_sys, hs.data(), desc_bytes, cudaMemcpyHostToDevice, s), "solve_cg_many");
     QCD_CHECK_CUDA(cudaMemcpyAsync(d_bs, block_sys.data(), bs_bytes, cudaMemcpyHostToDevice, s), "solve_cg_many");
     QCD_CHECK_CUDA(cudaMemcpyAsync(d_st, &h_st, sizeof(h_st), cudaMemcpyHostToDevice, s), "solve_cg_many");
     long long budget = wait_cycles > 0 ? wait_cycles : 4000000000LL;  // ~2 s at 2 GHz
-    int nn = n, nc = nchunk;
-    void *args[] = {&d_sys, &d_st, &d_part, &d_bs, &nn, &nc, &budget};
+    int nc = nchunk;
+    void *args[] = {&d_sys, &d_st, &d_part, &d_bs, &nc, &budget};
     QCD_CHECK_CUDA(cudaLaunchCooperativeKernel((const void *)many_cg_kernel, dim3(grid), dim3(kManyThreads), args, 0, s),
                    "solve_cg_many: launch");
     note_launches();
@@ -651,8 +662,8 @@ extern "C" qcd_status qcd_solve_cg_many(int n, const qcd_gauge *const *gauges, q
         else if (q.status != MS_DONE && result == QCD_OK)
             result = fail(QCD_ERR_NOT_CONVERGED, "solve_cg_many: maxiter reached (system %d)", k);
         if (stats) {
-            stats[k].iterations = q.status == MS_DONE ? q.iter_done : h_st.iter;
-            stats[k].reliable_updates = h_st.reliable;
+            stats[k].iterations = q.iter;
+            stats[k].reliable_updates = q.reliable;
             stats[k].true_rel_residual = q.b2 > 0.0 ? std::sqrt(q.rr_true / q.b2) : 0.0;
             stats[k].full_rel_residual = q.full_b2 > 0.0 ? std::sqrt(q.full_r2 / q.full_b2) : 0.0;
             stats[k].seconds = secs;

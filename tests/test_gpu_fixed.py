@@ -1,7 +1,8 @@
-"""The fixed-point FP64 hopping kernel (csrc/fixed.cuh) against the FP64 oracle.
+"""The fixed-point FP64 hopping kernels (csrc/fixed.cuh, csrc/fix_lanes.cuh)
+against the FP64 oracle.
 
-One thread pair per element is forced with qcd_set_hop_threads(1), so that
-small lattices run it too.  Bounds: the operator's sums round once (2^-53 of
+qcd_set_hop_threads forces the thread pair per element (1) and the sixteen
+lanes (8) whatever the lattice.  Bounds: the operator's sums round once (2^-53 of
 the result) over inputs held to 2^-56 of their site's largest component,
 far below 1e-15 norm-wise; site by site the error stays below 1e-15 of the
 largest components of the eight neighbours.
@@ -26,9 +27,9 @@ def q():
     return qcd
 
 
-@pytest.fixture(autouse=True)
-def one_thread(q):
-    q.set_hop_threads(1)
+@pytest.fixture(autouse=True, params=[1, 8])
+def threads(q, request):
+    q.set_hop_threads(request.param)
     yield
     q.set_hop_threads(0)
 
@@ -92,9 +93,9 @@ def test_fixed_unusual_values(q, case):
         with np.errstate(all="ignore"):
             want = oracle.dhop_eo(U, syn.to_half(psi, 1 - p), p)
             bound = syn.to_half(np.broadcast_to(_neighbour_max(psi)[..., None, None], psi.shape).copy(), p)
-        fine = np.isfinite(want).all(axis=(1, 2))
-        assert np.array_equal(fine, np.isfinite(got).all(axis=(1, 2)))
-        assert np.all(np.abs(got - want)[fine] <= 1e-15 * bound[fine] + 1e-322)
+            fine = np.isfinite(want).all(axis=(1, 2))
+            assert np.array_equal(fine, np.isfinite(got).all(axis=(1, 2)))
+            assert np.all(np.abs(got - want)[fine] <= 1e-15 * bound[fine] + 1e-322)
         if case == "zeros":
             assert np.all(got[bound[:, 0, 0] == 0] == 0)
 
