@@ -499,10 +499,10 @@ cudaError_t launch_dslash(int prec, int recon, const DslashLaunch &a, cudaStream
 // configuration outside stream capture times the FP32/16-bit kernel with 64,
 // 128 and 256 threads per block (CUDA events, three launches each on
 // scratch fields) and keeps the fastest.  FP64 reconstruct-18 launches with
-// one right-hand side choose between the kernel of large lattices (64 elements
-// per block; in fixed point timed with the pass that converts its input) and
-// the lane kernel (one hop per thread, 128-thread blocks), the latter winning
-// on small lattices; a choice is stored as tpb | (lanes << 16).  With QCD_TUNE_CACHE=<file> the choices
+// one right-hand side and links that do not fit the fixed-point form choose
+// between one thread per site (64-thread blocks) and the eight-lane kernel (one
+// hop per thread, 128-thread blocks), the latter winning on small lattices; a
+// choice is stored as tpb | (lanes << 16).  With QCD_TUNE_CACHE=<file> the choices
 // are read from and appended to that file, so later processes skip the
 // timing.
 static std::mutex g_tune_mu;
@@ -542,15 +542,16 @@ static void tune_store(const std::string &key, int v)
     fclose(f);
 }
 
-static std::string tune_key(const qcd_lattice *lat, int prec, int recon, int L, bool both, bool fix)
+static std::string tune_key(const qcd_lattice *lat, int prec, int recon, int L, bool both)
 {
     char k[160];
-    snprintf(k, sizeof(k), "dslash%s:p%d:r%d:n%d:b%d:%dx%dx%dx%d", fix ? "fix" : "", prec, recon, L, both ? 1 : 0, lat->dims[0], lat->dims[1],
+    snprintf(k, sizeof(k), "dslash:p%d:r%d:n%d:b%d:%dx%dx%dx%d", prec, recon, L, both ? 1 : 0, lat->dims[0], lat->dims[1],
              lat->dims[2], lat->dims[3]);
     return k;
 }
 
 constexpr int kLanes8 = 128 | (8 << 16);
+constexpr int kLanesMaxSites = 5000;  // output sites of a launch up to which the fixed-point lane kernel runs
 
 // Threads per output site of a choice: the lane kernels take eight in FP64,
 // sixteen in fixed point.
@@ -575,7 +576,10 @@ int tuned_tpb(const qcd_lattice *lat, const GaugeView &U, int prec, int recon, i
     const int force = g_force_tps.load();
     if (lanes8_ok && force == 8) return kLanes8;
     if (lanes8_ok && force == 1) return 64;
-    const std::string key = tune_key(lat, prec, recon, L, both, lanes8_ok && U.fix);
+    // in fixed point by size (FP64 CG, lanes against thread pairs: 12^3 x 4
+    // 1.94 against 2.33 ms, 12^3 x 8 3.05 against 2.68 ms)
+    if (lanes8_ok && U.fix) return (both ? 2 : 1) * lat->h <= kLanesMaxSites ? kLanes8 : 64;
+    const std::string key = tune_key(lat, prec, recon, L, both);
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
         tune_load();
@@ -588,16 +592,16 @@ int tuned_tpb(const qcd_lattice *lat, const GaugeView &U, int prec, int recon, i
     const FieldView ti = ws_field(lat, "tune_in", both ? 2 : 1, prec, L);
     const FieldView to = ws_field(lat, "tune_out", both ? 2 : 1, prec, L);
     if (!ti.hv[0].data || !to.hv[0].data || launch_zero(ti, s) != cudaSuccess) return fallback;
-    // the fixed-point kernel with the pass that brings its input into that form
-    const FieldView tf = lanes8_ok && U.fix ? ws_field(lat, "hop_in", both ? 2 : 1, kPrecFix, L) : FieldView{};
-    const bool fix = tf.hv[0].data != nullptr;
     DslashLaunch a;
     memset(&a, 0, sizeof(a));
     a.g = lat->geom;
     a.both = both ? 1 : 0;
     a.rhs_log2 = L;
     a.U = U;
-    for (int p = 0; p < 2; ++p) a.out[p] = to.hv[both ? p : 0];
+    for (int p = 0; p < 2; ++p) {
+        a.out[p] = to.hv[both ? p : 0];
+        a.in[p] = ti.hv[both ? 1 - p : 0];
+    }
     a.epi = EPI_PLAIN;
     a.state = lat->state;
     cudaEvent_t e0, e1;
@@ -610,19 +614,11 @@ int tuned_tpb(const qcd_lattice *lat, const GaugeView &U, int prec, int recon, i
         a.tpb = v & 0xffff;
         a.split = split_of(v, U);
         a.tmap = tmap_of(lat, prec, L, a.tpb, a.split);
-        const bool vfix = fix && a.split == 1;
-        a.U.fix = vfix || a.split == 16 ? U.fix : nullptr;
-        const FieldView &in = vfix ? tf : ti;
-        for (int p = 0; p < 2; ++p) a.in[p] = in.hv[both ? 1 - p : 0];
-        auto launch = [&] {
-            if (vfix && launch_convert(tf, ti, s) != cudaSuccess) return false;
-            return launch_dslash(prec, recon, a, s) == cudaSuccess;
-        };
-        bool ok = launch();  // warm-up
+        bool ok = launch_dslash(prec, recon, a, s) == cudaSuccess;  // warm-up
         float ms_min = 1e30f;
         for (int r = 0; r < 3 && ok; ++r) {
             cudaEventRecord(e0, s);
-            ok = launch();
+            ok = launch_dslash(prec, recon, a, s) == cudaSuccess;
             cudaEventRecord(e1, s);
             float ms = 0.f;
             if (ok && cudaEventSynchronize(e1) == cudaSuccess && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess)

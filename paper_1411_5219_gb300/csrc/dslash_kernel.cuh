@@ -265,14 +265,17 @@ __host__ __device__ constexpr int dslash_min_blocks()
 // 64 threads need six (<= 170 registers); the 16-bit kernels with 16-bit
 // links (mixed-precision products, 120-122 registers uncapped) five blocks of 128
 // or ten of 64 (96 registers, 20 warps per SM instead of 16, to hide their
-// memory latency); the other 4-byte kernels are not capped (64- and
-// 85-register caps spill and measured slower at 24^3x8 and 48^3x12), nor is
-// FP64 reconstruct-8, whose rebuild would spill under the cap.
+// memory latency); FP32 with reconstruct-12 four of 128 (128 registers, no
+// spills, 16 warps per SM instead of 12: 32^3 x 8 18.5 -> 16.85 us, sixteen
+// right-hand sides at 32^3 x 8 4 % faster in a solve; five and six blocks, 96
+// and 80 registers, 19.7 and 22.6 us); the other 4-byte kernels are not
+// capped, nor is FP64 reconstruct-8, whose rebuild would spill under the cap.
 template <typename SF, typename GF, int TPB>
 __host__ __device__ constexpr int dslash_min_blocks_tpb()
 {
     if constexpr (sizeof(typename SF::R) == 8 && GF::kRecon_ != 8) return TPB == 64 ? 6 : 1;
     if constexpr (is_mixed16<SF, GF>::value) return TPB == 64 ? 10 : TPB == 128 ? 5 : 2;
+    if constexpr (std::is_same<SF, SpF32>::value && GF::kRecon_ == 12) return 4 * 128 / TPB;
     return 1;
 }
 
