@@ -141,19 +141,27 @@ def _check(status: int, where: str):
         raise QcdError(status, where, lib().qcd_last_error().decode())
 
 
+_torch = None  # the torch module once its CUDA streams are there
+
+
 def _stream(stream):
     """cudaStream_t handle: an int, a torch stream, or torch's current stream."""
+    global _torch
     if stream is None:
+        if _torch is not None:  # two lookups: a call may cost little more than its launch
+            return _torch._C._cuda_getCurrentRawStream(_torch._C._cuda_getDevice())
         try:
             import torch
             if torch.cuda.is_available():
-                return _p(torch.cuda.current_stream().cuda_stream)
+                handle = torch.cuda.current_stream().cuda_stream  # (initialises CUDA in torch)
+                _torch = torch
+                return handle
         except ImportError:
             pass
-        return _p(0)
+        return 0
     if isinstance(stream, int):
-        return _p(stream)
-    return _p(stream.cuda_stream)
+        return stream
+    return stream.cuda_stream
 
 
 def _host_ptr(a, dtype=np.complex128):
