@@ -490,6 +490,23 @@ cudaError_t launch_dslash(int prec, int recon, const DslashLaunch &a, cudaStream
     }
 }
 
+cudaError_t launch_dslash_multi_f32(int recon, const DslashMulti &a, cudaStream_t s);
+cudaError_t launch_dslash_multi_f16(int recon, const DslashMulti &a, cudaStream_t s);
+cudaError_t launch_dslash_multi_bf16(int recon, const DslashMulti &a, cudaStream_t s);
+cudaError_t launch_dslash_fix_multi_d0(const DslashMulti &a, cudaStream_t s);
+cudaError_t launch_dslash_fix_multi_d1(const DslashMulti &a, cudaStream_t s);
+
+cudaError_t launch_dslash_multi(int prec, int recon, const DslashMulti &a, cudaStream_t s)
+{
+    switch (prec) {
+    case QCD_PREC_F64: return a.dagger ? launch_dslash_fix_multi_d1(a, s) : launch_dslash_fix_multi_d0(a, s);
+    case QCD_PREC_F32: return launch_dslash_multi_f32(recon, a, s);
+    case QCD_PREC_F16: return launch_dslash_multi_f16(recon, a, s);
+    case QCD_PREC_BF16: return launch_dslash_multi_bf16(recon, a, s);
+    default: return cudaErrorInvalidValue;
+    }
+}
+
 // ---- autotuner of the hopping-kernel block size
 //
 // The paper compiles its kernels for the lattice at hand and keeps the
@@ -643,6 +660,28 @@ bool fixed_hops(const qcd_lattice *lat, const GaugeView &U, int prec, int recon,
     return prec == QCD_PREC_F64 && U.fix && (tuned_tpb(lat, U, prec, recon, L, both, s) >> 16) != 8;
 }
 
+// One hopping launch, recorded with its time inside a profiling window: `sites`
+// output sites of n right-hand sides, `fields` spinors read or written each.
+template <typename Launch>
+static cudaError_t profiled(int prec, int recon, double sites, int n, int fields, cudaStream_t s, const Launch &launch)
+{
+    note_launches();
+    if (!g_prof_on) return launch();
+    std::lock_guard<std::mutex> lk(g_prof_mu);
+    ProfRec r;
+    r.e0 = pool_event();
+    r.e1 = pool_event();
+    r.prec = prec;
+    r.sites = sites * n;  // site x rhs elements
+    r.bytes = sites * 8 * link_bytes(prec, recon) + r.sites * fields * spinor_site_bytes(prec);
+    r.flops = r.sites * 1320.0;
+    cudaEventRecord(r.e0, s);
+    cudaError_t e = launch();
+    cudaEventRecord(r.e1, s);
+    g_prof.push_back(r);
+    return e;
+}
+
 // Whether the fixed-point kernel can take a launch: with its input to be
 // brought into that form, `in` becomes that workspace field (not allocated
 // under stream capture, where a launch without it stays with FP64).
@@ -730,26 +769,8 @@ cudaError_t hop(const qcd_lattice *lat, const GaugeView &U, int recon, const Hop
     a.red_out = lat->red_out;
     a.check_status = h.check_status;
     a.run_status = h.run_status;
-    const bool prof = g_prof_on;
-    if (!prof) {
-        note_launches();
-        return launch_dslash(prec, recon, a, s);
-    }
-    std::lock_guard<std::mutex> lk(g_prof_mu);
-    ProfRec r;
-    r.e0 = pool_event();
-    r.e1 = pool_event();
-    r.prec = prec;
-    r.sites = (double)(lat->h << h.out->rhs_log2) * (h.both ? 2 : 1);  // site x rhs elements
-    r.bytes = (double)lat->h * (h.both ? 2 : 1) * 8 * link_bytes(prec, recon) +
-              r.sites * (h.y ? 3 : 2) * spinor_site_bytes(prec);
-    r.flops = r.sites * 1320.0;
-    cudaEventRecord(r.e0, s);
-    note_launches();
-    cudaError_t e = launch_dslash(prec, recon, a, s);
-    cudaEventRecord(r.e1, s);
-    g_prof.push_back(r);
-    return e;
+    return profiled(prec, recon, lat->h * (h.both ? 2.0 : 1.0), 1 << h.out->rhs_log2, h.y ? 3 : 2, s,
+                    [&] { return launch_dslash(prec, recon, a, s); });
 }
 
 }  // namespace qcd
@@ -1315,15 +1336,86 @@ qcd_status qcd_apply_dslash_multi(const qcd_gauge *g, qcd_spinor *const *out, co
     qcd_status st;
     GaugeView U = hop_links(g, in[0]->prec, g->recon, s, &st);
     if (st != QCD_OK) return st;
+    const int nh = both ? 2 : 1, prec = in[0]->prec;
+    FieldView pv[kMaxRhs];
+    for (int k = 0; k < nrhs; ++k) pv[k] = view_of(in[k]);
+    // fields side by side: each is read and written in place (F64: through
+    // fixed-point copies of the inputs, whose workspace is not allocated under
+    // stream capture), unless an output overlaps another one's input
+    const size_t bytes = nh * spinor_half_bytes(prec, lat->stride), nbytes = nh * spinor_half_norm_bytes(prec, lat->stride);
+    const size_t fd = nh * spinor_half_bytes(kPrecFix, lat->stride), fn = nh * spinor_half_norm_bytes(kPrecFix, lat->stride);
+    auto overlap = [](const void *a, const void *b, size_t n) {
+        const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+        return x < y + n && y < x + n;
+    };
+    bool apart = prec != QCD_PREC_DF64 && (prec != QCD_PREC_F64 || U.fix);
+    for (int k = 0; k < nrhs; ++k)
+        for (int j = 0; j < nrhs; ++j)
+            apart = apart && !overlap(out[j]->data, in[k]->data, bytes) && !overlap(out[j]->norm, in[k]->norm, nbytes);
+    if (apart && prec == QCD_PREC_F64) {
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        const auto it = lat->ws.find("dm_fix");
+        if (it == lat->ws.end() || it->second.second < nrhs * (fd + fn))
+            apart = cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone;
+    }
+    if (apart) {
+        DslashMulti a;
+        memset(&a, 0, sizeof(a));
+        a.g = lat->geom;
+        a.out_parity = both ? 0 : out[0]->parity;
+        a.both = both ? 1 : 0;
+        a.dagger = dagger ? 1 : 0;
+        a.U = U;
+        a.n = nrhs;
+        // four fields to a warp, or the next smaller group that leaves fewer lanes idle
+        a.group_log2 = nrhs % 4 == 0 || nrhs > 8 ? 2 : nrhs % 2 == 0 || nrhs > 4 ? 1 : 0;
+        const size_t hd = spinor_half_bytes(prec, lat->stride), hn = spinor_half_norm_bytes(prec, lat->stride);
+        for (int p = 0; p < 2; ++p) {
+            a.in[p].stride = a.out[p].stride = lat->stride;
+            a.src_off[p] = both ? (1 - p) * hd : 0;
+            a.src_norm_off[p] = both ? (1 - p) * hn : 0;
+            a.dst_off[p] = both ? p * hd : 0;
+            a.dst_norm_off[p] = both ? p * hn : 0;
+        }
+        for (int k = 0; k < nrhs; ++k) {
+            a.src[k] = static_cast<const char *>(in[k]->data);
+            a.src_norm[k] = in[k]->norm;
+            a.dst[k] = static_cast<char *>(out[k]->data);
+            a.dst_norm[k] = out[k]->norm;
+        }
+        cudaError_t e = cudaSuccess;
+        if (prec == QCD_PREC_F64) {
+            char *ws = static_cast<char *>(workspace(lat, "dm_fix", nrhs * (fd + fn)));
+            if (!ws) return fail(QCD_ERR_OOM, "apply_dslash_multi: workspace");
+            FieldView f;
+            f.nh = nh;
+            f.h = lat->h;
+            f.prec = kPrecFix;
+            f.rhs_log2 = 0;
+            for (int h = 0; h < 2; ++h)
+                f.hv[h] = SpinorView{ws + (h < nh ? h : 0) * (fd / nh),
+                                     reinterpret_cast<float *>(ws + nrhs * fd + (h < nh ? h : 0) * (fn / nh)), lat->stride};
+            e = launch_fix_set(f, fd, fn, pv, nrhs, s);
+            for (int k = 0; k < nrhs; ++k) {
+                a.src[k] = ws + k * fd;
+                a.src_norm[k] = reinterpret_cast<const float *>(ws + nrhs * fd + k * fn);
+            }
+            for (int p = 0; p < 2; ++p) {
+                a.src_off[p] = both ? (1 - p) * (fd / nh) : 0;
+                a.src_norm_off[p] = both ? (1 - p) * (fn / nh) : 0;
+            }
+        }
+        if (e == cudaSuccess)
+            e = profiled(prec, g->recon, lat->h * (both ? 2.0 : 1.0), nrhs, 2, s,
+                         [&] { return launch_dslash_multi(prec, g->recon, a, s); });
+        return check_cuda(e, "apply_dslash_multi");
+    }
     int L = 0;
     while ((1 << L) < nrhs) ++L;
-    const int nh = both ? 2 : 1, prec = in[0]->prec;
     const bool fix = fixed_hops(lat, U, prec, g->recon, L, both, s);
     const FieldView bi = ws_field(lat, "dm_in", nh, fix ? kPrecFix : prec, L), bo = ws_field(lat, "dm_out", nh, prec, L);
     if (!bi.hv[0].data || !bo.hv[0].data) return fail(QCD_ERR_OOM, "apply_dslash_multi: workspace");
     cudaError_t e = launch_zero(bi, s);
-    FieldView pv[kMaxRhs];
-    for (int k = 0; k < nrhs; ++k) pv[k] = view_of(in[k]);
     if (e == cudaSuccess) e = launch_batch_copy(bi, pv, nrhs, 1, s);
     if (e != cudaSuccess) return check_cuda(e, "apply_dslash_multi: gather");
     HopArgs h{};

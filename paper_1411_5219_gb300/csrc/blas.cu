@@ -69,6 +69,19 @@ __global__ void __launch_bounds__(kThreads) convert_kernel(const FieldView out, 
     if (k < nsites(out)) st<SO>(out, k, cvt<typename SO::R>(ld<SI>(in, k)));
 }
 
+// out's half hh of field k from plain[k]: blockIdx.y = field
+__global__ void __launch_bounds__(kThreads) fix_set_kernel(const FieldView out, const size_t data_bytes,
+                                                           const size_t norm_bytes, const __grid_constant__ PlainSet pl)
+{
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= nsites(out)) return;
+    const int hh = k >= out.h, i = k - hh * out.h;
+    SpinorView v = out.hv[hh];
+    v.data = static_cast<char *>(v.data) + blockIdx.y * data_bytes;
+    v.norm = reinterpret_cast<float *>(reinterpret_cast<char *>(v.norm) + blockIdx.y * norm_bytes);
+    SpFix::store(v, i, SpF64::load(pl.f[blockIdx.y].hv[hh], i));
+}
+
 template <typename SF>
 __global__ void __launch_bounds__(kThreads) zero_kernel(const FieldView f)
 {
@@ -365,6 +378,20 @@ cudaError_t launch_convert(const FieldView &dst, const FieldView &src, cudaStrea
         return cudaGetLastError();
     }
     QCD_SP_CASES(dst.prec, SO, QCD_SP_CASES(src.prec, SI, convert_kernel<SO, SI><<<grid_of(dst), kThreads, 0, s>>>(dst, src)));
+    note_launches();
+    return cudaGetLastError();
+}
+
+cudaError_t launch_fix_set(const FieldView &out, size_t data_bytes, size_t norm_bytes, const FieldView *plain, int n,
+                           cudaStream_t s)
+{
+    if (n < 1 || n > kMaxRhs || out.prec != kPrecFix) return cudaErrorInvalidValue;
+    PlainSet pl;
+    for (int k = 0; k < n; ++k) {
+        if (plain[k].prec != QCD_PREC_F64 || plain[k].nh != out.nh || plain[k].h != out.h) return cudaErrorInvalidValue;
+        pl.f[k] = plain[k];
+    }
+    fix_set_kernel<<<dim3(grid_of(out).x, n), kThreads, 0, s>>>(out, data_bytes, norm_bytes, pl);
     note_launches();
     return cudaGetLastError();
 }

@@ -27,15 +27,21 @@ __device__ __forceinline__ void copy16(int4 *dst, const int4 *src)
 // (205 us for 1.05 GB, 76 % of HBM; the FP64 kernel took 945 us).  Three slots
 // at 12 warps per SM or two at 20 (96 registers, spills) measured slower than
 // two at 16.
-template <int kDagger, int kEpi, bool kReduce>
-__global__ void __launch_bounds__(kFixThreads, 4) dslash_fix_kernel(const DslashLaunch a)
+template <int kDagger, int kEpi, bool kReduce, typename Launch = DslashLaunch>
+__global__ void __launch_bounds__(kFixThreads, 4) dslash_fix_kernel(const __grid_constant__ Launch a)
 {
+    constexpr bool kMulti = std::is_same<Launch, DslashMulti>::value;  // separate fields, consecutive blocks one each
     if (a.check_status && a.state->status != a.run_status) return;
     constexpr int SF_ = kDagger ? -1 : +1, SB_ = -SF_;  // projector signs of forward and backward hops
     const int ne = a.g.h << a.rhs_log2;
-    const int nbp = (ne + kFixElems - 1) / kFixElems;
+    int nbp = (ne + kFixElems - 1) / kFixElems, field = 0;
+    if constexpr (kMulti) nbp *= a.n;
     const int p = a.both ? (int)(blockIdx.x >= (unsigned)nbp) : a.out_parity;
     int bl = blockIdx.x - (a.both ? p * nbp : 0);
+    if constexpr (kMulti) {
+        field = bl % a.n;
+        bl /= a.n;
+    }
     if (a.tmap) bl = (bl % a.g.L[3]) * a.tmap + bl / a.g.L[3];
     const int spin = (threadIdx.x >> 4) & 1;
     const int e = bl * kFixElems + (threadIdx.x >> 5) * 16 + (threadIdx.x & 15);
@@ -44,8 +50,13 @@ __global__ void __launch_bounds__(kFixThreads, 4) dslash_fix_kernel(const Dslash
     const int i = (act ? e : ne - 1) >> L;  // (the tail works on the last element and stores nothing)
     double red[1] = {0.0};
     const Geom &g = a.g;
-    const size_t is = a.in[p].stride, us = a.U.stride;
-    const int4 *in = static_cast<const int4 *>(a.in[p].data);
+    SpinorView inv = a.in[p], outv = a.out[p];
+    if constexpr (kMulti) {
+        inv = a.input(p, field);
+        outv = a.output(p, field);
+    }
+    const size_t is = inv.stride, us = a.U.stride;
+    const int4 *in = static_cast<const int4 *>(inv.data);
     const SiteCoords c = site_coords(g, i, p);
     const int base = i - c.xh;
     const bool wf = c.t == g.L[3] - 1, wb = c.t == 0, anti = antiperiodic(g);
@@ -61,7 +72,7 @@ __global__ void __launch_bounds__(kFixThreads, 4) dslash_fix_kernel(const Dslash
     int E[8], Em = 0;
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
-        E[k] = SpFix::exponent(a.in[p], (nb[k] << L) | rhs);
+        E[k] = SpFix::exponent(inv, (nb[k] << L) | rhs);
         Em = max(Em, E[k]);
     }
     const int sg = spin ? -1 : 1;
@@ -123,16 +134,16 @@ __global__ void __launch_bounds__(kFixThreads, 4) dslash_fix_kernel(const Dslash
         top |= __shfl_xor_sync(0xffffffffu, top, 16);
         const int sh = max(64 - __clzll((long long)top) - kFixBits, 0);
         if (act) {
-            int4 *o = static_cast<int4 *>(a.out[p].data) + e;
+            int4 *o = static_cast<int4 *>(outv.data) + e;
 #pragma unroll
             for (int k = 0; k < 6; ++k) {
                 const i64 *v = (k < 3 ? acc.up : acc.la) + 2 * (k % 3);
                 int4 q;
                 to_limbs(v[0] >> sh, q.x, q.y);
                 to_limbs(v[1] >> sh, q.z, q.w);
-                o[(size_t)((k < 3 ? 0 : 3) + 3 * spin + k) * a.out[p].stride] = q;
+                o[(size_t)((k < 3 ? 0 : 3) + 3 * spin + k) * outv.stride] = q;
             }
-            if (spin == 0) reinterpret_cast<int *>(a.out[p].norm)[e] = top == 0ull ? 0 : Em + sh;
+            if (spin == 0) reinterpret_cast<int *>(outv.norm)[e] = top == 0ull ? 0 : Em + sh;
         }
         return;
     }
@@ -144,7 +155,7 @@ __global__ void __launch_bounds__(kFixThreads, 4) dslash_fix_kernel(const Dslash
     }
     if (raw) {
         double2 t[12];
-        hop_site_f64(g, a.U.fix, a.U.stride, FixLoad{a.in[p], L, rhs}, p, i, kDagger != 0, t);
+        hop_site_f64(g, a.U.fix, a.U.stride, FixLoad{inv, L, rhs}, p, i, kDagger != 0, t);
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
             const double2 v = t[(k < 3 ? 0 : 3) + 3 * spin + k];
@@ -190,14 +201,14 @@ __global__ void __launch_bounds__(kFixThreads, 4) dslash_fix_kernel(const Dslash
         top = max(top, __shfl_xor_sync(0xffffffffu, top, 16));
         low |= __shfl_xor_sync(0xffffffffu, low, 16);
         Eo = fix_exponent(top, low);
-        if (act && spin == 0) reinterpret_cast<int *>(a.out[p].norm)[e] = Eo;
+        if (act && spin == 0) reinterpret_cast<int *>(outv.norm)[e] = Eo;
     }
     if (act) {
-        int4 *o = static_cast<int4 *>(a.out[p].data) + e;
+        int4 *o = static_cast<int4 *>(outv.data) + e;
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
             // (kFixRaw: the FP64 form)
-            o[(size_t)((k < 3 ? 0 : 3) + 3 * spin + k) * a.out[p].stride] = fix_store(d[2 * k], d[2 * k + 1], Eo);
+            o[(size_t)((k < 3 ? 0 : 3) + 3 * spin + k) * outv.stride] = fix_store(d[2 * k], d[2 * k + 1], Eo);
             if (kReduce) red[0] = fma(d[2 * k], d[2 * k], fma(d[2 * k + 1], d[2 * k + 1], red[0]));
         }
     }
@@ -271,6 +282,14 @@ inline cudaError_t launch_dslash_fix16(const DslashLaunch &a, cudaStream_t s)
     QCD_DSF16(EPI_CPLX_YD, true)
 #undef QCD_DSF16
     return cudaErrorInvalidValue;
+}
+
+template <int D>
+cudaError_t launch_dslash_fix_multi(const DslashMulti &a, cudaStream_t s)
+{
+    const dim3 grid((unsigned)((a.g.h + kFixElems - 1) / kFixElems) * a.n * (a.both ? 2 : 1)), block(kFixThreads);
+    dslash_fix_kernel<D, EPI_PLAIN, false, DslashMulti><<<grid, block, 0, s>>>(a);
+    return cudaGetLastError();
 }
 
 template <int D>

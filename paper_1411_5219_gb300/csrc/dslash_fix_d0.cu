@@ -6,4 +6,6 @@ namespace qcd {
 
 cudaError_t launch_dslash_fix_d0(const DslashLaunch &a, cudaStream_t s) { return launch_dslash_fix_dag<0>(a, s); }
 
+cudaError_t launch_dslash_fix_multi_d0(const DslashMulti &a, cudaStream_t s) { return launch_dslash_fix_multi<0>(a, s); }
+
 }  // namespace qcd

@@ -6,4 +6,6 @@ namespace qcd {
 
 cudaError_t launch_dslash_fix_d1(const DslashLaunch &a, cudaStream_t s) { return launch_dslash_fix_dag<1>(a, s); }
 
+cudaError_t launch_dslash_fix_multi_d1(const DslashMulti &a, cudaStream_t s) { return launch_dslash_fix_multi<1>(a, s); }
+
 }  // namespace qcd

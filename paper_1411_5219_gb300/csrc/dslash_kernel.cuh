@@ -280,23 +280,40 @@ __host__ __device__ constexpr int dslash_min_blocks_tpb()
 }
 
 template <typename SF, typename GF, int kDagger, int kEpi, bool kReduce, int TPB,
-          int kMinBlocks = dslash_min_blocks_tpb<SF, GF, TPB>()>
-__global__ void __launch_bounds__(TPB, kMinBlocks) dslash_kernel(const DslashLaunch a)
+          int kMinBlocks = dslash_min_blocks_tpb<SF, GF, TPB>(), typename Launch = DslashLaunch>
+__global__ void __launch_bounds__(TPB, kMinBlocks) dslash_kernel(const __grid_constant__ Launch a)
 {
     using R = typename SF::R;
+    constexpr bool kMulti = std::is_same<Launch, DslashMulti>::value;
     if (a.check_status && a.state->status != a.run_status) return;
     constexpr int SF_ = kDagger ? -1 : +1;  // projector sign of forward hops
     constexpr int SB_ = -SF_;                // ... of backward hops
-    // element e = site i * 2^rhs_log2 + rhs (one rhs: e = i)
+    // element e = site i * 2^rhs_log2 + rhs (one rhs: e = i); with separate
+    // fields a warp takes a few of them at consecutive sites, so that its lanes
+    // share link loads, and consecutive blocks the next fields at those sites
     const int ne = a.g.h << a.rhs_log2;
-    const int nbp = (ne + TPB - 1) / TPB;
+    int nbp = (ne + TPB - 1) / TPB, field = 0, ngroups = 1;
+    if constexpr (kMulti) {
+        ngroups = (a.n + (1 << a.group_log2) - 1) >> a.group_log2;
+        nbp = ((ne + (TPB >> a.group_log2) - 1) / (TPB >> a.group_log2)) * ngroups;
+    }
     const int p = a.both ? (int)(blockIdx.x >= (unsigned)nbp) : a.out_parity;
     int bl = blockIdx.x - (a.both ? p * nbp : 0);
+    if constexpr (kMulti) {
+        field = (bl % ngroups) << a.group_log2;
+        bl /= ngroups;
+    }
     // with tmap = blocks per time slice, consecutive blocks take the same
     // space chunk at consecutive t, so every neighbour is re-read within a
     // few MB of traffic (an L2 hit) even when a batched field exceeds L2
     if (a.tmap) bl = (bl % a.g.L[3]) * a.tmap + bl / a.g.L[3];
-    const int e = bl * blockDim.x + threadIdx.x;
+    int e = bl * blockDim.x + threadIdx.x;
+    if constexpr (kMulti) {
+        const int sites = 32 >> a.group_log2;  // of a warp
+        field += (threadIdx.x & 31) / sites;
+        e = (bl * (TPB / 32) + (threadIdx.x >> 5)) * sites + (threadIdx.x & (sites - 1));
+        if (field >= a.n) e = ne;
+    }
     const int L = a.rhs_log2, rhs = e & ((1 << L) - 1);
     const int i = e >> L;
     // fused norm: summed within the warp in float by the FP32/16-bit kernels
@@ -304,7 +321,8 @@ __global__ void __launch_bounds__(TPB, kMinBlocks) dslash_kernel(const DslashLau
     RedT red[1] = {RedT(0)};
     if (e < ne) {
         const Geom &g = a.g;
-        const SpinorView &in = a.in[p];
+        SpinorView in = a.in[p];
+        if constexpr (kMulti) in = a.input(p, field);
         const SiteCoords c = site_coords(g, i, p);
         const int base = i - c.xh;
         const int fwd = p * 4, bwd = (1 - p) * 4;
@@ -499,7 +517,10 @@ __global__ void __launch_bounds__(TPB, kMinBlocks) dslash_kernel(const DslashLau
                     for (int cc = 0; cc < 3; ++cc) out.c[s][cc] = cmac(cmul(cy[s >> 1], y.c[s][cc]), d[s >> 1], acc.c[s][cc]);
             }
         }
-        SF::store(a.out[p], e, out);
+        if constexpr (kMulti)
+            SF::store(a.output(p, field), e, out);
+        else
+            SF::store(a.out[p], e, out);
         if (kReduce) {
             R n = 0;
 #pragma unroll
@@ -618,6 +639,25 @@ cudaError_t launch_dslash_dag(const DslashLaunch &a, cudaStream_t s)
         return launch_dslash_tpb<SF, GF, D, 128>(a, s);
     }
     return cudaErrorInvalidValue;
+}
+
+// Separate fields: 128 threads, D or D^dagger without an epilogue.  Bound by
+// memory latency, the links from L2.  Gathering the fields into one batched
+// field, padded to a power of two, and scattering the results took 137 us for
+// twelve FP32 right-hand sides at 24^3 x 8 (floor 22 us), most of it those
+// passes; read in place, eight sites and four fields to a warp (128-byte
+// segments, link loads shared by four lanes), 51 us.
+template <typename SF, typename GF>
+cudaError_t launch_dslash_multi_fmt(const DslashMulti &a, cudaStream_t s)
+{
+    const int groups = (a.n + (1 << a.group_log2) - 1) >> a.group_log2, sites = 128 >> a.group_log2;
+    const dim3 grid((unsigned)((a.g.h + sites - 1) / sites) * groups * (a.both ? 2 : 1)), block(128);
+    constexpr int kMin = dslash_min_blocks_tpb<SF, GF, 128>();
+    if (a.dagger)
+        dslash_kernel<SF, GF, 1, EPI_PLAIN, false, 128, kMin, DslashMulti><<<grid, block, 0, s>>>(a);
+    else
+        dslash_kernel<SF, GF, 0, EPI_PLAIN, false, 128, kMin, DslashMulti><<<grid, block, 0, s>>>(a);
+    return cudaGetLastError();
 }
 
 template <typename SF, typename GF>

@@ -1208,7 +1208,34 @@ struct DslashLaunch {
     int run_status;     // the status the launch runs under (CG_RUNNING, or CG_VERIFY for a check)
 };
 
+// The plain hopping term of n separate fields of one kind in one launch: the
+// fields are read and written where they lie (in, out hold the plane strides
+// only).
+struct DslashMulti : DslashLaunch {
+    int n;
+    int group_log2;  // right-hand sides of one warp (its lanes / 2^group_log2 consecutive sites)
+    const char *src[kMaxRhs];
+    const float *src_norm[kMaxRhs];
+    char *dst[kMaxRhs];
+    float *dst_norm[kMaxRhs];
+    size_t src_off[2], src_norm_off[2], dst_off[2], dst_norm_off[2];  // bytes to the half of output parity p
+
+    __device__ __forceinline__ SpinorView input(int p, int k) const
+    {
+        return SpinorView{const_cast<char *>(src[k]) + src_off[p],
+                          reinterpret_cast<float *>(const_cast<char *>(reinterpret_cast<const char *>(src_norm[k])) + src_norm_off[p]),
+                          in[p].stride};
+    }
+    __device__ __forceinline__ SpinorView output(int p, int k) const
+    {
+        return SpinorView{dst[k] + dst_off[p],
+                          reinterpret_cast<float *>(reinterpret_cast<char *>(dst_norm[k]) + dst_norm_off[p]), out[p].stride};
+    }
+};
+
 cudaError_t launch_dslash(int prec, int recon, const DslashLaunch &a, cudaStream_t s);
+// Precisions F32, F16 and BF16, and F64 with fixed-point links and input.
+cudaError_t launch_dslash_multi(int prec, int recon, const DslashMulti &a, cudaStream_t s);
 
 // number of blocks / threads used by site kernels (for scratch sizing)
 constexpr int kThreads = 128;

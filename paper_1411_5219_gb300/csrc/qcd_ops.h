@@ -73,6 +73,11 @@ struct PlainSet {
 };
 cudaError_t launch_batch_copy(const FieldView &batched, const FieldView *plain, int n, int to_batch, cudaStream_t s);
 
+// n F64 fields into fixed point: field k at `out` + k * data_bytes (exponents
+// + k * norm_bytes), in one launch.
+cudaError_t launch_fix_set(const FieldView &out, size_t data_bytes, size_t norm_bytes, const FieldView *plain, int n,
+                           cudaStream_t s);
+
 // Staggered hopping term (csrc/staggered.cu).  in/out indexed by output
 // parity as for DslashLaunch; staggered fields hold 3 complex per site.
 struct KsLaunch {
