@@ -907,9 +907,9 @@ qcd_status qcd_lattice_create(const int dims[4], int t_bc, qcd_lattice **out)
     // per site of all V sites (the lane kernel in fixed point), two values each
     const size_t bmax = ((size_t)V + 7) / 8;
     lat->red_cap = std::max(red_partials_needed(2, bmax), red_partials_needed(1, bmax));
-    // tickets: one per group of the largest grid that shares them (64-thread
-    // blocks over a batch of kMaxRhs full fields), and the final one
-    const size_t counter_bytes = ((4 * (1 + (size_t)red_group_size((unsigned)(V * kMaxRhs / 64 + 1), 1)) + 255) / 256) * 256;
+    // tickets: one per group of the largest grid that shares them (32 elements
+    // a block over a batch of kMaxRhs full fields), and the final one
+    const size_t counter_bytes = ((4 * (1 + (size_t)red_group_size((unsigned)(V * kMaxRhs / 32 + 1), 1)) + 255) / 256) * 256;
     cudaError_t e = lat_alloc(lat, (void **)&lat->red_partials, lat->red_cap * sizeof(double));
     if (e == cudaSuccess) e = lat_alloc(lat, (void **)&lat->red_counter, counter_bytes);
     if (e == cudaSuccess) e = lat_alloc(lat, (void **)&lat->red_out, 8 * sizeof(double));

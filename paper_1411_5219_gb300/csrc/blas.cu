@@ -162,20 +162,18 @@ __global__ void cg_state_init_kernel(CgState *s, int nrhs, const RhsValues tol2,
 }
 
 
-// Graph control: run the reliable-update body when the iteration asked for it.
-__global__ void cg_ctrl_reliable_kernel(const CgState *st, cudaGraphConditionalHandle h)
+// The conditions of a CG graph from the state (one thread): set by the kernel
+// that finishes an iteration, so that no launch of its own is needed for it.
+__device__ __forceinline__ void set_loop(const CgGraphControl &ctl, const CgState *st)
 {
-    const int s = st->status;
-    cudaGraphSetConditional(h, (s == CG_RELIABLE || s == CG_CONVERGED) ? 1u : 0u);
+    const bool go = st->status == CG_RUNNING && st->iter < st->maxiter && st->trips < st->trip_limit;
+    cudaGraphSetConditional(ctl.loop, go ? 1u : 0u);
 }
-
-// Graph control: repeat the loop body while CG runs; the trip cap bounds the
-// loop whatever the state holds.
-__global__ void cg_ctrl_loop_kernel(CgState *st, cudaGraphConditionalHandle h)
+__device__ __forceinline__ void set_iteration(const CgGraphControl &ctl, CgState *st)
 {
     st->trips += 1;
-    const bool go = st->status == CG_RUNNING && st->iter < st->maxiter && st->trips < st->trip_limit;
-    cudaGraphSetConditional(h, go ? 1u : 0u);
+    cudaGraphSetConditional(ctl.reliable, (st->status == CG_RELIABLE || st->status == CG_CONVERGED) ? 1u : 0u);
+    set_loop(ctl, st);
 }
 
 // r = rhs, p = r (both in the CG precision), x = 0, xs = 0; |rhs|^2.
@@ -199,11 +197,15 @@ __global__ void __launch_bounds__(kThreads) cg_setup_kernel(const FieldView rhs,
 }
 
 // x += alpha p; r -= alpha q; |r|^2.
-template <typename SX, typename SF, typename SP = SF>
+template <typename SX, typename SF>
 __global__ void __launch_bounds__(kThreads) cg_xr_kernel(const FieldView x, const FieldView p, const FieldView r,
-                                                         const FieldView q, const Reduction red, CgState *stt)
+                                                         const FieldView q, const Reduction red, CgState *stt,
+                                                         const CgGraphControl ctl)
 {
-    if (stt->status != CG_RUNNING) return;
+    if (stt->status != CG_RUNNING) {  // (a breakdown in this iteration ends the loop)
+        if (ctl.on && blockIdx.x == 0 && threadIdx.x == 0) set_iteration(ctl, stt);
+        return;
+    }
     using R = typename SF::R;
     using RX = typename SX::R;
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
@@ -211,7 +213,7 @@ __global__ void __launch_bounds__(kThreads) cg_xr_kernel(const FieldView x, cons
     RedT v[1] = {RedT(0)};
     if (k < nsites(x)) {
         const double alpha = stt->r[k & ((1 << x.rhs_log2) - 1)].alpha;
-        const Spinor<R> pp = ld<SP>(p, k), qq = ld<SF>(q, k);
+        const Spinor<R> pp = ld<SF>(p, k), qq = ld<SF>(q, k);
         Spinor<R> rr = ld<SF>(r, k);
         Spinor<RX> xx = ld<SX>(x, k);
         const RX ax = (RX)alpha;
@@ -229,13 +231,57 @@ __global__ void __launch_bounds__(kThreads) cg_xr_kernel(const FieldView x, cons
         st<SF>(r, k, rr);
         v[0] = (RedT)norm2(rr);
     }
-    grid_reduce_rhs<1>(v, x.rhs_log2, red, FIN_CG_RR, stt, nullptr);
+    if (grid_reduce_rhs<1>(v, x.rhs_log2, red, FIN_CG_RR, stt, nullptr) && ctl.on) set_iteration(ctl, stt);
+}
+
+// The same in FP64, one thread per element and spin (a block's warps take the
+// four spins of 32 elements): bound by FP64 instructions, 72 a site, and the
+// latency of the reduction; one thread per element left them to too few warps
+// (FP64 CG, one thread per element against four: 12^3 x 8 2.59 / 2.47 ms, 16^3
+// x 8 3.06 / 2.97, 24^3 x 8 the same, 32^3 x 8 12.87 / 12.50).  kFix: p in fixed
+// point.
+template <bool kFix>
+__global__ void __launch_bounds__(kThreads) cg_xr_spin_kernel(const FieldView x, const FieldView p, const FieldView r,
+                                                              const FieldView q, const Reduction red, CgState *stt,
+                                                              const CgGraphControl ctl)
+{
+    if (stt->status != CG_RUNNING) {
+        if (ctl.on && blockIdx.x == 0 && threadIdx.x == 0) set_iteration(ctl, stt);
+        return;
+    }
+    const int spin = threadIdx.x >> 5, k = blockIdx.x * 32 + (threadIdx.x & 31);
+    double v[1] = {0.0};
+    if (k < nsites(x)) {
+        const double a = stt->r[k & ((1 << x.rhs_log2) - 1)].alpha;
+        const int hh = k >= x.h, i = k - hh * x.h;
+        const SpinorView vx = x.hv[hh], vp = p.hv[hh], vr = r.hv[hh], vq = q.hv[hh];
+        const int E = kFix ? SpFix::exponent(vp, i) : kFixRaw;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const size_t plane = 3 * spin + c;
+            const double2 pp = fix_load(__ldg(static_cast<const int4 *>(vp.data) + plane * vp.stride + i), E);
+            const double2 qq = __ldg(static_cast<const double2 *>(vq.data) + plane * vq.stride + i);
+            double2 *px = static_cast<double2 *>(vx.data) + plane * vx.stride + i;
+            double2 *pr = static_cast<double2 *>(vr.data) + plane * vr.stride + i;
+            double2 xx = *px, rr = *pr;
+            xx.x = fma(a, pp.x, xx.x);
+            xx.y = fma(a, pp.y, xx.y);
+            rr.x = fma(-a, qq.x, rr.x);
+            rr.y = fma(-a, qq.y, rr.y);
+            *px = xx;
+            *pr = rr;
+            v[0] = fma(rr.x, rr.x, fma(rr.y, rr.y, v[0]));
+        }
+    }
+    if (grid_reduce_rhs<1>(v, x.rhs_log2, red, FIN_CG_RR, stt, nullptr) && ctl.on) set_iteration(ctl, stt);
 }
 
 // p = r + beta p
 template <typename SF, typename SP = SF>
-__global__ void __launch_bounds__(kThreads) cg_p_kernel(const FieldView p, const FieldView r, const CgState *stt)
+__global__ void __launch_bounds__(kThreads) cg_p_kernel(const FieldView p, const FieldView r, const CgState *stt,
+                                                        const CgGraphControl ctl)
 {
+    if (ctl.on && blockIdx.x == 0 && threadIdx.x == 0) set_loop(ctl, stt);
     if (stt->status != CG_RUNNING) return;
     using R = typename SF::R;
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
@@ -467,20 +513,6 @@ cudaError_t launch_cg_state_init(CgState *stt, int nrhs, const RhsValues &tol2, 
 }
 
 
-cudaError_t launch_cg_ctrl_reliable(const CgState *stt, cudaGraphConditionalHandle h, cudaStream_t s)
-{
-    cg_ctrl_reliable_kernel<<<1, 1, 0, s>>>(stt, h);
-    note_launches();
-    return cudaGetLastError();
-}
-
-cudaError_t launch_cg_ctrl_loop(CgState *stt, cudaGraphConditionalHandle h, cudaStream_t s)
-{
-    cg_ctrl_loop_kernel<<<1, 1, 0, s>>>(stt, h);
-    note_launches();
-    return cudaGetLastError();
-}
-
 cudaError_t launch_cg_setup(const FieldView &rhs, const FieldView &r, const FieldView &p, const FieldView &x,
                             const FieldView *xs, const Reduction &red, CgState *stt, cudaStream_t s)
 {
@@ -504,17 +536,19 @@ cudaError_t launch_cg_setup(const FieldView &rhs, const FieldView &r, const Fiel
 }
 
 cudaError_t launch_cg_xr(const FieldView &x, const FieldView &p, const FieldView &r, const FieldView &q,
-                         const Reduction &red, CgState *stt, cudaStream_t s)
+                         const Reduction &red, CgState *stt, cudaStream_t s, const CgGraphControl &ctl)
 {
-    if (!reduction_fits(red, 1, x.rhs_log2, grid_of(x).x)) return cudaErrorInvalidValue;
-    if (x.prec == QCD_PREC_F64 && p.prec == kPrecFix) {
-        cg_xr_kernel<SpF64, SpF64, SpFix><<<grid_of(x), kThreads, 0, s>>>(x, p, r, q, red, stt);
-    } else if (x.prec == QCD_PREC_F64 && p.prec == QCD_PREC_F64) {
-        cg_xr_kernel<SpF64, SpF64><<<grid_of(x), kThreads, 0, s>>>(x, p, r, q, red, stt);
+    const dim3 spin_grid((nsites(x) + 31) / 32);
+    const bool f64 = x.prec == QCD_PREC_F64 && (p.prec == QCD_PREC_F64 || p.prec == kPrecFix);
+    if (!reduction_fits(red, 1, x.rhs_log2, (f64 ? spin_grid : grid_of(x)).x)) return cudaErrorInvalidValue;
+    if (f64 && p.prec == kPrecFix) {
+        cg_xr_spin_kernel<true><<<spin_grid, kThreads, 0, s>>>(x, p, r, q, red, stt, ctl);
+    } else if (f64) {
+        cg_xr_spin_kernel<false><<<spin_grid, kThreads, 0, s>>>(x, p, r, q, red, stt, ctl);
     } else if (x.prec == QCD_PREC_DF64 && p.prec == QCD_PREC_DF64) {
-        cg_xr_kernel<SpDF64, SpDF64><<<grid_of(x), kThreads, 0, s>>>(x, p, r, q, red, stt);
+        cg_xr_kernel<SpDF64, SpDF64><<<grid_of(x), kThreads, 0, s>>>(x, p, r, q, red, stt, ctl);
     } else if (x.prec == QCD_PREC_F32) {
-        QCD_SP_CASES(p.prec, SF, cg_xr_kernel<SpF32, SF><<<grid_of(x), kThreads, 0, s>>>(x, p, r, q, red, stt));
+        QCD_SP_CASES(p.prec, SF, cg_xr_kernel<SpF32, SF><<<grid_of(x), kThreads, 0, s>>>(x, p, r, q, red, stt, ctl));
     } else {
         return cudaErrorInvalidValue;
     }
@@ -522,12 +556,12 @@ cudaError_t launch_cg_xr(const FieldView &x, const FieldView &p, const FieldView
     return cudaGetLastError();
 }
 
-cudaError_t launch_cg_p(const FieldView &p, const FieldView &r, CgState *stt, cudaStream_t s)
+cudaError_t launch_cg_p(const FieldView &p, const FieldView &r, CgState *stt, cudaStream_t s, const CgGraphControl &ctl)
 {
     if (p.prec == kPrecFix)
-        cg_p_kernel<SpF64, SpFix><<<grid_of(p), kThreads, 0, s>>>(p, r, stt);
+        cg_p_kernel<SpF64, SpFix><<<grid_of(p), kThreads, 0, s>>>(p, r, stt, ctl);
     else
-        QCD_SP_CASES(p.prec, SF, cg_p_kernel<SF><<<grid_of(p), kThreads, 0, s>>>(p, r, stt));
+        QCD_SP_CASES(p.prec, SF, cg_p_kernel<SF><<<grid_of(p), kThreads, 0, s>>>(p, r, stt, ctl));
     note_launches();
     return cudaGetLastError();
 }

@@ -180,10 +180,7 @@ __global__ void __launch_bounds__(kFixThreads, 4) dslash_fix_kernel(const __grid
                 } else {
                     const int4 q = __ldg(static_cast<const int4 *>(a.y[p].data) + at + (size_t)k * a.y[p].stride);
                     const double2 y = fix_load(q, a.y_fix ? yE : kFixRaw);
-                    if (kEpi == EPI_REAL_YD)
-                        v = mk(fma(cd.re, v.re, cy.re * y.x), fma(cd.re, v.im, cy.re * y.y));
-                    else
-                        v = cmac(cmul(cy, mk(y.x, y.y)), cd, v);
+                    v = fix_epilogue<kEpi == EPI_REAL_YD>(v, y, cy, cd);
                 }
                 d[6 * chi + 2 * k] = v.re;
                 d[6 * chi + 2 * k + 1] = v.im;
@@ -254,10 +251,7 @@ __global__ void __launch_bounds__(128) dslash_fix16_kernel(const DslashLaunch a)
             v = cmul(d, v);
         } else if (kEpi == EPI_REAL_YD || kEpi == EPI_CPLX_YD) {
             const double2 y = __ldg(static_cast<const double2 *>(a.y[p].data) + (size_t)plane * a.y[p].stride + i);
-            if (kEpi == EPI_REAL_YD)
-                v = mk(fma(d.re, v.re, cy.re * y.x), fma(d.re, v.im, cy.re * y.y));
-            else
-                v = cmac(cmul(cy, mk(y.x, y.y)), d, v);
+            v = fix_epilogue<kEpi == EPI_REAL_YD>(v, y, cy, d);
         }
         static_cast<double2 *>(a.out[p].data)[(size_t)plane * a.out[p].stride + i] = make_double2(v.re, v.im);
         red[0] = fma(v.re, v.re, v.im * v.im);

@@ -79,6 +79,20 @@ __device__ __forceinline__ double fix_value(i64 P, int E)
     return P != 0 ? __hiloint2double(hi, __double2loint(v)) : 0.0;
 }
 
+// The same for a P of at most 53 significant bits (one that came from a
+// double), exactly and without FP64 instructions: a 64-bit conversion holds
+// the FP64 pipe for 74 cycles a warp, these dozen integer instructions do not.
+__device__ __forceinline__ double fix_value_exact(i64 P, int E)
+{
+    const unsigned long long m = (unsigned long long)(P < 0 ? -P : P);
+    const int z = __clzll((long long)m);
+    const unsigned long long n = m << (z & 63);  // leading one at bit 63
+    // (the leading one adds one to the exponent field)
+    const int hi = ((E - kFixBias + 1023 + 62 - z) << 20) + (int)(n >> 43);
+    const int lo = (int)(n >> 11);
+    return P == 0 ? 0.0 : __hiloint2double(hi | (P < 0 ? (int)0x80000000 : 0), lo);
+}
+
 // The exponent that a site is stored under: `top` its largest twice_hi, `low`
 // an or of its low words (wanted where top is zero: the smallest denormals).
 __device__ __forceinline__ int fix_exponent(unsigned top, unsigned low)
@@ -87,11 +101,12 @@ __device__ __forceinline__ int fix_exponent(unsigned top, unsigned low)
     return (top | low) == 0u ? 0 : (E < kFixLow || E > kFixHigh) ? kFixRaw : E;
 }
 
-// One stored component as FP64.
+// One stored component as FP64 (what the hop itself wrote may hold 56 bits:
+// cut to 53 here).
 __device__ __forceinline__ double2 fix_load(int4 q, int E)
 {
     if (E == kFixRaw) return make_double2(__hiloint2double(q.y, q.x), __hiloint2double(q.w, q.z));
-    return make_double2(fix_value(of_limbs(q.x, q.y), E), fix_value(of_limbs(q.z, q.w), E));
+    return make_double2(fix_value_exact(of_limbs(q.x, q.y), E), fix_value_exact(of_limbs(q.z, q.w), E));
 }
 __device__ __forceinline__ int4 fix_store(double re, double im, int E)
 {
@@ -146,6 +161,20 @@ struct SpFix {
         reinterpret_cast<int *>(v.norm)[i] = E;
     }
 };
+
+// The epilogue cy y + cd v of one complex component: fewer FP64 instructions
+// where cy is 1 or 1 + i a and cd real, as in M and its Schur complement.
+template <bool kReal>
+__device__ __forceinline__ cx<double> fix_epilogue(cx<double> v, double2 y, cx<double> cy, cx<double> cd)
+{
+    if (kReal) {
+        if (cy.re == 1.0) return mk(fma(cd.re, v.re, y.x), fma(cd.re, v.im, y.y));
+        return mk(fma(cd.re, v.re, cy.re * y.x), fma(cd.re, v.im, cy.re * y.y));
+    }
+    if (cy.re == 1.0 && cd.im == 0.0)
+        return mk(fma(cd.re, v.re, fma(-cy.im, y.y, y.x)), fma(cd.re, v.im, fma(cy.im, y.x, y.y)));
+    return cmac(cmul(cy, mk(y.x, y.y)), cd, v);
+}
 
 // The sums of one thread: spin s of the output (up) and what its spin s of
 // the half spinors gives to the lower spins, 2 + s in the z and t hops (la),

@@ -911,40 +911,52 @@ enum FinalizeKind : int {
     FIN_CG_TRUE_EST = 5,// true residual estimated in the inner precision (Mhat^dag of the FP64 defect)
 };
 
-// tot[r] = the reduced value of right-hand side r (first value only).
-__device__ __forceinline__ void cg_finalize_rhs(FinalizeKind kind, const double *tot, CgState *st)
+// The decisions that follow a reduction, by one warp: lane r takes right-hand
+// side r (its state `q` and the state's global fields loaded before the sums
+// were ready), `tot` holds the reduced value per right-hand side.  One thread
+// going through the state load by load took 30 us of a reducing kernel at
+// sixteen right-hand sides (FP32 x/r update at 32^3 x 8 211 -> 180 us, the hop
+// with the fused norm 187 -> 159 us) and 5 % of an FP64 solve at 8^3 x 4.
+struct CgGlobals {
+    int nrhs, iter, maxiter, status, reliable_updates;
+    double delta2;
+};
+__device__ __forceinline__ CgGlobals cg_globals(const CgState *st)
 {
-    const int n = st->nrhs;
+    return CgGlobals{st->nrhs, st->iter, st->maxiter, st->status, st->reliable_updates, st->delta2};
+}
+
+__device__ __forceinline__ void cg_finalize_warp(FinalizeKind kind, const double *tot, CgState *st, CgRhs q, CgGlobals g)
+{
+    constexpr unsigned kAll = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const bool on = lane < g.nrhs;
+    const double t = on ? tot[lane] : 0.0;
+    bool bad = on && !isfinite(t);
+    int status = g.status;
     if (kind == FIN_CG_INIT) {
-        bool all_done = true, bad = false;
-        for (int k = 0; k < n; ++k) {
-            CgRhs &q = st->r[k];
-            const double b2 = tot[k];
-            q.rr = q.rr_prev = q.rr_max = q.rr_true = q.b2 = b2;
-            q.rr_stop = q.tol2 * b2;
-            q.alpha = q.beta = q.pAp = 0.0;
-            q.iter_done = 0;
-            q.status = b2 == 0.0 ? CG_DONE : CG_RUNNING;
-            all_done = all_done && q.status == CG_DONE;
-            bad = bad || !isfinite(b2);
+        q.rr = q.rr_prev = q.rr_max = q.rr_true = q.b2 = t;
+        q.rr_stop = q.tol2 * t;
+        q.alpha = q.beta = q.pAp = 0.0;
+        q.iter_done = 0;
+        q.status = t == 0.0 ? CG_DONE : CG_RUNNING;
+        const bool all_done = __all_sync(kAll, !on || q.status == CG_DONE);
+        bad = __any_sync(kAll, bad);
+        status = bad ? CG_BREAKDOWN : all_done ? CG_DONE : CG_RUNNING;
+        if (lane == 0) {
+            st->iter = 0;
+            st->reliable_updates = 0;
         }
-        st->iter = 0;
-        st->reliable_updates = 0;
-        st->status = bad ? CG_BREAKDOWN : all_done ? CG_DONE : CG_RUNNING;
     } else if (kind == FIN_CG_ALPHA) {
-        for (int k = 0; k < n; ++k) {
-            CgRhs &q = st->r[k];
-            q.pAp = tot[k];
-            if (q.status == CG_DONE) {
-                q.alpha = 0.0;
-            } else if (!(tot[k] > 0.0) || !isfinite(tot[k])) {
-                q.alpha = 0.0;
+        q.pAp = t;
+        q.alpha = 0.0;
+        if (on && q.status != CG_DONE) {
+            if (!(t > 0.0) || bad)
                 q.status = CG_BREAKDOWN;
-                st->status = CG_BREAKDOWN;
-            } else {
-                q.alpha = q.rr / tot[k];
-            }
+            else
+                q.alpha = q.rr / t;
         }
+        if (__any_sync(kAll, on && q.status == CG_BREAKDOWN)) status = CG_BREAKDOWN;
     } else if (kind == FIN_CG_RR) {
         // A true-residual update runs when every running system is ready --
         // its residual fell by the reliable-update factor delta since the last
@@ -952,83 +964,57 @@ __device__ __forceinline__ void cg_finalize_rhs(FinalizeKind kind, const double 
         // fell by delta^2 (so one slow system cannot hold the others back).
         // A batch of similar systems thus pays about the updates of one
         // solve, and one final check rather than one per system.
-        st->iter += 1;
-        bool all_ready = true, urgent = false, bad = false;
-        const double d2 = st->delta2;
-        for (int k = 0; k < n; ++k) {
-            CgRhs &q = st->r[k];
-            if (q.status == CG_DONE) {
-                q.beta = 0.0;
-                continue;
-            }
-            const double rr_new = tot[k];
+        const bool run = on && q.status != CG_DONE;
+        const double d2 = g.delta2;
+        bool ready = true, urgent = false;
+        if (on) q.beta = 0.0;
+        if (run) {
             q.rr_prev = q.rr;
-            q.beta = rr_new / q.rr;
-            q.rr = rr_new;
-            if (!isfinite(rr_new)) bad = true;
-            const bool dropped = d2 > 0.0 && rr_new < d2 * q.rr_max;
-            all_ready = all_ready && (dropped || rr_new <= q.rr_stop);
-            urgent = urgent || (d2 > 0.0 && rr_new < d2 * d2 * q.rr_max);
-            if (rr_new > q.rr_max) q.rr_max = rr_new;
+            q.beta = t / q.rr;
+            q.rr = t;
+            const bool dropped = d2 > 0.0 && t < d2 * q.rr_max;
+            ready = dropped || t <= q.rr_stop;
+            urgent = d2 > 0.0 && t < d2 * d2 * q.rr_max;
+            if (t > q.rr_max) q.rr_max = t;
         }
+        bad = __any_sync(kAll, run && bad);
+        const bool update = __all_sync(kAll, ready) || __any_sync(kAll, urgent);
         if (bad)
-            st->status = CG_BREAKDOWN;
-        else if (all_ready || urgent)
-            st->status = CG_RELIABLE;
-        else if (st->iter >= st->maxiter)
-            st->status = CG_MAXITER;
-    } else if (kind == FIN_CG_TRUE_EST) {
-        // The FP64 defect rho = rhs0 - Mhat x, mapped by Mhat^dag in a lower
-        // precision: a system whose estimate meets its target is checked in
-        // FP64 next (CG_VERIFY); the others continue from the estimate.
-        st->reliable_updates += 1;
-        bool verify = false, bad = false;
-        for (int k = 0; k < n; ++k) {
-            CgRhs &q = st->r[k];
-            if (q.status == CG_DONE) {
-                q.beta = 0.0;
-                continue;
-            }
-            const double rt = tot[k];
-            q.rr_true = rt;
-            if (!isfinite(rt)) {
-                bad = true;
-            } else if (rt <= q.rr_stop) {
-                verify = true;
-            } else {
-                q.beta = rt / q.rr_prev;
-                q.rr = rt;
-                q.rr_max = rt;
-            }
-        }
-        st->status = bad ? CG_BREAKDOWN : verify ? CG_VERIFY : (st->iter >= st->maxiter ? CG_MAXITER : CG_RUNNING);
-    } else if (kind == FIN_CG_TRUE) {
-        if (st->status != CG_VERIFY) st->reliable_updates += 1;  // (a verification completes its update)
-        bool all_done = true, bad = false;
-        for (int k = 0; k < n; ++k) {
-            CgRhs &q = st->r[k];
-            if (q.status == CG_DONE) {
-                q.beta = 0.0;
-                continue;
-            }
-            const double rt = tot[k];
-            q.rr_true = rt;
-            if (!isfinite(rt)) {
-                bad = true;
-            } else if (rt <= q.rr_stop) {
+            status = CG_BREAKDOWN;
+        else if (update)
+            status = CG_RELIABLE;
+        else if (g.iter + 1 >= g.maxiter)
+            status = CG_MAXITER;
+        if (lane == 0) st->iter = g.iter + 1;
+    } else if (kind == FIN_CG_TRUE_EST || kind == FIN_CG_TRUE) {
+        // TRUE_EST: the FP64 defect rho = rhs0 - Mhat x, mapped by Mhat^dag in a
+        // lower precision: a system whose estimate meets its target is checked
+        // in FP64 next (CG_VERIFY); the others continue from the estimate.
+        const bool est = kind == FIN_CG_TRUE_EST, run = on && q.status != CG_DONE;
+        bool met = false;
+        if (on && !run) q.beta = 0.0;
+        if (run) {
+            q.rr_true = t;
+            met = !bad && t <= q.rr_stop;
+            if (met && !est) {
                 q.status = CG_DONE;
-                q.iter_done = st->iter;
+                q.iter_done = g.iter;
                 q.beta = 0.0;
-            } else {
-                q.beta = rt / q.rr_prev;
-                q.rr = rt;
-                q.rr_max = rt;
+            } else if (!met && !bad) {
+                q.beta = t / q.rr_prev;
+                q.rr = t;
+                q.rr_max = t;
             }
-            all_done = all_done && q.status == CG_DONE;
         }
-        st->status = bad ? CG_BREAKDOWN
-                         : all_done ? CG_DONE : (st->iter >= st->maxiter ? CG_MAXITER : CG_RUNNING);
+        bad = __any_sync(kAll, run && bad);
+        const bool verify = __any_sync(kAll, est && met), all_done = __all_sync(kAll, !on || q.status == CG_DONE);
+        const int next = g.iter >= g.maxiter ? CG_MAXITER : CG_RUNNING;
+        status = bad ? CG_BREAKDOWN : est ? (verify ? CG_VERIFY : next) : all_done ? CG_DONE : next;
+        // (a verification completes its update)
+        if (lane == 0 && (est || g.status != CG_VERIFY)) st->reliable_updates = g.reliable_updates + 1;
     }
+    if (on) st->r[lane] = q;
+    if (lane == 0) st->status = status;
 }
 
 // Grid-wide reduction segmented by right-hand side: element e of a batched
@@ -1041,8 +1027,8 @@ __device__ __forceinline__ void cg_finalize_rhs(FinalizeKind kind, const double 
 // thread of the block: T = blockDim / P threads per row (at least one; P and
 // blockDim powers of two), each taking every T-th element from its offset
 // with four accumulators (loads in flight), then the T sums of a row added
-// by a fixed binary tree into res[q] (shared).  The order is fixed, so the
-// sums are reproducible.
+// by warp shuffles, and over its warps in order, into res[q] (shared).  The
+// order is fixed, so the sums are reproducible.
 __device__ __forceinline__ void block_row_sums(const double *src, size_t stride, int P, unsigned count,
                                                double *res, double *scratch /* blockDim.x */)
 {
@@ -1062,21 +1048,22 @@ __device__ __forceinline__ void block_row_sums(const double *src, size_t stride,
             }
             for (; b < count; b += T) a0 += __ldcg(row + b);
         }
-        scratch[threadIdx.x] = (a0 + a1) + (a2 + a3);
+        double a = (a0 + a1) + (a2 + a3);
+        for (int off = (T < 32 ? T : 32) >> 1; off > 0; off >>= 1) a += __shfl_down_sync(0xffffffffu, a, off);
+        scratch[threadIdx.x] = a;
         __syncthreads();
-        for (int off = T >> 1; off > 0; off >>= 1) {
-            if (j < off) scratch[threadIdx.x] += scratch[threadIdx.x + off];
-            __syncthreads();
-        }
-        if (j == 0 && q < P) res[q] = scratch[threadIdx.x];
+        if (j == 0)
+            for (int w = 32; w < T; w += 32) a += scratch[threadIdx.x + w];
+        if (j == 0 && q < P) res[q] = a;
         __syncthreads();
     }
 }
 
 // (grid_reduce_rhs after the sums within each warp: lane r < nrhs holds
 // the warp's sum of rhs r)
+// Returns true in the one thread that finalised.
 template <int NV>
-__device__ __forceinline__ void grid_reduce_rhs_warp_summed(const double (&v)[NV], int rhs_log2, const Reduction &red,
+__device__ __forceinline__ bool grid_reduce_rhs_warp_summed(const double (&v)[NV], int rhs_log2, const Reduction &red,
                                                             FinalizeKind kind, CgState *st, double *out)
 {
     __shared__ double sw[NV][8][kMaxRhs];  // [value][warp][rhs]; blocks of <= 256 threads
@@ -1101,8 +1088,15 @@ __device__ __forceinline__ void grid_reduce_rhs_warp_summed(const double (&v)[NV
     __syncthreads();
     if (threadIdx.x == 0) is_last = atomicAdd(red.counter + 1 + grp, 1u) == gsize - 1;
     __syncthreads();
-    if (!is_last) return;
+    if (!is_last) return false;
     __threadfence();
+    CgRhs mine{};
+    CgGlobals glob{};
+    const bool decide = kind != FIN_STORE && threadIdx.x < 32;
+    if (decide) {
+        mine = st->r[threadIdx.x];
+        glob = cg_globals(st);
+    }
     // the last block of the group: the group's partials in block order
     block_row_sums(red.partials + (size_t)grp * G, nb, P, gsize, tot, scratch);
     if (ng > 1) {
@@ -1117,31 +1111,29 @@ __device__ __forceinline__ void grid_reduce_rhs_warp_summed(const double (&v)[NV
             is_last = atomicAdd(red.counter, 1u) == ng - 1;
         }
         __syncthreads();
-        if (!is_last) return;
+        if (!is_last) return false;
         __threadfence();
         // the last group: the group sums in group order
         block_row_sums(gsum, ng, P, ng, tot, scratch);
     }
+    if (decide) cg_finalize_warp(kind, tot, st, mine, glob);
+    if (kind == FIN_STORE && (int)threadIdx.x < P) out[threadIdx.x] = tot[threadIdx.x];
     if (threadIdx.x == 0) {
         red.counter[1] = 0u;  // (one group: its ticket; otherwise already reset)
-        if (kind == FIN_STORE) {
-            for (int q = 0; q < NV * n; ++q) out[q] = tot[q];
-        } else {
-            cg_finalize_rhs(kind, tot, st);
-        }
         *red.counter = 0u;
     }
+    return threadIdx.x == 0;
 }
 
 template <int NV>
-__device__ __forceinline__ void grid_reduce_rhs(double (&v)[NV], int rhs_log2, const Reduction &red,
+__device__ __forceinline__ bool grid_reduce_rhs(double (&v)[NV], int rhs_log2, const Reduction &red,
                                                 FinalizeKind kind, CgState *st, double *out)
 {
     const int n = 1 << rhs_log2;
 #pragma unroll
     for (int k = 0; k < NV; ++k)
         for (int off = 16; off >= n; off >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], off);
-    grid_reduce_rhs_warp_summed<NV>(v, rhs_log2, red, kind, st, out);
+    return grid_reduce_rhs_warp_summed<NV>(v, rhs_log2, red, kind, st, out);
 }
 
 // The same for FP32 values (the FP32 and 16-bit kernels' inner-solver
@@ -1150,7 +1142,7 @@ __device__ __forceinline__ void grid_reduce_rhs(double (&v)[NV], int rhs_log2, c
 // instructions hold the FP64 pipe 64 cycles per warp); the block and grid
 // sums stay in double and in a fixed order.
 template <int NV>
-__device__ __forceinline__ void grid_reduce_rhs(float (&vf)[NV], int rhs_log2, const Reduction &red,
+__device__ __forceinline__ bool grid_reduce_rhs(float (&vf)[NV], int rhs_log2, const Reduction &red,
                                                 FinalizeKind kind, CgState *st, double *out)
 {
     const int n = 1 << rhs_log2;
@@ -1160,7 +1152,7 @@ __device__ __forceinline__ void grid_reduce_rhs(float (&vf)[NV], int rhs_log2, c
         for (int off = 16; off >= n; off >>= 1) vf[k] += __shfl_xor_sync(0xffffffffu, vf[k], off);
         v[k] = (double)vf[k];
     }
-    grid_reduce_rhs_warp_summed<NV>(v, rhs_log2, red, kind, st, out);
+    return grid_reduce_rhs_warp_summed<NV>(v, rhs_log2, red, kind, st, out);
 }
 
 // ------------------------------------------------------------------ launch API

@@ -32,6 +32,14 @@ cudaError_t launch_norm2(const FieldView &f, const Reduction &red, FinalizeKind 
 cudaError_t launch_diff_norm2(const FieldView &a, const FieldView &b, const Reduction &red, double *out,
                               cudaStream_t s);
 
+// The conditional nodes of a CG graph, which kernels of its body set: the loop
+// goes on while the state is RUNNING (and within its caps), the reliable
+// update runs when an iteration asked for it.  Off outside a graph.
+struct CgGraphControl {
+    cudaGraphConditionalHandle loop, reliable;
+    bool on;
+};
+
 // CG vector steps.  The CG state lives on the device; every kernel below
 // except cg_true_residual returns at once unless state->status is RUNNING.
 // One double per right-hand side (kernel parameter).
@@ -43,12 +51,13 @@ cudaError_t launch_cg_state_init(CgState *st, int nrhs, const RhsValues &tol2, d
 // r = rhs (cast), p = r, x = 0, xs = 0 (if given); rr = |rhs|^2; status.
 cudaError_t launch_cg_setup(const FieldView &rhs, const FieldView &r, const FieldView &p, const FieldView &x,
                             const FieldView *xs, const Reduction &red, CgState *st, cudaStream_t s);
-// x += alpha p, r -= alpha q, |r|^2 -> beta / status.  x is F64 (plain) or
-// F32 (mixed), p, r, q share one precision.
+// x += alpha p, r -= alpha q, |r|^2 -> beta / status, and the conditions of the
+// graph.  x is F64 (plain) or F32 (mixed); p, r, q share one precision (an FP64
+// p may be in fixed point).
 cudaError_t launch_cg_xr(const FieldView &x, const FieldView &p, const FieldView &r, const FieldView &q,
-                         const Reduction &red, CgState *st, cudaStream_t s);
-// p = r + beta p
-cudaError_t launch_cg_p(const FieldView &p, const FieldView &r, CgState *st, cudaStream_t s);
+                         const Reduction &red, CgState *st, cudaStream_t s, const CgGraphControl &ctl);
+// p = r + beta p; with `ctl` it sets the loop condition (the last kernel of a reliable update)
+cudaError_t launch_cg_p(const FieldView &p, const FieldView &r, CgState *st, cudaStream_t s, const CgGraphControl &ctl);
 // xhi += xs, xs = 0 (mixed precision, before a reliable update)
 cudaError_t launch_cg_accum_x(const FieldView &xhi, const FieldView &xs, cudaStream_t s);
 // rho = rhs0 - q (F64 defect of the un-normalised system) and rs = cast(rho).
@@ -59,11 +68,6 @@ cudaError_t launch_cg_verify(const FieldView &f, const Reduction &red, CgState *
 // rhi = rhs - q (F64), |rhi|^2 -> reliable-update decision; rs = cast(rhi) if given.
 cudaError_t launch_cg_true_residual(const FieldView &rhs, const FieldView &q, const FieldView &rhi,
                                    const FieldView *rs, const Reduction &red, CgState *st, cudaStream_t s);
-
-
-// Graph control kernels (cudaGraphSetConditional on the loop / reliable-update handles).
-cudaError_t launch_cg_ctrl_reliable(const CgState *st, cudaGraphConditionalHandle h, cudaStream_t s);
-cudaError_t launch_cg_ctrl_loop(CgState *st, cudaGraphConditionalHandle h, cudaStream_t s);
 
 // Copy between rhs 0..n-1 of a batched field and n plain fields of the same
 // precision and halves, in one launch: to_batch = 1 copies plain[k] ->

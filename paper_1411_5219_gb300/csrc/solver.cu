@@ -259,18 +259,18 @@ struct CgFields {
 // One CG iteration: q = A p (|Mhat p|^2 -> alpha), x += alpha p, r -= alpha q
 // (|r|^2 -> beta and status), p = r + beta p.  All return at once unless
 // the state is RUNNING.
-cudaError_t enqueue_iteration(const CgFields &f, cudaStream_t s)
+cudaError_t enqueue_iteration(const CgFields &f, cudaStream_t s, const CgGraphControl &ctl)
 {
     cudaError_t e = apply_normal(f.c, f.Us, f.rs_recon, f.ps, f.qs, f.ts, f.ss, true, true, s);
-    if (e == cudaSuccess) e = launch_cg_xr(f.mixed ? f.xs : f.xh, f.ps, f.rs, f.qs, f.red, f.state, s);
-    if (e == cudaSuccess) e = launch_cg_p(f.ps, f.rs, f.state, s);
+    if (e == cudaSuccess) e = launch_cg_xr(f.mixed ? f.xs : f.xh, f.ps, f.rs, f.qs, f.red, f.state, s, ctl);
+    if (e == cudaSuccess) e = launch_cg_p(f.ps, f.rs, f.state, s, CgGraphControl{});
     return e;
 }
 
 // Reliable update / convergence check: x += xs (mixed), r = rhs - A x in
 // FP64 (|r|^2 -> DONE or RUNNING with beta = |r|^2 / |r_prev|^2), r_inner =
 // cast(r), then p = r + beta p.
-cudaError_t enqueue_true_residual(const CgFields &f, cudaStream_t s)
+cudaError_t enqueue_true_residual(const CgFields &f, cudaStream_t s, const CgGraphControl &ctl)
 {
     cudaError_t e = cudaSuccess;
     if (f.split) {
@@ -296,13 +296,13 @@ cudaError_t enqueue_true_residual(const CgFields &f, cudaStream_t s)
         }
         if (e == cudaSuccess) e = apply_dag(f.c, f.Uh, f.rh_recon, f.rh, f.qh, f.th, check, s);
         if (e == cudaSuccess) e = launch_cg_verify(f.qh, f.red, f.state, s);
-        if (e == cudaSuccess) e = launch_cg_p(f.ps, f.rs, f.state, s);
+        if (e == cudaSuccess) e = launch_cg_p(f.ps, f.rs, f.state, s, ctl);
         return e;
     }
     if (f.mixed) e = launch_cg_accum_x(f.xh, f.xs, s);
     if (e == cudaSuccess) e = apply_normal(f.c, f.Uh, f.rh_recon, f.xh, f.qh, f.th, f.sh, false, false, s);
     if (e == cudaSuccess) e = launch_cg_true_residual(f.rhs, f.qh, f.rh, f.mixed ? &f.rs : nullptr, f.red, f.state, s);
-    if (e == cudaSuccess) e = launch_cg_p(f.ps, f.rs, f.state, s);
+    if (e == cudaSuccess) e = launch_cg_p(f.ps, f.rs, f.state, s, ctl);
     return e;
 }
 
@@ -340,9 +340,9 @@ cudaError_t cg_eager(const qcd_lattice *lat, const CgFields &f, cudaStream_t s)
         const int status = lat->state_host->status;
         if (status == CG_DONE || status == CG_BREAKDOWN || status == CG_MAXITER) return cudaSuccess;
         if (status == CG_CONVERGED || status == CG_RELIABLE)
-            if ((e = enqueue_true_residual(f, s)) != cudaSuccess) return e;
+            if ((e = enqueue_true_residual(f, s, CgGraphControl{})) != cudaSuccess) return e;
         for (int k = 0; k < batch; ++k)
-            if ((e = enqueue_iteration(f, s)) != cudaSuccess) return e;
+            if ((e = enqueue_iteration(f, s, CgGraphControl{})) != cudaSuccess) return e;
         if ((e = read_state(lat, s)) != cudaSuccess) return e;
         const CgState &hs = *lat->state_host;
         const int done = hs.iter - last_iter;
@@ -360,8 +360,9 @@ cudaError_t cg_eager(const qcd_lattice *lat, const CgFields &f, cudaStream_t s)
 
 // The CG loop as one CUDA graph: a WHILE node whose body runs one iteration,
 // then an IF node that runs the reliable update when the iteration asked
-// for it, then a control kernel that keeps the loop going while the state
-// is RUNNING (bounded by iter < maxiter and a trip cap).  Built once per
+// for it.  The last kernel of either sets the loop condition, true while the
+// state is RUNNING (bounded by iter < maxiter and a trip cap); control kernels
+// of their own cost two launches an iteration.  Built once per
 // configuration and field addresses and cached on the lattice.
 qcd_status cg_graph(const qcd_lattice *lat, const CgFields &f, cudaGraphExec_t *out)
 {
@@ -399,6 +400,7 @@ qcd_status cg_graph(const qcd_lattice *lat, const CgFields &f, cudaGraphExec_t *
     if (e == cudaSuccess) e = (x);
     G_TRY(cudaGraphConditionalHandleCreate(&hloop, g, 1, cudaGraphCondAssignDefault));
     G_TRY(cudaGraphConditionalHandleCreate(&hrel, g, 0, cudaGraphCondAssignDefault));
+    const CgGraphControl ctl{hloop, hrel, true};
     cudaGraphNodeParams wp{};
     wp.type = cudaGraphNodeTypeConditional;
     wp.conditional.handle = hloop;
@@ -409,8 +411,7 @@ qcd_status cg_graph(const qcd_lattice *lat, const CgFields &f, cudaGraphExec_t *
     // body: one iteration, then the reliable-update decision
     G_TRY(cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
     if (e == cudaSuccess) {
-        cudaError_t ec = enqueue_iteration(f, cs);
-        if (ec == cudaSuccess) ec = launch_cg_ctrl_reliable(f.state, hrel, cs);
+        cudaError_t ec = enqueue_iteration(f, cs, ctl);
         if (ec == cudaSuccess) ec = cudaStreamGetCaptureInfo(cs, &cst, nullptr, nullptr, &deps, nullptr, &ndeps);
         if (ec == cudaSuccess && cst != cudaStreamCaptureStatusActive) ec = cudaErrorStreamCaptureInvalidated;
         if (ec == cudaSuccess && ndeps > 0 && !deps) ec = cudaErrorStreamCaptureInvalidated;
@@ -428,17 +429,10 @@ qcd_status cg_graph(const qcd_lattice *lat, const CgFields &f, cudaGraphExec_t *
         cudaGraph_t ibody = ip.conditional.phGraph_out[0];
         e = cudaStreamBeginCaptureToGraph(cs, ibody, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
-            cudaError_t ec = enqueue_true_residual(f, cs);
+            cudaError_t ec = enqueue_true_residual(f, cs, ctl);
             cudaError_t ee = cudaStreamEndCapture(cs, &tmp);
             e = ec != cudaSuccess ? ec : ee;
         }
-    }
-    // after the IF node: the loop condition
-    G_TRY(cudaStreamBeginCaptureToGraph(cs, body, &inode, nullptr, 1, cudaStreamCaptureModeThreadLocal));
-    if (e == cudaSuccess) {
-        cudaError_t ec = launch_cg_ctrl_loop(f.state, hloop, cs);
-        cudaError_t ee = cudaStreamEndCapture(cs, &tmp);
-        e = ec != cudaSuccess ? ec : ee;
     }
     G_TRY(cudaGraphInstantiate(&exec, g, 0));
 #undef G_TRY
@@ -568,7 +562,7 @@ qcd_status qcd::solve_impl(const qcd_gauge *g, qcd_spinor *const *x, const qcd_s
     // reduction scratch: NV (<= 2) x N partials per block of the largest grid
     Reduction red = reduction_of(lat);
     if (N > 1) {
-        const size_t bmax = ((size_t)2 * (lat->h << L) + 63) / 64;
+        const size_t bmax = ((size_t)2 * (lat->h << L) + 31) / 32;  // (the FP64 x/r update: 32 elements a block)
         const size_t need = std::max(red_partials_needed(2 * (size_t)N, bmax), red_partials_needed(N, bmax));
         red.partials = static_cast<double *>(workspace(lat, "cg_partials", need * sizeof(double)));
         red.cap = need;
@@ -708,11 +702,11 @@ qcd_status qcd::solve_impl(const qcd_gauge *g, qcd_spinor *const *x, const qcd_s
         }
         QCD_TRY(cudaGraphLaunch(exec, s), "solve_cg: graph launch");
         QCD_TRY(read_state(lat, s), "solve_cg: state");
-        // kernels the graph ran: per trip the iteration and two control
-        // kernels, per reliable update its body
+        // kernels the graph ran: per trip the iteration, per reliable update
+        // its body
         const int op = c.eo ? 4 : 2;
         const int per_update = split ? (c.eo ? 10 : 7) + (mid ? 1 : 0) : op + 2 + (mixed ? 1 : 0);
-        note_launches(lat->state_host->trips * (op + 4) + lat->state_host->reliable_updates * per_update);
+        note_launches(lat->state_host->trips * (op + 2) + lat->state_host->reliable_updates * per_update);
     } else {
         QCD_TRY(cg_eager(lat, F, s), "solve_cg: iterations");
     }
