@@ -157,7 +157,7 @@ __global__ void cg_state_init_kernel(CgState *s, int nrhs, const RhsValues tol2,
     s->maxiter = maxiter;
     s->status = CG_RUNNING;
     s->reliable_updates = 0;
-    s->trips = 0;
+    s->trips = s->skipped = 0;
     s->trip_limit = maxiter + 64;
 }
 
@@ -169,9 +169,10 @@ __device__ __forceinline__ void set_loop(const CgGraphControl &ctl, const CgStat
     const bool go = st->status == CG_RUNNING && st->iter < st->maxiter && st->trips < st->trip_limit;
     cudaGraphSetConditional(ctl.loop, go ? 1u : 0u);
 }
-__device__ __forceinline__ void set_iteration(const CgGraphControl &ctl, CgState *st)
+__device__ __forceinline__ void set_iteration(const CgGraphControl &ctl, CgState *st, bool ran)
 {
-    st->trips += 1;
+    st->trips += ran ? 1 : 0;
+    st->skipped += ran ? 0 : 1;
     cudaGraphSetConditional(ctl.reliable, (st->status == CG_RELIABLE || st->status == CG_CONVERGED) ? 1u : 0u);
     set_loop(ctl, st);
 }
@@ -202,8 +203,8 @@ __global__ void __launch_bounds__(kThreads) cg_xr_kernel(const FieldView x, cons
                                                          const FieldView q, const Reduction red, CgState *stt,
                                                          const CgGraphControl ctl)
 {
-    if (stt->status != CG_RUNNING) {  // (a breakdown in this iteration ends the loop)
-        if (ctl.on && blockIdx.x == 0 && threadIdx.x == 0) set_iteration(ctl, stt);
+    if (stt->status != CG_RUNNING) {  // (an update is due, or a breakdown ends the loop)
+        if (ctl.on && blockIdx.x == 0 && threadIdx.x == 0) set_iteration(ctl, stt, false);
         return;
     }
     using R = typename SF::R;
@@ -231,7 +232,7 @@ __global__ void __launch_bounds__(kThreads) cg_xr_kernel(const FieldView x, cons
         st<SF>(r, k, rr);
         v[0] = (RedT)norm2(rr);
     }
-    if (grid_reduce_rhs<1>(v, x.rhs_log2, red, FIN_CG_RR, stt, nullptr) && ctl.on) set_iteration(ctl, stt);
+    if (grid_reduce_rhs<1>(v, x.rhs_log2, red, FIN_CG_RR, stt, nullptr) && ctl.on) set_iteration(ctl, stt, true);
 }
 
 // The same in FP64, one thread per element and spin (a block's warps take the
@@ -246,7 +247,7 @@ __global__ void __launch_bounds__(kThreads) cg_xr_spin_kernel(const FieldView x,
                                                               const CgGraphControl ctl)
 {
     if (stt->status != CG_RUNNING) {
-        if (ctl.on && blockIdx.x == 0 && threadIdx.x == 0) set_iteration(ctl, stt);
+        if (ctl.on && blockIdx.x == 0 && threadIdx.x == 0) set_iteration(ctl, stt, false);
         return;
     }
     const int spin = threadIdx.x >> 5, k = blockIdx.x * 32 + (threadIdx.x & 31);
@@ -273,7 +274,7 @@ __global__ void __launch_bounds__(kThreads) cg_xr_spin_kernel(const FieldView x,
             v[0] = fma(rr.x, rr.x, fma(rr.y, rr.y, v[0]));
         }
     }
-    if (grid_reduce_rhs<1>(v, x.rhs_log2, red, FIN_CG_RR, stt, nullptr) && ctl.on) set_iteration(ctl, stt);
+    if (grid_reduce_rhs<1>(v, x.rhs_log2, red, FIN_CG_RR, stt, nullptr) && ctl.on) set_iteration(ctl, stt, true);
 }
 
 // p = r + beta p
@@ -418,8 +419,12 @@ static dim3 grid_of(const FieldView &f) { return dim3(site_blocks(nsites(f))); }
 cudaError_t launch_convert(const FieldView &dst, const FieldView &src, cudaStream_t s)
 {
     if (dst.prec == kPrecFix) {
-        if (src.prec != QCD_PREC_F64) return cudaErrorInvalidValue;
-        convert_kernel<SpFix, SpF64><<<grid_of(dst), kThreads, 0, s>>>(dst, src);
+        if (src.prec == QCD_PREC_F64)
+            convert_kernel<SpFix, SpF64><<<grid_of(dst), kThreads, 0, s>>>(dst, src);
+        else if (src.prec == QCD_PREC_DF64)
+            convert_kernel<SpFix, SpDF64><<<grid_of(dst), kThreads, 0, s>>>(dst, src);
+        else
+            return cudaErrorInvalidValue;
         note_launches();
         return cudaGetLastError();
     }

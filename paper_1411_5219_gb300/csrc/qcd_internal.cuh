@@ -898,7 +898,8 @@ struct CgState {
     int iter, maxiter;
     int status;       // global
     int reliable_updates;
-    int trips, trip_limit;  // device-driven loop: body executions and their cap
+    int trips, trip_limit;  // device-driven loop: iterations run and their cap
+    int skipped;            // iterations of a body whose kernels returned at once
 };
 
 // What the last block does with a finished reduction.
