@@ -6,6 +6,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <initializer_list>
 #include <mutex>
 #include <new>
 #include <vector>
@@ -397,7 +398,8 @@ GaugeView gauge_view(const qcd_gauge *g, int prec, int recon, cudaStream_t s, qc
 GaugeView hop_links(const qcd_gauge *g, int prec, int recon, cudaStream_t s, qcd_status *st)
 {
     GaugeView v = gauge_view(g, prec, recon, s, st);
-    if (*st != QCD_OK || prec != QCD_PREC_F64 || g->prec != prec || g->recon != recon) return v;
+    const bool df = prec == QCD_PREC_DF64 && recon == 18;
+    if (*st != QCD_OK || (prec != QCD_PREC_F64 && !df) || g->prec != QCD_PREC_F64 || g->recon != recon) return v;
     auto *gm = const_cast<qcd_gauge *>(g);
     std::lock_guard<std::mutex> lk(derived_mu);
     if (g->fix_state == qcd_gauge::FIX_STALE) {
@@ -415,7 +417,8 @@ GaugeView hop_links(const qcd_gauge *g, int prec, int recon, cudaStream_t s, qcd
             return v;
         }
         bool fits = false;
-        const cudaError_t e = gauge_to_fix(static_cast<int4 *>(gm->fix), v, recon, g->lat->geom, s, &fits);
+        const cudaError_t e = gauge_to_fix(static_cast<int4 *>(gm->fix), GaugeView{g->data, g->lat->stride, nullptr}, recon,
+                                           g->lat->geom, s, &fits);
         if (e != cudaSuccess) {
             *st = check_cuda(e, "fixed-point links");
             return v;
@@ -682,21 +685,34 @@ static cudaError_t profiled(int prec, int recon, double sites, int n, int fields
     return e;
 }
 
+// True when workspace fields of these names, precisions and halves exist or
+// may be allocated (not under stream capture).
+struct WsWanted {
+    const char *name;
+    int prec, nh;
+};
+static bool ws_available(const qcd_lattice *lat, int rhs_log2, int stride, std::initializer_list<WsWanted> fields, cudaStream_t s)
+{
+    bool have = true;
+    for (const WsWanted &f : fields) {
+        if (f.nh == 0) continue;
+        const auto it = lat->ws.find(ws_name(f.name, f.prec, rhs_log2));
+        have = have && it != lat->ws.end() &&
+               it->second.second >= f.nh * (spinor_half_bytes(f.prec, stride) + spinor_half_norm_bytes(f.prec, stride));
+    }
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (have || (cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone)) return true;
+    cudaGetLastError();
+    return false;
+}
+
 // Whether the fixed-point kernel can take a launch: with its input to be
 // brought into that form, `in` becomes that workspace field (not allocated
 // under stream capture, where a launch without it stays with FP64).
 static bool fix_input(const qcd_lattice *lat, const FieldView *&in, FieldView &ws, cudaStream_t s)
 {
     if (in->prec == kPrecFix) return true;
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    const auto it = lat->ws.find(ws_name("hop_in", kPrecFix, in->rhs_log2));
-    const size_t have = it == lat->ws.end() ? 0 : it->second.second;
-    const int stride = in->hv[0].stride;
-    const size_t need = in->nh * (spinor_half_bytes(kPrecFix, stride) + spinor_half_norm_bytes(kPrecFix, stride));
-    if (have < need && (cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone)) {
-        cudaGetLastError();
-        return false;
-    }
+    if (!ws_available(lat, in->rhs_log2, in->hv[0].stride, {{"hop_in", kPrecFix, in->nh}}, s)) return false;
     ws = ws_field(lat, "hop_in", in->nh, kPrecFix, in->rhs_log2);
     if (!ws.hv[0].data) return false;
     if (launch_convert(ws, *in, s) != cudaSuccess) return false;
@@ -704,8 +720,43 @@ static bool fix_input(const qcd_lattice *lat, const FieldView *&in, FieldView &w
     return true;
 }
 
+// A double-float hop through the fixed-point FP64 kernel: its input and y in
+// fixed point, its FP64 result rounded to double-float.  The double-float
+// kernel issues ~11,000 FP32 instructions a site at 200 registers: a hop and a
+// conversion of its result to FP64 took 1028 us at 48^3 x 12 and 79.7 at
+// 24^3 x 8, here 513 and 64.1 (the hop and five passes over its fields, bound
+// by HBM), with an error of 8e-16 instead of 4e-15.  `done` is false where the workspace is not to be had.
+static cudaError_t hop_df64(const qcd_lattice *lat, const GaugeView &U, int recon, const HopArgs &h, cudaStream_t s, bool *done)
+{
+    const int nh = h.both ? 2 : 1, L = h.out->rhs_log2;
+    *done = false;
+    if (!ws_available(lat, L, h.out->hv[0].stride,
+                      {{"hop_in", kPrecFix, nh}, {"df_y", kPrecFix, h.y ? nh : 0}, {"df_out", QCD_PREC_F64, nh}}, s))
+        return cudaSuccess;
+    const FieldView in = ws_field(lat, "hop_in", nh, kPrecFix, L), out = ws_field(lat, "df_out", nh, QCD_PREC_F64, L);
+    const FieldView y = h.y ? ws_field(lat, "df_y", nh, kPrecFix, L) : FieldView{};
+    if (!in.hv[0].data || !out.hv[0].data || (h.y && !y.hv[0].data)) return cudaSuccess;
+    *done = true;
+    HopArgs f = h;
+    f.in = &in;
+    f.out = &out;
+    f.y = h.y ? &y : nullptr;
+    f.count_as = QCD_PREC_DF64;
+    cudaError_t e = launch_convert(in, *h.in, s);
+    if (e == cudaSuccess && h.y) e = launch_convert(y, *h.y, s);
+    if (e == cudaSuccess) e = hop(lat, U, recon, f, s);
+    if (e == cudaSuccess) e = launch_convert(*h.out, out, s);
+    return e;
+}
+
 cudaError_t hop(const qcd_lattice *lat, const GaugeView &U, int recon, const HopArgs &h, cudaStream_t s)
 {
+    // (a launch that may return at once would have its result rounded all the same)
+    if (h.out->prec == QCD_PREC_DF64 && U.fix && !h.check_status) {
+        bool done;
+        const cudaError_t e = hop_df64(lat, U, recon, h, s, &done);
+        if (done || e != cudaSuccess) return e;
+    }
     // fields in fixed point are FP64 fields as far as the launch shape goes
     const int prec = h.out->prec == kPrecFix ? (int)QCD_PREC_F64 : h.out->prec;
     const bool fix_fields = h.in->prec == kPrecFix || h.out->prec == kPrecFix || (h.y && h.y->prec == kPrecFix);
@@ -769,7 +820,7 @@ cudaError_t hop(const qcd_lattice *lat, const GaugeView &U, int recon, const Hop
     a.red_out = lat->red_out;
     a.check_status = h.check_status;
     a.run_status = h.run_status;
-    return profiled(prec, recon, lat->h * (h.both ? 2.0 : 1.0), 1 << h.out->rhs_log2, h.y ? 3 : 2, s,
+    return profiled(h.count_as ? h.count_as : prec, recon, lat->h * (h.both ? 2.0 : 1.0), 1 << h.out->rhs_log2, h.y ? 3 : 2, s,
                     [&] { return launch_dslash(prec, recon, a, s); });
 }
 
