@@ -19,11 +19,12 @@
 // * Hopping phases use sixteen threads per site, one hop and one spin each,
 //   in fixed point (fix_lanes.cuh); where the links do not fit that form,
 //   eight threads per site in FP64 (hop_lanes.cuh).  Bound by latency: at
-//   8^3 x 4 an iteration takes 42 us for six phases of one pass each.  Twelve
-//   systems of 432 to 5184 sites per parity: 17.4 ms with FP64 phases, one
-//   barrier over all blocks and its last block adding up every system in
-//   turn; 10.8 ms with the fixed-point phases; 7.8 ms with a barrier per
-//   system, whose last block sums that system alone.
+//   8^3 x 4 an iteration takes 38 us for six phases of one pass each (42 us
+//   when each barrier read its generation, the error flag and the status from
+//   memory).  Twelve systems of 432 to 5184 sites per parity: 17.4 ms with FP64
+//   phases, one barrier over all blocks and its last block adding up every
+//   system in turn; 10.8 ms with the fixed-point phases; 7.7 ms with a barrier
+//   per system, whose last block sums that system alone.
 // * Every barrier wait is bounded by a clock64 budget.  When it runs out the
 //   kernel records QCD_ERR_TIMEOUT and every block returns; the call then
 //   fails with that status and the context stays usable.
@@ -98,7 +99,7 @@ struct alignas(128) ManySysState {
     int iter;              // CG iterations
     int reliable;          // true-residual passes
     unsigned arrive;       // arrivals at this system's barrier (zero at launch)
-    unsigned gen;          // generation of that barrier
+    unsigned gen;          // barriers passed
 };
 
 struct ManyState {
@@ -145,21 +146,22 @@ __device__ __forceinline__ double chunk_sum(const Ctx &x, int slot, int k, int i
     return block_total(a);
 }
 
-// A barrier over the blocks of system k (the systems do not wait for one
-// another).  Before it, each block has written its chunk partials for this
-// phase; the last block to arrive runs `fin` with all its threads (sums, CG
-// decisions by thread 0), then releases the others.  Returns false when the
-// wait ran out, here or in another system (the kernel must return).
+// Barrier number `where` (0, 1, ...) over the blocks of system k; the systems
+// do not wait for one another.  Before it, each block has written its chunk
+// partials for this phase; the last block to arrive runs `fin` with all its
+// threads (sums, CG decisions by thread 0), then releases the others.
+// Returns false when the wait ran out, here or in another block (the kernel
+// must return).  The generation is the barrier's number, known to every block,
+// and the error flag is read while waiting only: each read of global memory
+// that all blocks wait for costs a third of a microsecond.
 template <typename Fin>
 __device__ bool sys_barrier(const Ctx &x, int k, int where, Fin fin)
 {
     __shared__ int ok, last;
-    __shared__ unsigned my_gen;
     ManySysState &q = x.st->s[k];
     __syncthreads();
     if (threadIdx.x == 0) {
         ok = 1;
-        my_gen = *(volatile unsigned *)&q.gen;
         __threadfence();
         last = atomicAdd(&q.arrive, 1u) == (unsigned)x.sys[k].nblocks - 1;
     }
@@ -171,13 +173,14 @@ __device__ bool sys_barrier(const Ctx &x, int k, int where, Fin fin)
         if (threadIdx.x == 0) {
             q.arrive = 0;
             __threadfence();
-            atomicAdd(&q.gen, 1u);
+            *(volatile unsigned *)&q.gen = (unsigned)where + 1u;
         }
     } else if (threadIdx.x == 0) {
         volatile unsigned *genp = &q.gen;
         const long long t0 = clock64();
-        while (*genp == my_gen) {
-            if (*(volatile int *)&x.st->error != 0 || clock64() - t0 > x.budget) {
+        for (unsigned poll = 0; *genp != (unsigned)where + 1u; ++poll) {
+            const bool out = clock64() - t0 > x.budget;
+            if (out || ((poll & 15u) == 15u && *(volatile int *)&x.st->error != 0)) {
                 if (atomicCAS(&x.st->error, 0, QCD_ERR_TIMEOUT) == 0) x.st->timeout_where = where;
                 ok = 0;
                 break;
@@ -185,7 +188,6 @@ __device__ bool sys_barrier(const Ctx &x, int k, int where, Fin fin)
         }
         __threadfence();
     }
-    if (threadIdx.x == 0 && *(volatile int *)&x.st->error != 0) ok = 0;
     __syncthreads();
     return ok != 0;
 }
@@ -223,12 +225,10 @@ __device__ __forceinline__ int hop_threads(const ManySys &S) { return S.fix ? 16
 // optionally |out|^2 -> slot.  Without `out`, |b - that|^2 is reduced and
 // nothing is stored.
 __device__ void hop_phase(const Ctx &x, int k, int lb, int coef, int p, bool dagger, HV ManySys::*in, HV ManySys::*y,
-                          HV ManySys::*out, int red_slot, bool skip_done)
+                          HV ManySys::*out, int red_slot)
 {
     const ManySys &S = x.sys[k];
     const PhaseCoef &pc = S.pc[coef];
-    const int run = __ldcg(&x.st->s[k].status);
-    if (skip_done && run != MS_RUNNING) return;
     // (copies: a store through a field would have the compiler load the
     // descriptor again in every pass of the loop)
     const Geom g = S.g;
@@ -383,11 +383,11 @@ __global__ void __launch_bounds__(kManyThreads, 3) many_cg_kernel(const ManySys 
     //      rhs = A^dag b' - kappa^2 D_eo^dag t (|rhs|^2) ; r = p = rhs, x_e = 0
     vec_phase(x, k, lb, V_TWIST_BO, -1);
     QCD_SYNC(;)
-    hop_phase(x, k, lb, MC_SRC_B, 0, false, &ManySys::t, &ManySys::be, &ManySys::bp, -1, false);
+    hop_phase(x, k, lb, MC_SRC_B, 0, false, &ManySys::t, &ManySys::be, &ManySys::bp, -1);
     QCD_SYNC(;)
-    hop_phase(x, k, lb, MC_SRC_T, 1, true, &ManySys::bp, nullptr, &ManySys::t, -1, false);
+    hop_phase(x, k, lb, MC_SRC_T, 1, true, &ManySys::bp, nullptr, &ManySys::t, -1);
     QCD_SYNC(;)
-    hop_phase(x, k, lb, MC_SRC_R, 0, true, &ManySys::t, &ManySys::bp, &ManySys::rhs, 0, false);
+    hop_phase(x, k, lb, MC_SRC_R, 0, true, &ManySys::t, &ManySys::bp, &ManySys::rhs, 0);
     QCD_SYNC({
         const double b2 = chunk_sum(x, 0, k, ht);
         if (threadIdx.x == 0) {
@@ -406,9 +406,9 @@ __global__ void __launch_bounds__(kManyThreads, 3) many_cg_kernel(const ManySys 
         const int status = __ldcg(&q.status);
         if (status == MS_RUNNING && __ldcg(&q.iter) < st->maxiter) {
             // ---- one CG iteration
-            hop_phase(x, k, lb, MC_OP1, 1, false, &ManySys::p, nullptr, &ManySys::t, -1, true);
+            hop_phase(x, k, lb, MC_OP1, 1, false, &ManySys::p, nullptr, &ManySys::t, -1);
             QCD_SYNC(;)
-            hop_phase(x, k, lb, MC_OP2, 0, false, &ManySys::t, &ManySys::p, &ManySys::s, 0, true);
+            hop_phase(x, k, lb, MC_OP2, 0, false, &ManySys::t, &ManySys::p, &ManySys::s, 0);
             QCD_SYNC({
                 const double pAp = chunk_sum(x, 0, k, ht);
                 if (threadIdx.x == 0) {
@@ -421,9 +421,9 @@ __global__ void __launch_bounds__(kManyThreads, 3) many_cg_kernel(const ManySys 
                     }
                 }
             })
-            hop_phase(x, k, lb, MC_OP3, 1, true, &ManySys::s, nullptr, &ManySys::t, -1, true);
+            hop_phase(x, k, lb, MC_OP3, 1, true, &ManySys::s, nullptr, &ManySys::t, -1);
             QCD_SYNC(;)
-            hop_phase(x, k, lb, MC_OP4, 0, true, &ManySys::t, &ManySys::s, &ManySys::q, -1, true);
+            hop_phase(x, k, lb, MC_OP4, 0, true, &ManySys::t, &ManySys::s, &ManySys::q, -1);
             QCD_SYNC(;)
             vec_phase(x, k, lb, V_XR, 0);
             QCD_SYNC({
@@ -446,13 +446,13 @@ __global__ void __launch_bounds__(kManyThreads, 3) many_cg_kernel(const ManySys 
         } else if (status == MS_CONVERGED) {
             // ---- FP64 true residual: q = Mhat^dag Mhat x_e (via s, t), r = rhs - q;
             //      DONE if it meets the target, else CG restarts from it
-            hop_phase(x, k, lb, MC_OP1, 1, false, &ManySys::xe, nullptr, &ManySys::t, -1, false);
+            hop_phase(x, k, lb, MC_OP1, 1, false, &ManySys::xe, nullptr, &ManySys::t, -1);
             QCD_SYNC(;)
-            hop_phase(x, k, lb, MC_OP2, 0, false, &ManySys::t, &ManySys::xe, &ManySys::s, -1, false);
+            hop_phase(x, k, lb, MC_OP2, 0, false, &ManySys::t, &ManySys::xe, &ManySys::s, -1);
             QCD_SYNC(;)
-            hop_phase(x, k, lb, MC_OP3, 1, true, &ManySys::s, nullptr, &ManySys::t, -1, false);
+            hop_phase(x, k, lb, MC_OP3, 1, true, &ManySys::s, nullptr, &ManySys::t, -1);
             QCD_SYNC(;)
-            hop_phase(x, k, lb, MC_OP4, 0, true, &ManySys::t, &ManySys::s, &ManySys::q, -1, false);
+            hop_phase(x, k, lb, MC_OP4, 0, true, &ManySys::t, &ManySys::s, &ManySys::q, -1);
             QCD_SYNC(;)
             vec_phase(x, k, lb, V_TRUE, 0);
             QCD_SYNC({
@@ -480,11 +480,11 @@ __global__ void __launch_bounds__(kManyThreads, 3) many_cg_kernel(const ManySys 
         }
     }
     // ---- odd sites x_o = A^-1 b_o + kappa A^-1 D_oe x_e, then |b - M x|^2, |b|^2
-    hop_phase(x, k, lb, MC_RECON, 1, false, &ManySys::xe, &ManySys::bo, &ManySys::xo, -1, false);
+    hop_phase(x, k, lb, MC_RECON, 1, false, &ManySys::xe, &ManySys::bo, &ManySys::xo, -1);
     QCD_SYNC(;)
     // M x per parity: out = A x - kappa D x (even from x_o, odd from x_e)
-    hop_phase(x, k, lb, MC_FULL, 0, false, &ManySys::xo, &ManySys::xe, nullptr, 0, false);
-    hop_phase(x, k, lb, MC_FULL, 1, false, &ManySys::xe, &ManySys::xo, nullptr, 1, false);
+    hop_phase(x, k, lb, MC_FULL, 0, false, &ManySys::xo, &ManySys::xe, nullptr, 0);
+    hop_phase(x, k, lb, MC_FULL, 1, false, &ManySys::xe, &ManySys::xo, nullptr, 1);
     bnorm_phase(x, k, lb, 2);
     QCD_SYNC({
         const double r0 = chunk_sum(x, 0, k, ht);
