@@ -124,7 +124,8 @@ void qcd_lattice_destroy(qcd_lattice *lat);
  * on the device per (parity, mu) block, site-fastest (SoA, Sec. 4), in
  * precision `prec` and with `recon` reals per link.  The field also keeps
  * derived copies in other precisions, made on the device from this one on
- * first use by a Dslash of that precision.  The field is zero when the
+ * first use by a Dslash of that precision (for F64 a fixed-point copy of 144
+ * bytes per link).  The field is zero when the
  * call returns (it waits for the legacy default stream).  Errors:
  * INVALID_ARG; OOM; CUDA. */
 qcd_status qcd_gauge_create(const qcd_lattice *lat, qcd_prec prec, qcd_recon recon, qcd_gauge **out);
@@ -217,7 +218,9 @@ qcd_status qcd_norm2_noalloc(const double *x_device, size_t n, double *result_de
  * (Sec. 1 and 6).  With out of parity p (EVEN or ODD) and in of parity 1-p
  * this is the block D_eo (p = EVEN) or D_oe (p = ODD); with both FULL it is
  * the hopping term on the whole lattice.  out and in share the precision
- * (F64: FP64 arithmetic; F32/F16/BF16: FP32 arithmetic); the gauge field's
+ * (F64: sums of 60-bit fixed-point products, no less exact than FP64
+ * arithmetic, which links with entries above 1 and sites with extreme or
+ * non-finite values take; F32/F16/BF16: FP32 arithmetic); the gauge field's
  * copy in that precision and with the gauge field's recon is used.
  * Errors: INVALID_ARG (parities, lattices, precisions); CUDA. */
 qcd_status qcd_apply_dslash(const qcd_gauge *g, qcd_spinor *out, const qcd_spinor *in, int dagger, void *stream);
@@ -454,12 +457,14 @@ qcd_status qcd_profile_end(qcd_profile *out);
 /* Number of CUDA kernels this library has launched since it was loaded. */
 unsigned long long qcd_kernel_launches(void);
 
-/* Launch shape of the FP64 reconstruct-18 hopping kernel (one right-hand
- * side): 0 (default) lets the autotuner choose between one thread per
- * output site and eight (one hop each, for small lattices); 1 or 8 forces
- * that choice for later launches (tests and benchmarks of either kernel).
- * The paper compiles kernels per configuration (Sec. 4); here both are
- * compiled and one is picked per lattice.  INVALID_ARG for other values. */
+/* Launch shape of the FP64 hopping kernel (one right-hand side): 0 (default)
+ * chooses by lattice size between the kernel of large lattices (a thread pair
+ * per output site in fixed point, one thread in FP64 arithmetic) and the lane
+ * kernel of small ones (one hop per thread: sixteen in fixed point, eight in
+ * FP64 arithmetic on reconstruct-18 links); 1 or 8 forces the first or the
+ * second for later launches (tests and benchmarks of either kernel).  The
+ * paper compiles kernels per configuration (Sec. 4); here both are compiled
+ * and one is picked per lattice.  INVALID_ARG for other values. */
 qcd_status qcd_set_hop_threads(int threads_per_site);
 
 /* Host-side failure injection for tests of the error paths (no device

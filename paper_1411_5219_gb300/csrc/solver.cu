@@ -539,9 +539,9 @@ qcd_status qcd::solve_impl(const qcd_gauge *g, qcd_spinor *const *x, const qcd_s
     // arithmetic costs more than the bytes it saves)
     const int srecon = !mixed ? g->recon : (sp == QCD_PREC_DF64 ? 18 : prm->inner_recon);
     qcd_status st;
-    const GaugeView Uh = hop_links(g, QCD_PREC_F64, g->recon, s, &st);
+    GaugeView Uh = hop_links(g, QCD_PREC_F64, g->recon, s, &st);
     if (st != QCD_OK) return st;
-    const GaugeView Us = mixed ? gauge_view(g, sp, srecon, s, &st) : Uh;
+    GaugeView Us = mixed ? gauge_view(g, sp, srecon, s, &st) : Uh;
     if (st != QCD_OK) return st;
 
     int L = 0;
@@ -604,9 +604,14 @@ qcd_status qcd::solve_impl(const qcd_gauge *g, qcd_spinor *const *x, const qcd_s
 
     // fixed-point FP64 hops keep the fields that only hops (and p, which the
     // vector updates) read in that form
-    const bool fix = fixed_hops(lat, Uh, QCD_PREC_F64, g->recon, L, !c.eo, s);
+    bool fix = fixed_hops(lat, Uh, QCD_PREC_F64, g->recon, L, !c.eo, s);
+    if (fix && !ws_field(lat, "hop_in", 2, kPrecFix, L).hv[0].data) {
+        // no memory to convert x in: FP64 hops, as for links that do not fit
+        fix = false;
+        Uh.fix = nullptr;
+        if (!mixed) Us.fix = nullptr;
+    }
     const int hp = fix ? kPrecFix : (int)QCD_PREC_F64;
-    if (fix && !ws_field(lat, "hop_in", 2, kPrecFix, L).hv[0].data) return fail(QCD_ERR_OOM, "solve_cg: workspace");
 
     // FP64 fields
     FieldView rhs = c.eo ? ws_field(lat, "cg_rhs", 1, QCD_PREC_F64, L) : bf;
