@@ -6,7 +6,6 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
-#include <initializer_list>
 #include <mutex>
 #include <new>
 #include <vector>
@@ -685,39 +684,31 @@ static cudaError_t profiled(int prec, int recon, double sites, int n, int fields
     return e;
 }
 
-// True when workspace fields of these names, precisions and halves exist or
-// may be allocated (not under stream capture).
-struct WsWanted {
-    const char *name;
-    int prec, nh;
-};
-static bool ws_available(const qcd_lattice *lat, int rhs_log2, int stride, std::initializer_list<WsWanted> fields, cudaStream_t s)
+static bool capturing(cudaStream_t s)
 {
-    bool have = true;
-    for (const WsWanted &f : fields) {
-        if (f.nh == 0) continue;
-        const auto it = lat->ws.find(ws_name(f.name, f.prec, rhs_log2));
-        have = have && it != lat->ws.end() &&
-               it->second.second >= f.nh * (spinor_half_bytes(f.prec, stride) + spinor_half_norm_bytes(f.prec, stride));
-    }
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (have || (cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone)) return true;
+    if (cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone) return false;
     cudaGetLastError();
-    return false;
+    return true;
 }
 
-// Whether the fixed-point kernel can take a launch: with its input to be
-// brought into that form, `in` becomes that workspace field (not allocated
-// under stream capture, where a launch without it stays with FP64).
-static bool fix_input(const qcd_lattice *lat, const FieldView *&in, FieldView &ws, cudaStream_t s)
+// The lattice's workspace for the input of a fixed-point hop of nh halves.  It
+// always holds both: a caller's graph keeps the address of a launch that it
+// captured, so the buffer must not be replaced when a later call needs more.
+static FieldView fix_input_ws(const qcd_lattice *lat, int nh, int rhs_log2)
 {
-    if (in->prec == kPrecFix) return true;
-    if (!ws_available(lat, in->rhs_log2, in->hv[0].stride, {{"hop_in", kPrecFix, in->nh}}, s)) return false;
-    ws = ws_field(lat, "hop_in", in->nh, kPrecFix, in->rhs_log2);
-    if (!ws.hv[0].data) return false;
-    if (launch_convert(ws, *in, s) != cudaSuccess) return false;
-    in = &ws;
-    return true;
+    FieldView f = ws_field(lat, "hop_in", 2, kPrecFix, rhs_log2);
+    f.nh = nh;
+    if (nh == 1) f.hv[1] = f.hv[0];
+    return f;
+}
+
+GaugeView with_fix_input(const qcd_lattice *lat, GaugeView U, int prec, int recon, int rhs_log2, bool both, cudaStream_t s)
+{
+    if (!fixed_hops(lat, U, prec, recon, rhs_log2, both, s)) return U;
+    const bool have = lat->ws.find(ws_name("hop_in", kPrecFix, rhs_log2)) != lat->ws.end();
+    if (!have && (capturing(s) || !fix_input_ws(lat, 1, rhs_log2).hv[0].data)) U.fix = nullptr;
+    return U;
 }
 
 // A double-float hop through the fixed-point FP64 kernel: its input and y in
@@ -725,15 +716,15 @@ static bool fix_input(const qcd_lattice *lat, const FieldView *&in, FieldView &w
 // kernel issues ~11,000 FP32 instructions a site at 200 registers: a hop and a
 // conversion of its result to FP64 took 1028 us at 48^3 x 12 and 79.7 at
 // 24^3 x 8, here 513 and 64.1 (the hop and five passes over its fields, bound
-// by HBM), with an error of 8e-16 instead of 4e-15.  `done` is false where the workspace is not to be had.
+// by HBM), with an error of 8e-16 instead of 4e-15.  `done` is false where the
+// workspace is not to be had, and under stream capture: its fields grow with a
+// later call, so a caller's graph must not hold them.
 static cudaError_t hop_df64(const qcd_lattice *lat, const GaugeView &U, int recon, const HopArgs &h, cudaStream_t s, bool *done)
 {
     const int nh = h.both ? 2 : 1, L = h.out->rhs_log2;
     *done = false;
-    if (!ws_available(lat, L, h.out->hv[0].stride,
-                      {{"hop_in", kPrecFix, nh}, {"df_y", kPrecFix, h.y ? nh : 0}, {"df_out", QCD_PREC_F64, nh}}, s))
-        return cudaSuccess;
-    const FieldView in = ws_field(lat, "hop_in", nh, kPrecFix, L), out = ws_field(lat, "df_out", nh, QCD_PREC_F64, L);
+    if (capturing(s)) return cudaSuccess;
+    const FieldView in = fix_input_ws(lat, nh, L), out = ws_field(lat, "df_out", nh, QCD_PREC_F64, L);
     const FieldView y = h.y ? ws_field(lat, "df_y", nh, kPrecFix, L) : FieldView{};
     if (!in.hv[0].data || !out.hv[0].data || (h.y && !y.hv[0].data)) return cudaSuccess;
     *done = true;
@@ -763,8 +754,15 @@ cudaError_t hop(const qcd_lattice *lat, const GaugeView &U, int recon, const Hop
     const int cfg = fix_fields ? 64 : tuned_tpb(lat, U, prec, recon, h.out->rhs_log2, h.both, s);
     const FieldView *in = h.in;
     FieldView in_ws;
-    const bool fix = prec == QCD_PREC_F64 && U.fix && (cfg >> 16) != 8 && fix_input(lat, in, in_ws, s);
+    const bool fix = prec == QCD_PREC_F64 && U.fix && (cfg >> 16) != 8;
     if (!fix && fix_fields) return cudaErrorInvalidValue;
+    if (fix && in->prec != kPrecFix) {
+        in_ws = fix_input_ws(lat, in->nh, in->rhs_log2);
+        if (!in_ws.hv[0].data) return cudaErrorMemoryAllocation;
+        const cudaError_t e = launch_convert(in_ws, *in, s);
+        if (e != cudaSuccess) return e;
+        in = &in_ws;
+    }
     DslashLaunch a;
     memset(&a, 0, sizeof(a));
     a.g = lat->geom;
@@ -1353,6 +1351,7 @@ qcd_status qcd_apply_dslash(const qcd_gauge *g, qcd_spinor *out, const qcd_spino
     qcd_status st;
     GaugeView U = hop_links(g, out->prec, g->recon, s, &st);
     if (st != QCD_OK) return st;
+    U = with_fix_input(g->lat, U, out->prec, g->recon, 0, both, s);
     const FieldView fo = view_of(out), fi = view_of(in);
     HopArgs h{};
     h.out = &fo;
@@ -1463,6 +1462,7 @@ qcd_status qcd_apply_dslash_multi(const qcd_gauge *g, qcd_spinor *const *out, co
     }
     int L = 0;
     while ((1 << L) < nrhs) ++L;
+    U = with_fix_input(lat, U, prec, g->recon, L, both, s);
     const bool fix = fixed_hops(lat, U, prec, g->recon, L, both, s);
     const FieldView bi = ws_field(lat, "dm_in", nh, fix ? kPrecFix : prec, L), bo = ws_field(lat, "dm_out", nh, prec, L);
     if (!bi.hv[0].data || !bo.hv[0].data) return fail(QCD_ERR_OOM, "apply_dslash_multi: workspace");
@@ -1499,6 +1499,7 @@ qcd_status qcd_apply_M(const qcd_gauge *g, qcd_spinor *out, const qcd_spinor *in
     qcd_status st;
     GaugeView U = hop_links(g, out->prec, g->recon, s, &st);
     if (st != QCD_OK) return st;
+    U = with_fix_input(g->lat, U, out->prec, g->recon, 0, !eo, s);
     const double a = 2.0 * kappa * mu, b = dagger ? -a : a;
     const bool tw = a != 0.0;
     const FieldView fo = view_of(out), fi = view_of(in);
@@ -1515,9 +1516,11 @@ qcd_status qcd_apply_M(const qcd_gauge *g, qcd_spinor *out, const qcd_spinor *in
         h.twisted = tw;
         return check_cuda(hop(g->lat, U, g->recon, h, s), "apply_M");
     }
-    const bool fix = fixed_hops(g->lat, U, out->prec, g->recon, 0, false, s);
-    const FieldView t = ws_field(g->lat, "applyM_t", 1, fix ? kPrecFix : out->prec);
+    // (one buffer for the temporary in either form, so that a captured call
+    // finds the one that an earlier call made whatever kernel it takes)
+    FieldView t = ws_field(g->lat, "applyM_t", 1, out->prec == QCD_PREC_F64 ? kPrecFix : out->prec);
     if (!t.hv[0].data) return fail(QCD_ERR_OOM, "apply_M: workspace");
+    if (!fixed_hops(g->lat, U, out->prec, g->recon, 0, false, s)) t.prec = out->prec;
     h.out = &t;
     h.in = &fi;
     h.y = nullptr;

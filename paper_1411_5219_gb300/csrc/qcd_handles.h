@@ -160,6 +160,13 @@ cudaError_t hop(const qcd_lattice *lat, const GaugeView &U, int recon, const Hop
 bool fixed_hops(const qcd_lattice *lat, const GaugeView &U, int prec, int recon, int rhs_log2, bool both,
                 cudaStream_t s);
 
+// The links for a call's launches: without their fixed-point copy where the
+// fixed-point kernel would want a workspace for its input that is not to be
+// had (no memory, or a first use under stream capture), so that the FP64
+// kernels run.
+GaugeView with_fix_input(const qcd_lattice *lat, GaugeView U, int prec, int recon, int rhs_log2, bool both,
+                         cudaStream_t s);
+
 // The CG solve behind qcd_solve_cg / qcd_solve_cg_multi, with an optional
 // context lattice (scratch, state, graphs) other than the gauge field's.
 // prm holds one parameter set per right-hand side (kappa, mu and tol may

@@ -604,13 +604,9 @@ qcd_status qcd::solve_impl(const qcd_gauge *g, qcd_spinor *const *x, const qcd_s
 
     // fixed-point FP64 hops keep the fields that only hops (and p, which the
     // vector updates) read in that form
-    bool fix = fixed_hops(lat, Uh, QCD_PREC_F64, g->recon, L, !c.eo, s);
-    if (fix && !ws_field(lat, "hop_in", 2, kPrecFix, L).hv[0].data) {
-        // no memory to convert x in: FP64 hops, as for links that do not fit
-        fix = false;
-        Uh.fix = nullptr;
-        if (!mixed) Us.fix = nullptr;
-    }
+    Uh = with_fix_input(lat, Uh, QCD_PREC_F64, g->recon, L, !c.eo, s);
+    if (!mixed) Us = Uh;
+    const bool fix = fixed_hops(lat, Uh, QCD_PREC_F64, g->recon, L, !c.eo, s);
     const int hp = fix ? kPrecFix : (int)QCD_PREC_F64;
 
     // FP64 fields

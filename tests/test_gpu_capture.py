@@ -1,0 +1,142 @@
+"""Operator calls captured into a CUDA graph of the caller: a replay gives the
+result of a call, whatever other calls on the lattice came between (against
+the FP64 oracle).
+
+qcd_set_hop_threads forces the thread pair per site (1), whose input goes
+through a workspace of the lattice, and the sixteen lanes (8), on small
+lattices.
+"""
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_1411_5219_gb300 import synthetic as syn
+from tests import _fields as F
+
+pytestmark = pytest.mark.gpu
+
+DIMS = (6, 4, 2, 8)
+KAPPA, MU = 0.14, 0.02
+
+
+@pytest.fixture(scope="module")
+def q():
+    from paper_1411_5219_gb300 import _build, qcd
+    _build.build()
+    import torch
+    assert torch.cuda.is_available()
+    return qcd
+
+
+@pytest.fixture(params=[1, 8])
+def threads(q, request):
+    q.set_hop_threads(request.param)
+    yield request.param
+    q.set_hop_threads(0)
+
+
+def _setup(q, seed=1701):
+    lat = q.Lattice(DIMS, -1)
+    U = syn.gauge_field(DIMS, 0.3, seed)
+    g = q.Gauge(lat, "f64", 18)
+    g.upload(U)
+    psi = syn.gaussian_spinor(DIMS, seed + 1)
+    return lat, U, g, psi
+
+
+class _Call:
+    """One operator call on fields of its own: run() it, its result, the oracle's."""
+
+    def __init__(self, q, lat, g, psi, kind, prec="f64", dagger=False):
+        self.q, self.g, self.psi, self.kind, self.dagger = q, g, psi, kind, dagger
+        p_in, p_out = {"half": ("odd", "even"), "mhat": ("even", "even")}.get(kind, ("full", "full"))
+        self.i, self.o = q.Spinor(lat, p_in, prec), q.Spinor(lat, p_out, prec)
+        self.i.upload({"half": lambda: syn.to_half(psi, 1), "mhat": lambda: syn.to_half(psi, 0)}.get(kind, lambda: psi)())
+
+    def run(self):
+        if self.kind in ("half", "full"):
+            self.q.apply_dslash(self.g, self.o, self.i, dagger=self.dagger)
+        else:
+            self.q.apply_M(self.g, self.o, self.i, KAPPA, MU, eo=self.kind == "mhat", dagger=self.dagger)
+
+    def error(self, U):
+        got, d = self.o.download(), self.dagger
+        if self.kind == "half":
+            want = oracle.dhop_eo(U, syn.to_half(self.psi, 1), 0, dagger=d)
+        elif self.kind == "full":
+            want = oracle.dhop(U, self.psi, dagger=d)
+        elif self.kind == "mhat":
+            want = oracle.apply_mhat(U, syn.to_half(self.psi, 0), KAPPA, MU, dagger=d)
+        else:
+            want = oracle.apply_m(U, self.psi, KAPPA, MU, dagger=d)
+        self.o.zero()
+        return F.rel_err(got, want)
+
+
+def _capture(q, run):
+    import torch
+    q.stream_sync()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        run()
+    return graph
+
+
+def _replay(graph):
+    import torch
+    graph.replay()
+    torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("kind", ["half", "mhat"])
+@pytest.mark.parametrize("larger", ["full", "m", "solve"])
+def test_replay_after_a_larger_call(q, threads, kind, larger):
+    """The workspaces that a captured launch holds are not replaced when a
+    call on more of the lattice needs its own."""
+    lat, U, g, psi = _setup(q)
+    call = _Call(q, lat, g, psi, kind)
+    call.run()
+    graph = _capture(q, call.run)
+    if larger == "solve":
+        b, x = q.Spinor(lat, "full", "f64"), q.Spinor(lat, "full", "f64")
+        b.upload(psi)
+        q.solve_cg(g, x, b, KAPPA, MU, eo=False)
+    else:
+        _Call(q, lat, g, psi, larger).run()
+    q.stream_sync()
+    call.o.zero()
+    _replay(graph)
+    assert call.error(U) < 1e-15
+
+
+@pytest.mark.parametrize("kind", ["half", "mhat", "full", "m"])
+def test_capture_after_a_call_of_another_form(q, kind):
+    """A call captured after one eager call needs no new workspace, whichever
+    kernel the earlier call took."""
+    lat, U, g, psi = _setup(q, seed=1711)
+    call = _Call(q, lat, g, psi, kind, dagger=True)
+    for first, then in ((8, 1), (1, 8)):
+        q.set_hop_threads(first)
+        call.run()
+        q.set_hop_threads(then)
+        try:
+            graph = _capture(q, call.run)
+        finally:
+            q.set_hop_threads(0)
+        call.o.zero()
+        _replay(graph)
+        assert call.error(U) < 1e-15
+
+
+def test_double_float_replay(q):
+    """A captured double-float operator holds no workspace that grows."""
+    lat, U, g, psi = _setup(q, seed=1721)
+    call = _Call(q, lat, g, psi, "half", prec="df64")
+    call.run()
+    graph = _capture(q, call.run)
+    _Call(q, lat, g, psi, "full", prec="df64").run()
+    q.stream_sync()
+    call.o.zero()
+    _replay(graph)
+    assert call.error(U) < 1e-13
