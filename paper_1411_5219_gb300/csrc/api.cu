@@ -1337,6 +1337,20 @@ qcd_status qcd_spinor_norm2(const qcd_spinor *s, double *result_device, void *st
                       "spinor_norm2");
 }
 
+// out = D in (dagger: D^dagger in) on output parity p, or on both.
+static HopArgs plain_hop(const FieldView &out, const FieldView &in, bool both, int p, int dagger)
+{
+    HopArgs h{};
+    h.out = &out;
+    h.in = &in;
+    h.out_parity = both ? 0 : p;
+    h.both = both;
+    h.dagger = dagger ? 1 : 0;
+    h.plain = true;
+    h.fin = FIN_STORE;
+    return h;
+}
+
 qcd_status qcd_apply_dslash(const qcd_gauge *g, qcd_spinor *out, const qcd_spinor *in, int dagger, void *stream)
 {
     if (!g || !out || !in) return fail(QCD_ERR_INVALID_ARG, "apply_dslash: NULL argument");
@@ -1353,16 +1367,7 @@ qcd_status qcd_apply_dslash(const qcd_gauge *g, qcd_spinor *out, const qcd_spino
     if (st != QCD_OK) return st;
     U = with_fix_input(g->lat, U, out->prec, g->recon, 0, both, s);
     const FieldView fo = view_of(out), fi = view_of(in);
-    HopArgs h{};
-    h.out = &fo;
-    h.in = &fi;
-    h.y = nullptr;
-    h.out_parity = both ? 0 : out->parity;
-    h.both = both;
-    h.dagger = dagger ? 1 : 0;
-    h.plain = true;
-    h.fin = FIN_STORE;
-    return check_cuda(hop(g->lat, U, g->recon, h, s), "apply_dslash");
+    return check_cuda(hop(g->lat, U, g->recon, plain_hop(fo, fi, both, out->parity, dagger), s), "apply_dslash");
 }
 
 qcd_status qcd_apply_dslash_multi(const qcd_gauge *g, qcd_spinor *const *out, const qcd_spinor *const *in, int nrhs,
@@ -1390,8 +1395,8 @@ qcd_status qcd_apply_dslash_multi(const qcd_gauge *g, qcd_spinor *const *out, co
     FieldView pv[kMaxRhs];
     for (int k = 0; k < nrhs; ++k) pv[k] = view_of(in[k]);
     // fields side by side: each is read and written in place (F64: through
-    // fixed-point copies of the inputs, whose workspace is not allocated under
-    // stream capture), unless an output overlaps another one's input
+    // fixed-point copies of the inputs), unless an output overlaps another
+    // one's input
     const size_t bytes = nh * spinor_half_bytes(prec, lat->stride), nbytes = nh * spinor_half_norm_bytes(prec, lat->stride);
     const size_t fd = nh * spinor_half_bytes(kPrecFix, lat->stride), fn = nh * spinor_half_norm_bytes(kPrecFix, lat->stride);
     auto overlap = [](const void *a, const void *b, size_t n) {
@@ -1402,11 +1407,16 @@ qcd_status qcd_apply_dslash_multi(const qcd_gauge *g, qcd_spinor *const *out, co
     for (int k = 0; k < nrhs; ++k)
         for (int j = 0; j < nrhs; ++j)
             apart = apart && !overlap(out[j]->data, in[k]->data, bytes) && !overlap(out[j]->norm, in[k]->norm, nbytes);
-    if (apart && prec == QCD_PREC_F64) {
-        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-        const auto it = lat->ws.find("dm_fix");
-        if (it == lat->ws.end() || it->second.second < nrhs * (fd + fn))
-            apart = cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone;
+    if (apart && prec == QCD_PREC_F64 && capturing(s)) {
+        // one launch per field: the copies' buffer grows with nrhs, so a
+        // caller's graph must not hold it, and it is not allocated here
+        U = with_fix_input(lat, U, prec, g->recon, 0, both, s);
+        cudaError_t e = cudaSuccess;
+        for (int k = 0; k < nrhs && e == cudaSuccess; ++k) {
+            const FieldView fo = view_of(out[k]);
+            e = hop(lat, U, g->recon, plain_hop(fo, pv[k], both, out[0]->parity, dagger), s);
+        }
+        return check_cuda(e, "apply_dslash_multi");
     }
     if (apart) {
         DslashMulti a;
@@ -1462,22 +1472,17 @@ qcd_status qcd_apply_dslash_multi(const qcd_gauge *g, qcd_spinor *const *out, co
     }
     int L = 0;
     while ((1 << L) < nrhs) ++L;
-    U = with_fix_input(lat, U, prec, g->recon, L, both, s);
-    const bool fix = fixed_hops(lat, U, prec, g->recon, L, both, s);
-    const FieldView bi = ws_field(lat, "dm_in", nh, fix ? kPrecFix : prec, L), bo = ws_field(lat, "dm_out", nh, prec, L);
+    // (buffers of their own for one half and for two, and of one size for either
+    // form of an F64 input: a caller's graph keeps their addresses)
+    const std::string halves = std::to_string(nh);
+    FieldView bi = ws_field(lat, "dm_in" + halves, nh, prec == QCD_PREC_F64 ? kPrecFix : prec, L);
+    const FieldView bo = ws_field(lat, "dm_out" + halves, nh, prec, L);
     if (!bi.hv[0].data || !bo.hv[0].data) return fail(QCD_ERR_OOM, "apply_dslash_multi: workspace");
+    if (!fixed_hops(lat, U, prec, g->recon, L, both, s)) bi.prec = prec;
     cudaError_t e = launch_zero(bi, s);
     if (e == cudaSuccess) e = launch_batch_copy(bi, pv, nrhs, 1, s);
     if (e != cudaSuccess) return check_cuda(e, "apply_dslash_multi: gather");
-    HopArgs h{};
-    h.out = &bo;
-    h.in = &bi;
-    h.out_parity = both ? 0 : out[0]->parity;
-    h.both = both;
-    h.dagger = dagger ? 1 : 0;
-    h.plain = true;
-    h.fin = FIN_STORE;
-    e = hop(lat, U, g->recon, h, s);
+    e = hop(lat, U, g->recon, plain_hop(bo, bi, both, out[0]->parity, dagger), s);
     for (int k = 0; k < nrhs; ++k) pv[k] = view_of(out[k]);
     if (e == cudaSuccess) e = launch_batch_copy(bo, pv, nrhs, 0, s);
     return check_cuda(e, "apply_dslash_multi");

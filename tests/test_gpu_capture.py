@@ -140,3 +140,45 @@ def test_double_float_replay(q):
     call.o.zero()
     _replay(graph)
     assert call.error(U) < 1e-13
+
+
+@pytest.mark.parametrize("prec", ["f64", "df64"])
+@pytest.mark.parametrize("overlapping", [False, True])
+def test_multi_capture_with_more_fields(q, threads, prec, overlapping):
+    """apply_dslash_multi of eight fields captured after a call with five (or,
+    gathered because an output is another one's input, with eight), replayed
+    after one with sixteen and one on both halves."""
+    lat, U, g, psi = _setup(q, seed=1731)
+    fields = [syn.to_half(syn.gaussian_spinor(DIMS, 1740 + k), 1) for k in range(8)]
+    full = [q.Spinor(lat, "full", prec) for _ in range(9)]
+    ins, outs = ([q.Spinor(lat, p, prec) for _ in range(16)] for p in ("odd", "even"))
+    for s, v in zip(ins, fields):
+        s.upload(v)
+    gathered = overlapping or prec == "df64"
+
+    def call(n=8):
+        if overlapping:  # both halves of field k + 1 from field k
+            q.apply_dslash_multi(g, full[1:n + 1], full[:n])
+        else:
+            q.apply_dslash_multi(g, outs[:n], ins[:n])
+
+    def fill():
+        for k in range(8):
+            full[k].upload(syn.gaussian_spinor(DIMS, 1740 + k))
+
+    fill()
+    call(8 if gathered else 5)
+    graph = _capture(q, call)
+    fill()
+    q.apply_dslash_multi(g, outs, ins)
+    q.apply_dslash_multi(g, [q.Spinor(lat, "full", prec) for _ in range(8)], full[:8])
+    for o in outs:
+        o.zero()
+    q.stream_sync()
+    _replay(graph)
+    tol = 1e-15 if prec == "f64" else 1e-13
+    for k in range(8):
+        if overlapping:
+            assert F.rel_err(full[k + 1].download(), oracle.dhop(U, syn.gaussian_spinor(DIMS, 1740 + k))) < tol, k
+        else:
+            assert F.rel_err(outs[k].download(), oracle.dhop_eo(U, fields[k], 0)) < tol, k
