@@ -394,42 +394,82 @@ GaugeView gauge_view(const qcd_gauge *g, int prec, int recon, cudaStream_t s, qc
     return dst;
 }
 
-GaugeView hop_links(const qcd_gauge *g, int prec, int recon, cudaStream_t s, qcd_status *st)
+static bool capturing(cudaStream_t s)
 {
-    GaugeView v = gauge_view(g, prec, recon, s, st);
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone) return false;
+    cudaGetLastError();
+    return true;
+}
+
+static void fix_free(qcd_gauge::FixLinks &f)
+{
+    cudaFree(f.links);
+    if (f.unfit_host) cudaFreeHost(f.unfit_host);
+    if (f.known) cudaEventDestroy(f.known);
+    f = qcd_gauge::FixLinks{};
+}
+
+static bool fix_alloc(qcd_gauge *g)
+{
+    const size_t bytes = gauge_bytes(QCD_PREC_F64, 18, g->lat->stride);
+    qcd_gauge::FixLinks f;
+    if (cudaMalloc(&f.links, bytes + 256) == cudaSuccess && cudaMallocHost(&f.unfit_host, sizeof(unsigned)) == cudaSuccess &&
+        cudaEventCreateWithFlags(&f.known, cudaEventDisableTiming) == cudaSuccess) {
+        f.unfit = reinterpret_cast<unsigned *>(reinterpret_cast<char *>(f.links) + bytes);
+        g->fix = f;
+        return true;
+    }
+    cudaGetLastError();
+    fix_free(f);
+    return false;
+}
+
+// Queue the fixed-point copy of the field's links after what wrote them on `s`
+// (captured: as part of the caller's graph).
+static cudaError_t fix_refresh(qcd_gauge *g, cudaStream_t s, bool captured)
+{
+    cudaError_t e = gauge_to_fix(g->fix.links, g->fix.unfit, GaugeView{g->data, g->lat->stride}, g->recon, g->lat->geom, s);
+    if (e != cudaSuccess || captured) return e;
+    e = cudaMemcpyAsync(g->fix.unfit_host, g->fix.unfit, sizeof(unsigned), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaEventRecord(g->fix.known, s);
+    if (e == cudaSuccess && g->fix_state != qcd_gauge::FIX_OFF) g->fix_state = qcd_gauge::FIX_PENDING;
+    return e;
+}
+
+HopLinks hop_links(const qcd_gauge *g, int prec, int recon, cudaStream_t s, bool settle, qcd_status *st)
+{
+    HopLinks u{{gauge_view(g, prec, recon, s, st)}, 1};
     const bool df = prec == QCD_PREC_DF64 && recon == 18;
-    if (*st != QCD_OK || (prec != QCD_PREC_F64 && !df) || g->prec != QCD_PREC_F64 || g->recon != recon) return v;
+    if (*st != QCD_OK || (prec != QCD_PREC_F64 && !df) || g->prec != QCD_PREC_F64 || g->recon != recon) return u;
     auto *gm = const_cast<qcd_gauge *>(g);
     std::lock_guard<std::mutex> lk(derived_mu);
-    if (g->fix_state == qcd_gauge::FIX_STALE) {
-        // as for a derived copy: complete before any stream may read it
-        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
-            cudaGetLastError();
-            return v;
-        }
-        DeviceLock dl(device_mutex());
-        if (!gm->fix && cudaMalloc(&gm->fix, gauge_bytes(QCD_PREC_F64, 18, g->lat->stride)) != cudaSuccess) {
-            cudaGetLastError();
-            gm->fix = nullptr;
-            gm->fix_state = qcd_gauge::FIX_UNFIT;  // not asked for again before the next upload
-            return v;
-        }
-        bool fits = false;
-        const cudaError_t e = gauge_to_fix(static_cast<int4 *>(gm->fix), GaugeView{g->data, g->lat->stride, nullptr}, recon,
-                                           g->lat->geom, s, &fits);
-        if (e != cudaSuccess) {
-            *st = check_cuda(e, "fixed-point links");
-            return v;
-        }
-        gm->fix_state = fits ? qcd_gauge::FIX_READY : qcd_gauge::FIX_UNFIT;
-        if (!fits) {
-            cudaFree(gm->fix);
-            gm->fix = nullptr;
-        }
+    if (capturing(s)) {
+        // whether the links fit is for the device to see when the graph runs
+        if (settle || df || (g->fix_state != qcd_gauge::FIX_PENDING && g->fix_state != qcd_gauge::FIX_READY)) return u;
+        u.form[0].unfit = g->fix.unfit;
+        u.form[1] = u.form[0];
+        u.form[0].fix = g->fix.links;
+        u.n = 2;
+        return u;
     }
-    if (g->fix_state == qcd_gauge::FIX_READY) v.fix = static_cast<const int4 *>(g->fix);
-    return v;
+    cudaError_t e = cudaSuccess;
+    if (g->fix_state == qcd_gauge::FIX_NONE) {
+        DeviceLock dl(device_mutex());
+        if (!g->fix.links && !fix_alloc(gm)) {
+            gm->fix_state = qcd_gauge::FIX_UNFIT;  // not asked for again before the next upload
+            return u;
+        }
+        e = fix_refresh(gm, s, false);
+    }
+    if (e == cudaSuccess && g->fix_state == qcd_gauge::FIX_PENDING) {
+        // as for a derived copy: complete before any stream may read it
+        e = cudaEventSynchronize(g->fix.known);
+        if (e == cudaSuccess) gm->fix_state = *g->fix.unfit_host ? qcd_gauge::FIX_UNFIT : qcd_gauge::FIX_READY;
+    }
+    if (e != cudaSuccess) *st = check_cuda(e, "fixed-point links");
+    if (g->fix_state == qcd_gauge::FIX_READY) u.form[0].fix = g->fix.links;
+    return u;
 }
 
 // ----------------------------------------------------------------- hop
@@ -605,9 +645,8 @@ int tuned_tpb(const qcd_lattice *lat, const GaugeView &U, int prec, int recon, i
         auto it = g_tune.find(key);
         if (it != g_tune.end()) return it->second;
     }
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     const int fallback = lanes8_ok ? 64 : 128;
-    if (cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return fallback;
+    if (capturing(s)) return fallback;
     const FieldView ti = ws_field(lat, "tune_in", both ? 2 : 1, prec, L);
     const FieldView to = ws_field(lat, "tune_out", both ? 2 : 1, prec, L);
     if (!ti.hv[0].data || !to.hv[0].data || launch_zero(ti, s) != cudaSuccess) return fallback;
@@ -684,14 +723,6 @@ static cudaError_t profiled(int prec, int recon, double sites, int n, int fields
     return e;
 }
 
-static bool capturing(cudaStream_t s)
-{
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone) return false;
-    cudaGetLastError();
-    return true;
-}
-
 // The lattice's workspace for the input of a fixed-point hop of nh halves.  It
 // always holds both: a caller's graph keeps the address of a launch that it
 // captured, so the buffer must not be replaced when a later call needs more.
@@ -703,12 +734,13 @@ static FieldView fix_input_ws(const qcd_lattice *lat, int nh, int rhs_log2)
     return f;
 }
 
-GaugeView with_fix_input(const qcd_lattice *lat, GaugeView U, int prec, int recon, int rhs_log2, bool both, cudaStream_t s)
+HopLinks with_fix_input(const qcd_lattice *lat, const HopLinks &U, int prec, int recon, int rhs_log2, bool both,
+                        cudaStream_t s)
 {
-    if (!fixed_hops(lat, U, prec, recon, rhs_log2, both, s)) return U;
+    if (!fixed_hops(lat, U.form[0], prec, recon, rhs_log2, both, s)) return U;
     const bool have = lat->ws.find(ws_name("hop_in", kPrecFix, rhs_log2)) != lat->ws.end();
-    if (!have && (capturing(s) || !fix_input_ws(lat, 1, rhs_log2).hv[0].data)) U.fix = nullptr;
-    return U;
+    if (have || (!capturing(s) && fix_input_ws(lat, 1, rhs_log2).hv[0].data)) return U;
+    return HopLinks{{GaugeView{U.form[0].data, U.form[0].stride}}, 1};
 }
 
 // A double-float hop through the fixed-point FP64 kernel: its input and y in
@@ -1070,7 +1102,15 @@ qcd_status qcd_gauge_upload(qcd_gauge *g, const double *host, void *stream)
     if (!g || !host) return fail(QCD_ERR_INVALID_ARG, "gauge_upload: NULL argument");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const size_t bytes = (size_t)g->lat->h * 2 * 4 * 9 * 16;
-    g->fix_state = qcd_gauge::FIX_STALE;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    const bool captured = cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusActive;
+    {
+        std::lock_guard<std::mutex> lk(derived_mu);
+        if (captured)
+            g->fix_state = qcd_gauge::FIX_OFF;
+        else if (g->fix_state != qcd_gauge::FIX_OFF)
+            g->fix_state = qcd_gauge::FIX_NONE;
+    }
     if (!g->derived.empty()) {
         cudaStreamSynchronize(s);
         DeviceLock dl(device_mutex());
@@ -1083,6 +1123,10 @@ qcd_status qcd_gauge_upload(qcd_gauge *g, const double *host, void *stream)
     const GaugeView dst{g->data, g->lat->stride, nullptr};
     if (e == cudaSuccess)
         e = launch_gauge_pack(dst, g->prec, g->recon, static_cast<const double2 *>(stage), g->lat->geom, s);
+    if (e == cudaSuccess && g->fix.links) {
+        std::lock_guard<std::mutex> lk(derived_mu);
+        e = fix_refresh(g, s, captured);
+    }
     qcd_status st = QCD_OK;
     if (e == cudaSuccess && g->recon == 8)
         st = check_recon8(dst, g->prec, static_cast<const double2 *>(stage), dst, g->prec, g->recon, g->lat->geom, s,
@@ -1098,7 +1142,7 @@ qcd_status qcd_gauge_prepare(qcd_gauge *g, qcd_prec prec, qcd_recon recon, void 
     if (!g) return fail(QCD_ERR_INVALID_ARG, "gauge_prepare: NULL argument");
     if (!valid_prec(prec) || !valid_recon(recon)) return fail(QCD_ERR_INVALID_ARG, "gauge_prepare: bad prec/recon");
     qcd_status st;
-    hop_links(g, prec, recon, static_cast<cudaStream_t>(stream), &st);
+    hop_links(g, prec, recon, static_cast<cudaStream_t>(stream), true, &st);
     return st;
 }
 
@@ -1110,7 +1154,7 @@ void qcd_gauge_destroy(qcd_gauge *g)
         DeviceLock dl(device_mutex());
         cudaDeviceSynchronize();
         drop_derived(g);
-        cudaFree(g->fix);
+        fix_free(g->fix);
         cudaFree(g->data);
         delete g;
     }
@@ -1363,11 +1407,14 @@ qcd_status qcd_apply_dslash(const qcd_gauge *g, qcd_spinor *out, const qcd_spino
         return fail(QCD_ERR_INVALID_ARG, "apply_dslash: parities must be (EVEN, ODD), (ODD, EVEN) or (FULL, FULL)");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     qcd_status st;
-    GaugeView U = hop_links(g, out->prec, g->recon, s, &st);
+    HopLinks U = hop_links(g, out->prec, g->recon, s, false, &st);
     if (st != QCD_OK) return st;
     U = with_fix_input(g->lat, U, out->prec, g->recon, 0, both, s);
     const FieldView fo = view_of(out), fi = view_of(in);
-    return check_cuda(hop(g->lat, U, g->recon, plain_hop(fo, fi, both, out->parity, dagger), s), "apply_dslash");
+    cudaError_t e = cudaSuccess;
+    for (int f = 0; f < U.n && e == cudaSuccess; ++f)
+        e = hop(g->lat, U.form[f], g->recon, plain_hop(fo, fi, both, out->parity, dagger), s);
+    return check_cuda(e, "apply_dslash");
 }
 
 qcd_status qcd_apply_dslash_multi(const qcd_gauge *g, qcd_spinor *const *out, const qcd_spinor *const *in, int nrhs,
@@ -1389,7 +1436,7 @@ qcd_status qcd_apply_dslash_multi(const qcd_gauge *g, qcd_spinor *const *out, co
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const qcd_lattice *lat = g->lat;
     qcd_status st;
-    GaugeView U = hop_links(g, in[0]->prec, g->recon, s, &st);
+    HopLinks U = hop_links(g, in[0]->prec, g->recon, s, false, &st);
     if (st != QCD_OK) return st;
     const int nh = both ? 2 : 1, prec = in[0]->prec;
     FieldView pv[kMaxRhs];
@@ -1403,7 +1450,7 @@ qcd_status qcd_apply_dslash_multi(const qcd_gauge *g, qcd_spinor *const *out, co
         const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
         return x < y + n && y < x + n;
     };
-    bool apart = prec != QCD_PREC_DF64 && (prec != QCD_PREC_F64 || U.fix);
+    bool apart = prec != QCD_PREC_DF64 && (prec != QCD_PREC_F64 || U.form[0].fix);
     for (int k = 0; k < nrhs; ++k)
         for (int j = 0; j < nrhs; ++j)
             apart = apart && !overlap(out[j]->data, in[k]->data, bytes) && !overlap(out[j]->norm, in[k]->norm, nbytes);
@@ -1414,7 +1461,8 @@ qcd_status qcd_apply_dslash_multi(const qcd_gauge *g, qcd_spinor *const *out, co
         cudaError_t e = cudaSuccess;
         for (int k = 0; k < nrhs && e == cudaSuccess; ++k) {
             const FieldView fo = view_of(out[k]);
-            e = hop(lat, U, g->recon, plain_hop(fo, pv[k], both, out[0]->parity, dagger), s);
+            for (int f = 0; f < U.n && e == cudaSuccess; ++f)
+                e = hop(lat, U.form[f], g->recon, plain_hop(fo, pv[k], both, out[0]->parity, dagger), s);
         }
         return check_cuda(e, "apply_dslash_multi");
     }
@@ -1425,7 +1473,7 @@ qcd_status qcd_apply_dslash_multi(const qcd_gauge *g, qcd_spinor *const *out, co
         a.out_parity = both ? 0 : out[0]->parity;
         a.both = both ? 1 : 0;
         a.dagger = dagger ? 1 : 0;
-        a.U = U;
+        a.U = U.form[0];
         a.n = nrhs;
         // four fields to a warp, or the next smaller group that leaves fewer lanes idle
         a.group_log2 = nrhs % 4 == 0 || nrhs > 8 ? 2 : nrhs % 2 == 0 || nrhs > 4 ? 1 : 0;
@@ -1478,11 +1526,13 @@ qcd_status qcd_apply_dslash_multi(const qcd_gauge *g, qcd_spinor *const *out, co
     FieldView bi = ws_field(lat, "dm_in" + halves, nh, prec == QCD_PREC_F64 ? kPrecFix : prec, L);
     const FieldView bo = ws_field(lat, "dm_out" + halves, nh, prec, L);
     if (!bi.hv[0].data || !bo.hv[0].data) return fail(QCD_ERR_OOM, "apply_dslash_multi: workspace");
-    if (!fixed_hops(lat, U, prec, g->recon, L, both, s)) bi.prec = prec;
-    cudaError_t e = launch_zero(bi, s);
-    if (e == cudaSuccess) e = launch_batch_copy(bi, pv, nrhs, 1, s);
-    if (e != cudaSuccess) return check_cuda(e, "apply_dslash_multi: gather");
-    e = hop(lat, U, g->recon, plain_hop(bo, bi, both, out[0]->parity, dagger), s);
+    cudaError_t e = cudaSuccess;
+    for (int f = 0; f < U.n && e == cudaSuccess; ++f) {
+        bi.prec = fixed_hops(lat, U.form[f], prec, g->recon, L, both, s) ? kPrecFix : prec;
+        e = launch_zero(bi, s);
+        if (e == cudaSuccess) e = launch_batch_copy(bi, pv, nrhs, 1, s);
+        if (e == cudaSuccess) e = hop(lat, U.form[f], g->recon, plain_hop(bo, bi, both, out[0]->parity, dagger), s);
+    }
     for (int k = 0; k < nrhs; ++k) pv[k] = view_of(out[k]);
     if (e == cudaSuccess) e = launch_batch_copy(bo, pv, nrhs, 0, s);
     return check_cuda(e, "apply_dslash_multi");
@@ -1502,7 +1552,7 @@ qcd_status qcd_apply_M(const qcd_gauge *g, qcd_spinor *out, const qcd_spinor *in
         return fail(QCD_ERR_INVALID_ARG, "apply_M: eo = 0 needs FULL fields");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     qcd_status st;
-    GaugeView U = hop_links(g, out->prec, g->recon, s, &st);
+    HopLinks U = hop_links(g, out->prec, g->recon, s, false, &st);
     if (st != QCD_OK) return st;
     U = with_fix_input(g->lat, U, out->prec, g->recon, 0, !eo, s);
     const double a = 2.0 * kappa * mu, b = dagger ? -a : a;
@@ -1511,30 +1561,26 @@ qcd_status qcd_apply_M(const qcd_gauge *g, qcd_spinor *out, const qcd_spinor *in
     HopArgs h{};
     h.dagger = dagger ? 1 : 0;
     h.fin = FIN_STORE;
+    h.in = &fi;
+    h.twisted = tw;
+    cudaError_t e = cudaSuccess;
     if (!eo) {
         h.out = &fo;
-        h.in = &fi;
         h.y = &fi;
         h.both = true;
         h.cy = coef_twist(b);
         h.cd = coef_real(-kappa);
-        h.twisted = tw;
-        return check_cuda(hop(g->lat, U, g->recon, h, s), "apply_M");
+        for (int f = 0; f < U.n && e == cudaSuccess; ++f) e = hop(g->lat, U.form[f], g->recon, h, s);
+        return check_cuda(e, "apply_M");
     }
     // (one buffer for the temporary in either form, so that a captured call
     // finds the one that an earlier call made whatever kernel it takes)
     FieldView t = ws_field(g->lat, "applyM_t", 1, out->prec == QCD_PREC_F64 ? kPrecFix : out->prec);
     if (!t.hv[0].data) return fail(QCD_ERR_OOM, "apply_M: workspace");
-    if (!fixed_hops(g->lat, U, out->prec, g->recon, 0, false, s)) t.prec = out->prec;
     h.out = &t;
-    h.in = &fi;
-    h.y = nullptr;
     h.out_parity = 1;
     h.plain = !tw;
-    h.twisted = tw;
     h.cd = coef_twist_inv(b);
-    cudaError_t e = hop(g->lat, U, g->recon, h, s);
-    if (e != cudaSuccess) return check_cuda(e, "apply_M");
     HopArgs h2{};
     h2.dagger = h.dagger;
     h2.fin = FIN_STORE;
@@ -1545,7 +1591,12 @@ qcd_status qcd_apply_M(const qcd_gauge *g, qcd_spinor *out, const qcd_spinor *in
     h2.cy = coef_twist(b);
     h2.cd = coef_real(-kappa * kappa);
     h2.twisted = tw;
-    return check_cuda(hop(g->lat, U, g->recon, h2, s), "apply_M");
+    for (int f = 0; f < U.n && e == cudaSuccess; ++f) {
+        t.prec = fixed_hops(g->lat, U.form[f], out->prec, g->recon, 0, false, s) ? kPrecFix : out->prec;
+        e = hop(g->lat, U.form[f], g->recon, h, s);
+        if (e == cudaSuccess) e = hop(g->lat, U.form[f], g->recon, h2, s);
+    }
+    return check_cuda(e, "apply_M");
 }
 
 }  // extern "C"

@@ -32,6 +32,7 @@ __global__ void __launch_bounds__(kFixThreads, 4) dslash_fix_kernel(const __grid
 {
     constexpr bool kMulti = std::is_same<Launch, DslashMulti>::value;  // separate fields, consecutive blocks one each
     if (a.check_status && a.state->status != a.run_status) return;
+    if (a.U.unfit && *a.U.unfit) return;
     constexpr int SF_ = kDagger ? -1 : +1, SB_ = -SF_;  // projector signs of forward and backward hops
     const int ne = a.g.h << a.rhs_log2;
     int nbp = (ne + kFixElems - 1) / kFixElems, field = 0;
@@ -225,6 +226,7 @@ template <int kEpi, bool kReduce>
 __global__ void __launch_bounds__(128) dslash_fix16_kernel(const DslashLaunch a)
 {
     if (a.check_status && a.state->status != a.run_status) return;
+    if (a.U.unfit && *a.U.unfit) return;
     const int items = a.g.h * 16;
     const int nbp = (items + 127) / 128;
     const int p = a.both ? (int)(blockIdx.x >= (unsigned)nbp) : a.out_parity;

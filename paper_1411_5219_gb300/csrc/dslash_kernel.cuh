@@ -286,6 +286,8 @@ __global__ void __launch_bounds__(TPB, kMinBlocks) dslash_kernel(const __grid_co
     using R = typename SF::R;
     constexpr bool kMulti = std::is_same<Launch, DslashMulti>::value;
     if (a.check_status && a.state->status != a.run_status) return;
+    if constexpr (std::is_same<SF, SpF64>::value)
+        if (a.U.unfit && !*a.U.unfit) return;
     constexpr int SF_ = kDagger ? -1 : +1;  // projector sign of forward hops
     constexpr int SB_ = -SF_;                // ... of backward hops
     // element e = site i * 2^rhs_log2 + rhs (one rhs: e = i); with separate
@@ -544,6 +546,7 @@ template <int kDagger, int kEpi, bool kReduce>
 __global__ void __launch_bounds__(128) dslash_lanes8_kernel(const DslashLaunch a)
 {
     if (a.check_status && a.state->status != a.run_status) return;
+    if (a.U.unfit && !*a.U.unfit) return;
     const int items = a.g.h * 8;
     const int nbp = (items + 127) / 128;
     const int p = a.both ? (int)(blockIdx.x >= (unsigned)nbp) : a.out_parity;

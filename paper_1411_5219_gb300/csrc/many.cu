@@ -580,7 +580,7 @@ extern "C" qcd_status qcd_solve_cg_many(int n, const qcd_gauge *const *gauges, q
         const qcd_gauge *g = gauges[k];
         const qcd_lattice *lat = x[k]->lat;
         qcd_status st = QCD_OK;
-        GaugeView U = hop_links(g, QCD_PREC_F64, g->recon, s, &st);
+        GaugeView U = hop_links(g, QCD_PREC_F64, g->recon, s, true, &st).form[0];
         if (st != QCD_OK) return st;
         if (!U.fix && g->recon != 18) U = gauge_view(g, QCD_PREC_F64, 18, s, &st);  // (the FP64 phases read all nine entries)
         if (st != QCD_OK) return st;

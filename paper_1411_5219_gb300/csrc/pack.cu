@@ -288,29 +288,19 @@ cudaError_t launch_gauge_convert(const GaugeView &dst, int dprec, int drecon, co
     return cudaGetLastError();
 }
 
-cudaError_t gauge_to_fix(int4 *dst, const GaugeView &src, int srecon, const Geom &g, cudaStream_t s, bool *fits)
+cudaError_t gauge_to_fix(int4 *dst, unsigned *unfit, const GaugeView &src, int srecon, const Geom &g, cudaStream_t s)
 {
-    unsigned *d = nullptr, unfit = 1;
-    cudaError_t e = cudaMallocAsync(&d, sizeof(*d), s);
+    const cudaError_t e = cudaMemsetAsync(unfit, 0, sizeof(*unfit), s);
     if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(d, 0, sizeof(*d), s);
-    if (e == cudaSuccess) {
-        const dim3 grid((g.h + 127) / 128, 8);
-        if (srecon == 18)
-            gauge_fix_kernel<GF64<18>><<<grid, 128, 0, s>>>(dst, src, g.h, d);
-        else if (srecon == 12)
-            gauge_fix_kernel<GF64<12>><<<grid, 128, 0, s>>>(dst, src, g.h, d);
-        else
-            gauge_fix_kernel<GF64<8>><<<grid, 128, 0, s>>>(dst, src, g.h, d);
-        note_launches();
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&unfit, d, sizeof(unfit), cudaMemcpyDeviceToHost, s);
-    cudaError_t e2 = cudaFreeAsync(d, s);
-    if (e == cudaSuccess) e = e2;
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    *fits = unfit == 0;
-    return e;
+    const dim3 grid((g.h + 127) / 128, 8);
+    if (srecon == 18)
+        gauge_fix_kernel<GF64<18>><<<grid, 128, 0, s>>>(dst, src, g.h, unfit);
+    else if (srecon == 12)
+        gauge_fix_kernel<GF64<12>><<<grid, 128, 0, s>>>(dst, src, g.h, unfit);
+    else
+        gauge_fix_kernel<GF64<8>><<<grid, 128, 0, s>>>(dst, src, g.h, unfit);
+    note_launches();
+    return cudaGetLastError();
 }
 
 // Largest entry error of a reconstruct-8 field `dst` against its FP64

@@ -62,10 +62,20 @@ struct qcd_gauge {
     size_t bytes = 0;
     // Copies in other (prec, recon) formats, keyed by prec * 100 + recon.
     std::map<int, std::pair<void *, size_t>> derived;
-    // F64 links in fixed point (fixed.cuh) for the FP64 hopping kernels, made on first use: the buffer outlives an upload,
-    // which only marks its contents out of date.
-    void *fix = nullptr;
-    enum FixState { FIX_STALE, FIX_READY, FIX_UNFIT } fix_state = FIX_STALE;  // UNFIT: an entry above 1 or non-finite
+    // F64 links in fixed point (fixed.cuh) for the FP64 hopping kernels, made on
+    // first use.  The buffer lives as long as the field, since a caller's graph
+    // keeps its address, and every upload writes it again in stream order, so
+    // that a replay sees the links of the day.
+    struct FixLinks {
+        int4 *links = nullptr;
+        unsigned *unfit = nullptr;       // device: not zero when an entry is above 1 or not finite
+        unsigned *unfit_host = nullptr;  // pinned: its value, once `known` has been reached
+        cudaEvent_t known = nullptr;
+    } fix;
+    // NONE: not made, or out of date; PENDING: queued, whether it fits not looked
+    // at; UNFIT: the FP64 kernels run (also when there is no memory for it); OFF:
+    // an upload was captured, whose replays change the links unseen
+    enum FixState { FIX_NONE, FIX_PENDING, FIX_READY, FIX_UNFIT, FIX_OFF } fix_state = FIX_NONE;
 };
 
 struct qcd_spinor {
@@ -115,11 +125,19 @@ FieldView view_of(const qcd_spinor *s);
 FieldView view_half(const qcd_spinor *s, int half);  // half of a FULL field
 FieldView ws_field(const qcd_lattice *lat, const std::string &name, int nh, int prec, int rhs_log2 = 0);
 GaugeView gauge_view(const qcd_gauge *g, int prec, int recon, cudaStream_t s, qcd_status *st);
-// gauge_view for the Wilson hopping term: an F64 field's view carries
-// its fixed-point copy where there is one (built here on first use;
-// left out under stream capture, without memory for it and for links that
-// do not fit, which the FP64 kernels take).
-GaugeView hop_links(const qcd_gauge *g, int prec, int recon, cudaStream_t s, qcd_status *st);
+// The links of an operator call: its launches are queued once for each of the
+// forms 0 .. n-1, in this order.  One form as a rule; two under stream capture,
+// where the links may change before the graph runs: in fixed point and in
+// FP64, of which the device lets one run (GaugeView::unfit).
+struct HopLinks {
+    GaugeView form[2];
+    int n;
+};
+// gauge_view for the Wilson hopping term: an F64 field's view carries its
+// fixed-point copy where there is one (built here on first use; left out without
+// memory for it and for links that do not fit, which the FP64 kernels take).
+// settle: one form also under capture (FP64 then).
+HopLinks hop_links(const qcd_gauge *g, int prec, int recon, cudaStream_t s, bool settle, qcd_status *st);
 Reduction reduction_of(const qcd_lattice *lat);
 
 cudaError_t launch_dslash(int prec, int recon, const DslashLaunch &a, cudaStream_t s);
@@ -164,8 +182,8 @@ bool fixed_hops(const qcd_lattice *lat, const GaugeView &U, int prec, int recon,
 // fixed-point kernel would want a workspace for its input that is not to be
 // had (no memory, or a first use under stream capture), so that the FP64
 // kernels run.
-GaugeView with_fix_input(const qcd_lattice *lat, GaugeView U, int prec, int recon, int rhs_log2, bool both,
-                         cudaStream_t s);
+HopLinks with_fix_input(const qcd_lattice *lat, const HopLinks &U, int prec, int recon, int rhs_log2, bool both,
+                        cudaStream_t s);
 
 // The CG solve behind qcd_solve_cg / qcd_solve_cg_multi, with an optional
 // context lattice (scratch, state, graphs) other than the gauge field's.

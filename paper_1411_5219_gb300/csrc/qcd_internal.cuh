@@ -108,6 +108,10 @@ struct GaugeView {
     void *data;      // block (parity, mu) = parity*4 + mu, planes inside each block
     int stride;      // sites per plane (padded)
     const int4 *fix; // FP64 links in fixed point (fixed.cuh): nine int4 planes per block, or nullptr
+    // FP64 operators queued in both forms: a launch with `fix` runs only while
+    // this device word is zero (the links fit that form), one without only
+    // while it is not.  nullptr: no condition.
+    const unsigned *unfit;
 };
 
 // Spinor storage formats.  load() returns the full 4x3 spinor of site i in

@@ -101,9 +101,9 @@ cudaError_t launch_gauge_pack(const GaugeView &dst, int prec, int recon, const d
                               cudaStream_t s);
 cudaError_t launch_gauge_convert(const GaugeView &dst, int dprec, int drecon, const GaugeView &src, int sprec,
                                  int srecon, const Geom &g, cudaStream_t s);
-// The fixed-point copy (fixed.cuh) of F64 links, all nine entries; *fits is
-// false when an entry is above 1 or not finite.  Synchronises the stream.
-cudaError_t gauge_to_fix(int4 *dst, const GaugeView &src, int srecon, const Geom &g, cudaStream_t s, bool *fits);
+// The fixed-point copy (fixed.cuh) of F64 links, all nine entries; the device
+// word *unfit becomes 1 when an entry is above 1 or not finite, else 0.
+cudaError_t gauge_to_fix(int4 *dst, unsigned *unfit, const GaugeView &src, int srecon, const Geom &g, cudaStream_t s);
 cudaError_t gauge_recon8_error(const GaugeView &dst, int prec, const double2 *aos, const GaugeView &src, int sprec,
                                int srecon, const Geom &g, cudaStream_t s, double *max_err);
 // parity: 0/1 for a half field in parity-compacted host layout, 2 for a

@@ -539,8 +539,9 @@ qcd_status qcd::solve_impl(const qcd_gauge *g, qcd_spinor *const *x, const qcd_s
     // arithmetic costs more than the bytes it saves)
     const int srecon = !mixed ? g->recon : (sp == QCD_PREC_DF64 ? 18 : prm->inner_recon);
     qcd_status st;
-    GaugeView Uh = hop_links(g, QCD_PREC_F64, g->recon, s, &st);
+    HopLinks links = hop_links(g, QCD_PREC_F64, g->recon, s, true, &st);
     if (st != QCD_OK) return st;
+    GaugeView Uh = links.form[0];
     GaugeView Us = mixed ? gauge_view(g, sp, srecon, s, &st) : Uh;
     if (st != QCD_OK) return st;
 
@@ -604,7 +605,7 @@ qcd_status qcd::solve_impl(const qcd_gauge *g, qcd_spinor *const *x, const qcd_s
 
     // fixed-point FP64 hops keep the fields that only hops (and p, which the
     // vector updates) read in that form
-    Uh = with_fix_input(lat, Uh, QCD_PREC_F64, g->recon, L, !c.eo, s);
+    Uh = with_fix_input(lat, links, QCD_PREC_F64, g->recon, L, !c.eo, s).form[0];
     if (!mixed) Us = Uh;
     const bool fix = fixed_hops(lat, Uh, QCD_PREC_F64, g->recon, L, !c.eo, s);
     const int hp = fix ? kPrecFix : (int)QCD_PREC_F64;

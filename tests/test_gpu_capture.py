@@ -182,3 +182,66 @@ def test_multi_capture_with_more_fields(q, threads, prec, overlapping):
             assert F.rel_err(full[k + 1].download(), oracle.dhop(U, syn.gaussian_spinor(DIMS, 1740 + k))) < tol, k
         else:
             assert F.rel_err(outs[k].download(), oracle.dhop_eo(U, fields[k], 0)) < tol, k
+
+
+@pytest.mark.parametrize("kind", ["half", "full", "mhat", "m"])
+@pytest.mark.parametrize("first", [1.0, 4.0])
+def test_replay_after_uploads(q, threads, kind, first):
+    """A replay applies the links of the last upload, also where those have
+    entries above 1 (scaled by four), which the fixed-point form does not hold,
+    and whatever eager calls came between."""
+    lat, U, g, psi = _setup(q, seed=1751)
+    g.upload(first * U)
+    call = _Call(q, lat, g, psi, kind, dagger=True)
+    call.run()
+    graph = _capture(q, call.run)
+    for k, (scale, eager) in enumerate([(1.0, False), (4.0, False), (4.0, True), (1.0, True), (1.0, False)]):
+        V = scale * syn.gauge_field(DIMS, 0.3, 1760 + k)
+        g.upload(V)
+        if eager:
+            call.run()
+            assert call.error(V) < 1e-15, k
+        q.stream_sync()
+        _replay(graph)
+        assert call.error(V) < 1e-15, k
+
+
+def test_multi_replay_after_uploads(q, threads):
+    lat, U, g, psi = _setup(q, seed=1771)
+    fields = [syn.to_half(syn.gaussian_spinor(DIMS, 1780 + k), 1) for k in range(3)]
+    ins, outs = ([q.Spinor(lat, p, "f64") for _ in fields] for p in ("odd", "even"))
+    for s, v in zip(ins, fields):
+        s.upload(v)
+    q.apply_dslash(g, outs[0], ins[0])
+    graph = _capture(q, lambda: q.apply_dslash_multi(g, outs, ins))
+    for scale in (4.0, 1.0):
+        V = scale * syn.gauge_field(DIMS, 0.3, 1772)
+        g.upload(V)
+        q.stream_sync()
+        _replay(graph)
+        for o, v in zip(outs, fields):
+            assert F.rel_err(o.download(), oracle.dhop_eo(V, v, 0)) < 1e-15
+
+
+def test_captured_upload(q, threads):
+    """Replays of a captured upload change the links without a call of the
+    library: eager operators and captured ones apply the new ones."""
+    import torch
+    lat, U, g, psi = _setup(q, seed=1791)
+    call = _Call(q, lat, g, psi, "half")
+    call.run()
+    captured = _capture(q, call.run)
+    host = torch.from_numpy(U.copy()).pin_memory()
+    upload = _capture(q, lambda: g.upload(host))
+    b, x = q.Spinor(lat, "full", "f64"), q.Spinor(lat, "full", "f64")
+    b.upload(psi)
+    for k in range(2):
+        V = syn.gauge_field(DIMS, 0.3, 1792 + k)
+        host.copy_(torch.from_numpy(V))
+        _replay(upload)
+        call.run()
+        assert call.error(V) < 1e-15
+        _replay(captured)
+        assert call.error(V) < 1e-15
+        q.solve_cg(g, x, b, KAPPA, MU, tol=1e-11)
+        assert F.rel_err(oracle.apply_m(V, x.download(), KAPPA, MU), psi) < 1e-9
