@@ -444,15 +444,22 @@ HopLinks hop_links(const qcd_gauge *g, int prec, int recon, cudaStream_t s, bool
     if (*st != QCD_OK || (prec != QCD_PREC_F64 && !df) || g->prec != QCD_PREC_F64 || g->recon != recon) return u;
     auto *gm = const_cast<qcd_gauge *>(g);
     std::lock_guard<std::mutex> lk(derived_mu);
-    if (capturing(s)) {
-        // whether the links fit is for the device to see when the graph runs
-        if (settle || df || (g->fix_state != qcd_gauge::FIX_PENDING && g->fix_state != qcd_gauge::FIX_READY)) return u;
+    const bool captured = capturing(s);
+    settle = settle || df;
+    // whether the links fit is for the device to see: when the graph runs, or
+    // when the stream gets past an upload that the host need not wait for
+    bool both = g->fix_state == qcd_gauge::FIX_PENDING || (captured && g->fix_state == qcd_gauge::FIX_READY);
+    if (both && !settle && !captured) {
+        both = !profiling_active() && cudaEventQuery(g->fix.known) == cudaErrorNotReady;
+        cudaGetLastError();
+    }
+    if (both && !settle) {
         u.form[0].unfit = g->fix.unfit;
         u.form[1] = u.form[0];
         u.form[0].fix = g->fix.links;
         u.n = 2;
-        return u;
     }
+    if (captured || u.n == 2) return u;
     cudaError_t e = cudaSuccess;
     if (g->fix_state == qcd_gauge::FIX_NONE) {
         DeviceLock dl(device_mutex());
@@ -463,7 +470,7 @@ HopLinks hop_links(const qcd_gauge *g, int prec, int recon, cudaStream_t s, bool
         e = fix_refresh(gm, s, false);
     }
     if (e == cudaSuccess && g->fix_state == qcd_gauge::FIX_PENDING) {
-        // as for a derived copy: complete before any stream may read it
+        // a new copy, as a derived one, is complete before any stream may read it
         e = cudaEventSynchronize(g->fix.known);
         if (e == cudaSuccess) gm->fix_state = *g->fix.unfit_host ? qcd_gauge::FIX_UNFIT : qcd_gauge::FIX_READY;
     }
@@ -1454,18 +1461,20 @@ qcd_status qcd_apply_dslash_multi(const qcd_gauge *g, qcd_spinor *const *out, co
     for (int k = 0; k < nrhs; ++k)
         for (int j = 0; j < nrhs; ++j)
             apart = apart && !overlap(out[j]->data, in[k]->data, bytes) && !overlap(out[j]->norm, in[k]->norm, nbytes);
-    if (apart && prec == QCD_PREC_F64 && capturing(s)) {
-        // one launch per field: the copies' buffer grows with nrhs, so a
-        // caller's graph must not hold it, and it is not allocated here
-        U = with_fix_input(lat, U, prec, g->recon, 0, both, s);
+    // one launch per field and form from `first`
+    auto each_field = [&](const HopLinks &links, int first) {
         cudaError_t e = cudaSuccess;
-        for (int k = 0; k < nrhs && e == cudaSuccess; ++k) {
+        for (int k = 0; k < nrhs; ++k) {
             const FieldView fo = view_of(out[k]);
-            for (int f = 0; f < U.n && e == cudaSuccess; ++f)
-                e = hop(lat, U.form[f], g->recon, plain_hop(fo, pv[k], both, out[0]->parity, dagger), s);
+            for (int f = first; f < links.n && e == cudaSuccess; ++f)
+                e = hop(lat, links.form[f], g->recon, plain_hop(fo, pv[k], both, out[0]->parity, dagger), s);
         }
         return check_cuda(e, "apply_dslash_multi");
-    }
+    };
+    // (captured: the copies' buffer grows with nrhs, so a caller's graph must
+    // not hold it, and it is not allocated here)
+    if (apart && prec == QCD_PREC_F64 && capturing(s))
+        return each_field(with_fix_input(lat, U, prec, g->recon, 0, both, s), 0);
     if (apart) {
         DslashMulti a;
         memset(&a, 0, sizeof(a));
@@ -1516,7 +1525,7 @@ qcd_status qcd_apply_dslash_multi(const qcd_gauge *g, qcd_spinor *const *out, co
         if (e == cudaSuccess)
             e = profiled(prec, g->recon, lat->h * (both ? 2.0 : 1.0), nrhs, 2, s,
                          [&] { return launch_dslash_multi(prec, g->recon, a, s); });
-        return check_cuda(e, "apply_dslash_multi");
+        return e == cudaSuccess ? each_field(U, 1) : check_cuda(e, "apply_dslash_multi");
     }
     int L = 0;
     while ((1 << L) < nrhs) ++L;

@@ -127,8 +127,9 @@ FieldView ws_field(const qcd_lattice *lat, const std::string &name, int nh, int 
 GaugeView gauge_view(const qcd_gauge *g, int prec, int recon, cudaStream_t s, qcd_status *st);
 // The links of an operator call: its launches are queued once for each of the
 // forms 0 .. n-1, in this order.  One form as a rule; two under stream capture,
-// where the links may change before the graph runs: in fixed point and in
-// FP64, of which the device lets one run (GaugeView::unfit).
+// where the links may change before the graph runs, and while an upload is
+// still under way: in fixed point and in FP64, of which the device lets one run
+// (GaugeView::unfit).
 struct HopLinks {
     GaugeView form[2];
     int n;
@@ -136,7 +137,7 @@ struct HopLinks {
 // gauge_view for the Wilson hopping term: an F64 field's view carries its
 // fixed-point copy where there is one (built here on first use; left out without
 // memory for it and for links that do not fit, which the FP64 kernels take).
-// settle: one form also under capture (FP64 then).
+// settle: one form, waiting for an upload under way (under capture: FP64).
 HopLinks hop_links(const qcd_gauge *g, int prec, int recon, cudaStream_t s, bool settle, qcd_status *st);
 Reduction reduction_of(const qcd_lattice *lat);
 

@@ -245,3 +245,37 @@ def test_captured_upload(q, threads):
         assert call.error(V) < 1e-15
         q.solve_cg(g, x, b, KAPPA, MU, tol=1e-11)
         assert F.rel_err(oracle.apply_m(V, x.download(), KAPPA, MU), psi) < 1e-9
+
+
+@pytest.mark.parametrize("scale", [1.0, 4.0])
+def test_first_call_after_an_upload_does_not_wait(q, threads, scale):
+    """Operators queued behind an upload that the GPU has not reached return
+    at once, and apply the uploaded links, in either form."""
+    import time
+    import torch
+    lat, U, g, psi = _setup(q, seed=1801)
+    calls = [_Call(q, lat, g, psi, kind) for kind in ("half", "full", "mhat", "m")]
+    ins, outs = ([q.Spinor(lat, p, "f64") for _ in range(3)] for p in ("odd", "even"))
+    for s in ins:
+        s.upload(syn.to_half(psi, 1))
+
+    def multi():
+        q.apply_dslash_multi(g, outs, ins)
+
+    for run in [c.run for c in calls] + [multi]:
+        run()
+    V = scale * syn.gauge_field(DIMS, 0.3, 1802)
+    host = torch.from_numpy(V).pin_memory()
+    q.stream_sync()
+    torch.cuda._sleep(1_000_000_000)  # half a second at 2 GHz
+    t0 = time.perf_counter()
+    g.upload(host)
+    for run in [c.run for c in calls] + [multi]:
+        run()
+    waited = time.perf_counter() - t0
+    q.stream_sync()
+    assert waited < 0.5 * (time.perf_counter() - t0)
+    for c in calls:
+        assert c.error(V) < 1e-15
+    for o in outs:
+        assert F.rel_err(o.download(), oracle.dhop_eo(V, syn.to_half(psi, 1), 0)) < 1e-15
