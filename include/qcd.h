@@ -135,7 +135,8 @@ qcd_status qcd_gauge_create(const qcd_lattice *lat, qcd_prec prec, qcd_recon rec
  * reach, see qcd_recon); CUDA. */
 qcd_status qcd_gauge_upload(qcd_gauge *g, const double *host, void *stream);
 /* Build (if missing) the derived copy used by kernels of precision
- * `prec` with `recon` reals per link.  Optional: calls build it on first
+ * `prec` with `recon` reals per link (for F64 also the lattice's workspace
+ * that the operators convert their input into).  Optional: calls build it on first
  * use, outside stream capture (a new copy is complete, its stream
  * synchronised, before any stream may read it; a call on a capturing stream
  * that needs a missing copy fails with INVALID_ARG).  Errors: INVALID_ARG

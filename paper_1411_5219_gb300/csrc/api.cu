@@ -1148,8 +1148,12 @@ qcd_status qcd_gauge_prepare(qcd_gauge *g, qcd_prec prec, qcd_recon recon, void 
 {
     if (!g) return fail(QCD_ERR_INVALID_ARG, "gauge_prepare: NULL argument");
     if (!valid_prec(prec) || !valid_recon(recon)) return fail(QCD_ERR_INVALID_ARG, "gauge_prepare: bad prec/recon");
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
     qcd_status st;
-    hop_links(g, prec, recon, static_cast<cudaStream_t>(stream), true, &st);
+    const HopLinks U = hop_links(g, prec, recon, s, true, &st);
+    // (the input workspace of the fixed-point hops too, so that the first call
+    // does not pay its allocation; without memory for it they run in FP64)
+    if (st == QCD_OK) with_fix_input(g->lat, U, prec, recon, 0, true, s);
     return st;
 }
 

@@ -279,3 +279,21 @@ def test_first_call_after_an_upload_does_not_wait(q, threads, scale):
         assert c.error(V) < 1e-15
     for o in outs:
         assert F.rel_err(o.download(), oracle.dhop_eo(V, syn.to_half(psi, 1), 0)) < 1e-15
+
+
+def test_prepare_leaves_nothing_to_allocate(q):
+    """After qcd_gauge_prepare the first F64 operator calls allocate no device
+    memory: the free memory stays what it is."""
+    import torch
+    q.set_hop_threads(0)
+    dims = (16, 16, 16, 8)  # 6.4 MB of input workspace
+    lat = q.Lattice(dims, -1)
+    g = q.Gauge(lat, "f64", 18)
+    g.prepare("f64", 18)
+    i, o = q.Spinor(lat, "full", "f64"), q.Spinor(lat, "full", "f64")
+    q.stream_sync()
+    before = torch.cuda.mem_get_info()[0]
+    q.apply_dslash(g, o, i)
+    q.apply_M(g, o, i, KAPPA, MU)
+    q.stream_sync()
+    assert torch.cuda.mem_get_info()[0] == before
