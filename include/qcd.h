@@ -125,7 +125,9 @@ void qcd_lattice_destroy(qcd_lattice *lat);
  * precision `prec` and with `recon` reals per link.  The field also keeps
  * derived copies in other precisions, made on the device from this one on
  * first use by a Dslash of that precision (for F64 a fixed-point copy of 144
- * bytes per link).  The field is zero when the
+ * bytes per link; a call that finds no memory gives this copy and the lattice's
+ * workspaces of that form back, unless a caller's graph holds them, and runs in
+ * FP64 arithmetic until the next upload).  The field is zero when the
  * call returns (it waits for the legacy default stream).  Errors:
  * INVALID_ARG; OOM; CUDA. */
 qcd_status qcd_gauge_create(const qcd_lattice *lat, qcd_prec prec, qcd_recon recon, qcd_gauge **out);
@@ -471,9 +473,11 @@ qcd_status qcd_set_hop_threads(int threads_per_site);
 /* Host-side failure injection for tests of the error paths (no device
  * fault is involved): the next `count` calls of kind `what` fail with
  * QCD_ERR_OOM before touching the device.  QCD_INJECT_SPINOR_CREATE:
- * qcd_spinor_create.  count = 0 clears.  The paper has no counterpart (its
+ * qcd_spinor_create; QCD_INJECT_WORKSPACE: the allocation of a lattice's
+ * workspace, inside any call that needs a new one.  count = 0 clears.  The paper has no counterpart (its
  * Sec. 5 asks that every part of the code be testable on its own). */
 #define QCD_INJECT_SPINOR_CREATE 1
+#define QCD_INJECT_WORKSPACE 2
 qcd_status qcd_debug_inject(int what, int count);
 
 #ifdef __cplusplus

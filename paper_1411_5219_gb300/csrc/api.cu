@@ -30,7 +30,7 @@ void note_launches(int n) { g_launches.fetch_add((unsigned long long)n, std::mem
 
 // ---- host-side failure injection (qcd_debug_inject): the next `count`
 // calls of the chosen kind fail as if their allocation had failed
-static std::atomic<int> g_inject[2] = {};
+static std::atomic<int> g_inject[3] = {};
 
 static bool take_injected_failure(int what)
 {
@@ -230,19 +230,26 @@ static void pinned_put(void *state, void *coef)
 
 // ----------------------------------------------------------------- views
 
+// The solver's cached graphs: they hold the addresses of workspaces.
+static void drop_graphs(const qcd_lattice *lat)
+{
+    for (auto &kv : lat->graphs) {
+        cudaGraphExecDestroy(kv.second.exec);
+        cudaGraphDestroy(kv.second.graph);
+    }
+    lat->graphs.clear();
+}
+
 void *workspace(const qcd_lattice *lat, const std::string &name, size_t bytes)
 {
     auto it = lat->ws.find(name);
     if (it != lat->ws.end() && it->second.second >= bytes) return it->second.first;
+    if (take_injected_failure(QCD_INJECT_WORKSPACE)) return nullptr;
     if (lat->alloc_stream) {
         // stream-ordered: only this lattice's own stream is waited for
         if (it != lat->ws.end()) {
             cudaStreamSynchronize(lat->alloc_stream);
-            for (auto &kv : lat->graphs) {
-                cudaGraphExecDestroy(kv.second.exec);
-                cudaGraphDestroy(kv.second.graph);
-            }
-            lat->graphs.clear();
+            drop_graphs(lat);
             lat_free(lat, it->second.first);
             lat->ws.erase(it);
         }
@@ -258,11 +265,7 @@ void *workspace(const qcd_lattice *lat, const std::string &name, size_t bytes)
     if (it != lat->ws.end()) {
         // cached CG graphs may hold this buffer's address: drop them all
         cudaDeviceSynchronize();
-        for (auto &kv : lat->graphs) {
-            cudaGraphExecDestroy(kv.second.exec);
-            cudaGraphDestroy(kv.second.graph);
-        }
-        lat->graphs.clear();
+        drop_graphs(lat);
         cudaFree(it->second.first);
         lat->ws.erase(it);
     }
@@ -437,15 +440,15 @@ static cudaError_t fix_refresh(qcd_gauge *g, cudaStream_t s, bool captured)
     return e;
 }
 
-HopLinks hop_links(const qcd_gauge *g, int prec, int recon, cudaStream_t s, bool settle, qcd_status *st)
+HopLinks hop_links(const qcd_gauge *g, int prec, int recon, cudaStream_t s, LinkWait wait, qcd_status *st)
 {
     HopLinks u{{gauge_view(g, prec, recon, s, st)}, 1};
-    const bool df = prec == QCD_PREC_DF64 && recon == 18;
-    if (*st != QCD_OK || (prec != QCD_PREC_F64 && !df) || g->prec != QCD_PREC_F64 || g->recon != recon) return u;
+    const bool df = prec == QCD_PREC_DF64 && recon == 18, settle = wait == LINKS_SETTLE || df;
+    if (*st != QCD_OK || wait == LINKS_FP64 || (prec != QCD_PREC_F64 && !df) || g->prec != QCD_PREC_F64 || g->recon != recon) return u;
     auto *gm = const_cast<qcd_gauge *>(g);
     std::lock_guard<std::mutex> lk(derived_mu);
     const bool captured = capturing(s);
-    settle = settle || df;
+    u.use = g->fix_use;
     // whether the links fit is for the device to see: when the graph runs, or
     // when the stream gets past an upload that the host need not wait for
     bool both = g->fix_state == qcd_gauge::FIX_PENDING || (captured && g->fix_state == qcd_gauge::FIX_READY);
@@ -458,6 +461,7 @@ HopLinks hop_links(const qcd_gauge *g, int prec, int recon, cudaStream_t s, bool
         u.form[1] = u.form[0];
         u.form[0].fix = g->fix.links;
         u.n = 2;
+        gm->fix_captured = g->fix_captured || captured;
     }
     if (captured || u.n == 2) return u;
     cudaError_t e = cudaSuccess;
@@ -477,6 +481,39 @@ HopLinks hop_links(const qcd_gauge *g, int prec, int recon, cudaStream_t s, bool
     if (e != cudaSuccess) *st = check_cuda(e, "fixed-point links");
     if (g->fix_state == qcd_gauge::FIX_READY) u.form[0].fix = g->fix.links;
     return u;
+}
+
+bool give_back_fixed(const qcd_gauge *g, const qcd_lattice *lat, cudaStream_t s)
+{
+    if (capturing(s)) return false;
+    // (not the buffers that either form uses, which a caller's graph may hold)
+    const std::string fixed = "/p" + std::to_string(kPrecFix) + "/";
+    auto optional = [&](const std::string &name) {
+        const auto starts = [&](const char *t) { return name.rfind(t, 0) == 0; };
+        return name == "dm_fix" || starts("df_") ||
+               (name.find(fixed) != std::string::npos && (starts("cg_") || (starts("hop_in") && !lat->hop_in_captured)));
+    };
+    bool any = false;
+    std::lock_guard<std::mutex> lk(derived_mu);
+    DeviceLock dl(device_mutex());
+    cudaDeviceSynchronize();
+    for (auto it = lat->ws.begin(); it != lat->ws.end();) {
+        if (!optional(it->first)) {
+            ++it;
+            continue;
+        }
+        if (!any) drop_graphs(lat);
+        any = true;
+        lat_free(lat, it->second.first);
+        it = lat->ws.erase(it);
+    }
+    auto *gm = const_cast<qcd_gauge *>(g);
+    if (g->fix.links && !g->fix_captured && g->fix_use.use_count() == 1) {
+        fix_free(gm->fix);
+        if (g->fix_state != qcd_gauge::FIX_OFF) gm->fix_state = qcd_gauge::FIX_UNFIT;
+        any = true;
+    }
+    return any;
 }
 
 // ----------------------------------------------------------------- hop
@@ -746,6 +783,7 @@ HopLinks with_fix_input(const qcd_lattice *lat, const HopLinks &U, int prec, int
 {
     if (!fixed_hops(lat, U.form[0], prec, recon, rhs_log2, both, s)) return U;
     const bool have = lat->ws.find(ws_name("hop_in", kPrecFix, rhs_log2)) != lat->ws.end();
+    lat->hop_in_captured = lat->hop_in_captured || (have && capturing(s));
     if (have || (!capturing(s) && fix_input_ws(lat, 1, rhs_log2).hv[0].data)) return U;
     return HopLinks{{GaugeView{U.form[0].data, U.form[0].stride}}, 1};
 }
@@ -908,7 +946,7 @@ qcd_status qcd_set_hop_threads(int threads_per_site)
 
 qcd_status qcd_debug_inject(int what, int count)
 {
-    if (what != QCD_INJECT_SPINOR_CREATE || count < 0)
+    if ((what != QCD_INJECT_SPINOR_CREATE && what != QCD_INJECT_WORKSPACE) || count < 0)
         return fail(QCD_ERR_INVALID_ARG, "debug_inject: unknown kind %d or negative count", what);
     g_inject[what].store(count);
     return QCD_OK;
@@ -1027,10 +1065,7 @@ static void lattice_free(qcd_lattice *lat)
         // stream-ordered: wait for this lattice's own stream only (its graphs
         // and staging must be idle), then free in stream order
         cudaStreamSynchronize(lat->alloc_stream);
-        for (auto &kv : lat->graphs) {
-            cudaGraphExecDestroy(kv.second.exec);
-            cudaGraphDestroy(kv.second.graph);
-        }
+        drop_graphs(lat);
         for (void *p : {(void *)lat->red_partials, (void *)lat->red_counter, (void *)lat->red_out,
                         (void *)lat->red_out_big, (void *)lat->state})
             lat_free(lat, p);
@@ -1050,10 +1085,7 @@ static void lattice_free(qcd_lattice *lat)
     if (lat->state_host) cudaFreeHost(lat->state_host);
     if (lat->coef_host) cudaFreeHost(lat->coef_host);
     for (auto &kv : lat->ws) cudaFree(kv.second.first);
-    for (auto &kv : lat->graphs) {
-        cudaGraphExecDestroy(kv.second.exec);
-        cudaGraphDestroy(kv.second.graph);
-    }
+    drop_graphs(lat);
     if (lat->capture_stream) cudaStreamDestroy(lat->capture_stream);
     delete lat;
 }
@@ -1133,6 +1165,7 @@ qcd_status qcd_gauge_upload(qcd_gauge *g, const double *host, void *stream)
     if (e == cudaSuccess && g->fix.links) {
         std::lock_guard<std::mutex> lk(derived_mu);
         e = fix_refresh(g, s, captured);
+        g->fix_captured = g->fix_captured || captured;
     }
     qcd_status st = QCD_OK;
     if (e == cudaSuccess && g->recon == 8)
@@ -1149,12 +1182,14 @@ qcd_status qcd_gauge_prepare(qcd_gauge *g, qcd_prec prec, qcd_recon recon, void 
     if (!g) return fail(QCD_ERR_INVALID_ARG, "gauge_prepare: NULL argument");
     if (!valid_prec(prec) || !valid_recon(recon)) return fail(QCD_ERR_INVALID_ARG, "gauge_prepare: bad prec/recon");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    qcd_status st;
-    const HopLinks U = hop_links(g, prec, recon, s, true, &st);
-    // (the input workspace of the fixed-point hops too, so that the first call
-    // does not pay its allocation; without memory for it they run in FP64)
-    if (st == QCD_OK) with_fix_input(g->lat, U, prec, recon, 0, true, s);
-    return st;
+    return with_memory(g, g->lat, s, LINKS_SETTLE, [&](LinkWait wait) {
+        qcd_status st;
+        const HopLinks U = hop_links(g, prec, recon, s, wait, &st);
+        // (the input workspace of the fixed-point hops too, so that the first call
+        // does not pay its allocation; without memory for it they run in FP64)
+        if (st == QCD_OK) with_fix_input(g->lat, U, prec, recon, 0, true, s);
+        return st;
+    });
 }
 
 void qcd_gauge_destroy(qcd_gauge *g)
@@ -1417,16 +1452,21 @@ qcd_status qcd_apply_dslash(const qcd_gauge *g, qcd_spinor *out, const qcd_spino
     if (!both && !(out->parity != QCD_PARITY_FULL && in->parity == 1 - out->parity))
         return fail(QCD_ERR_INVALID_ARG, "apply_dslash: parities must be (EVEN, ODD), (ODD, EVEN) or (FULL, FULL)");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    qcd_status st;
-    HopLinks U = hop_links(g, out->prec, g->recon, s, false, &st);
-    if (st != QCD_OK) return st;
-    U = with_fix_input(g->lat, U, out->prec, g->recon, 0, both, s);
-    const FieldView fo = view_of(out), fi = view_of(in);
-    cudaError_t e = cudaSuccess;
-    for (int f = 0; f < U.n && e == cudaSuccess; ++f)
-        e = hop(g->lat, U.form[f], g->recon, plain_hop(fo, fi, both, out->parity, dagger), s);
-    return check_cuda(e, "apply_dslash");
+    return with_memory(g, g->lat, s, LINKS_QUEUE, [&](LinkWait wait) {
+        qcd_status st;
+        HopLinks U = hop_links(g, out->prec, g->recon, s, wait, &st);
+        if (st != QCD_OK) return st;
+        U = with_fix_input(g->lat, U, out->prec, g->recon, 0, both, s);
+        const FieldView fo = view_of(out), fi = view_of(in);
+        cudaError_t e = cudaSuccess;
+        for (int f = 0; f < U.n && e == cudaSuccess; ++f)
+            e = hop(g->lat, U.form[f], g->recon, plain_hop(fo, fi, both, out->parity, dagger), s);
+        return check_cuda(e, "apply_dslash");
+    });
 }
+
+static qcd_status dslash_multi(const qcd_gauge *g, qcd_spinor *const *out, const qcd_spinor *const *in, int nrhs, bool both,
+                               int dagger, LinkWait wait, cudaStream_t s);
 
 qcd_status qcd_apply_dslash_multi(const qcd_gauge *g, qcd_spinor *const *out, const qcd_spinor *const *in, int nrhs,
                                   int dagger, void *stream)
@@ -1445,9 +1485,16 @@ qcd_status qcd_apply_dslash_multi(const qcd_gauge *g, qcd_spinor *const *out, co
     if (!both && !(out[0]->parity != QCD_PARITY_FULL && in[0]->parity == 1 - out[0]->parity))
         return fail(QCD_ERR_INVALID_ARG, "apply_dslash_multi: parities must be (EVEN, ODD), (ODD, EVEN) or (FULL, FULL)");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    return with_memory(g, g->lat, s, LINKS_QUEUE,
+                       [&](LinkWait wait) { return dslash_multi(g, out, in, nrhs, both, dagger, wait, s); });
+}
+
+static qcd_status dslash_multi(const qcd_gauge *g, qcd_spinor *const *out, const qcd_spinor *const *in, int nrhs, bool both,
+                               int dagger, LinkWait wait, cudaStream_t s)
+{
     const qcd_lattice *lat = g->lat;
     qcd_status st;
-    HopLinks U = hop_links(g, in[0]->prec, g->recon, s, false, &st);
+    HopLinks U = hop_links(g, in[0]->prec, g->recon, s, wait, &st);
     if (st != QCD_OK) return st;
     const int nh = both ? 2 : 1, prec = in[0]->prec;
     FieldView pv[kMaxRhs];
@@ -1507,7 +1554,7 @@ qcd_status qcd_apply_dslash_multi(const qcd_gauge *g, qcd_spinor *const *out, co
         cudaError_t e = cudaSuccess;
         if (prec == QCD_PREC_F64) {
             char *ws = static_cast<char *>(workspace(lat, "dm_fix", nrhs * (fd + fn)));
-            if (!ws) return fail(QCD_ERR_OOM, "apply_dslash_multi: workspace");
+            if (!ws) return each_field(with_fix_input(lat, U, prec, g->recon, 0, both, s), 0);
             FieldView f;
             f.nh = nh;
             f.h = lat->h;
@@ -1551,6 +1598,9 @@ qcd_status qcd_apply_dslash_multi(const qcd_gauge *g, qcd_spinor *const *out, co
     return check_cuda(e, "apply_dslash_multi");
 }
 
+static qcd_status apply_m(const qcd_gauge *g, qcd_spinor *out, const qcd_spinor *in, double kappa, double mu, int eo,
+                          int dagger, LinkWait wait, cudaStream_t s);
+
 qcd_status qcd_apply_M(const qcd_gauge *g, qcd_spinor *out, const qcd_spinor *in, double kappa, double mu, int eo,
                        int dagger, void *stream)
 {
@@ -1564,8 +1614,15 @@ qcd_status qcd_apply_M(const qcd_gauge *g, qcd_spinor *out, const qcd_spinor *in
     if (!eo && (out->parity != QCD_PARITY_FULL || in->parity != QCD_PARITY_FULL))
         return fail(QCD_ERR_INVALID_ARG, "apply_M: eo = 0 needs FULL fields");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    return with_memory(g, g->lat, s, LINKS_QUEUE,
+                       [&](LinkWait wait) { return apply_m(g, out, in, kappa, mu, eo, dagger, wait, s); });
+}
+
+static qcd_status apply_m(const qcd_gauge *g, qcd_spinor *out, const qcd_spinor *in, double kappa, double mu, int eo,
+                          int dagger, LinkWait wait, cudaStream_t s)
+{
     qcd_status st;
-    HopLinks U = hop_links(g, out->prec, g->recon, s, false, &st);
+    HopLinks U = hop_links(g, out->prec, g->recon, s, wait, &st);
     if (st != QCD_OK) return st;
     U = with_fix_input(g->lat, U, out->prec, g->recon, 0, !eo, s);
     const double a = 2.0 * kappa * mu, b = dagger ? -a : a;

@@ -510,10 +510,9 @@ void put(PhaseCoef &pc, const Coef &cy, const Coef &cd)
 
 using namespace qcd;
 
-extern "C" qcd_status qcd_solve_cg_many(int n, const qcd_gauge *const *gauges, qcd_spinor *const *x,
-                                        const qcd_spinor *const *b, const qcd_solver_params *prm,
-                                        qcd_solver_stats *stats, long long wait_cycles, int max_blocks,
-                                        void *stream)
+static qcd_status solve_many(LinkWait wait, int n, const qcd_gauge *const *gauges, qcd_spinor *const *x,
+                             const qcd_spinor *const *b, const qcd_solver_params *prm, qcd_solver_stats *stats,
+                             long long wait_cycles, int max_blocks, void *stream)
 {
     const auto t0 = std::chrono::steady_clock::now();
     if (n < 1 || n > kManyMax) return fail(QCD_ERR_INVALID_ARG, "solve_cg_many: n = %d not in 1..%d", n, kManyMax);
@@ -576,11 +575,13 @@ extern "C" qcd_status qcd_solve_cg_many(int n, const qcd_gauge *const *gauges, q
     std::vector<int> block_sys;
     int nchunk = 0;  // reduction chunks per partial slot, all systems
     const qcd_lattice *lat0 = x[0]->lat;
+    std::vector<HopLinks> links(n);  // (held until the solve is done)
     for (int k = 0; k < n; ++k) {
         const qcd_gauge *g = gauges[k];
         const qcd_lattice *lat = x[k]->lat;
         qcd_status st = QCD_OK;
-        GaugeView U = hop_links(g, QCD_PREC_F64, g->recon, s, true, &st).form[0];
+        links[k] = hop_links(g, QCD_PREC_F64, g->recon, s, wait, &st);
+        GaugeView U = links[k].form[0];
         if (st != QCD_OK) return st;
         if (!U.fix && g->recon != 18) U = gauge_view(g, QCD_PREC_F64, 18, s, &st);  // (the FP64 phases read all nine entries)
         if (st != QCD_OK) return st;
@@ -670,4 +671,16 @@ extern "C" qcd_status qcd_solve_cg_many(int n, const qcd_gauge *const *gauges, q
         }
     }
     return result;
+}
+
+extern "C" qcd_status qcd_solve_cg_many(int n, const qcd_gauge *const *gauges, qcd_spinor *const *x,
+                                        const qcd_spinor *const *b, const qcd_solver_params *prm,
+                                        qcd_solver_stats *stats, long long wait_cycles, int max_blocks,
+                                        void *stream)
+{
+    const qcd_status st = solve_many(LINKS_SETTLE, n, gauges, x, b, prm, stats, wait_cycles, max_blocks, stream);
+    if (st != QCD_ERR_OOM) return st;
+    bool any = false;  // (as with_memory, for every system's field)
+    for (int k = 0; k < n; ++k) any = give_back_fixed(gauges[k], x[k]->lat, static_cast<cudaStream_t>(stream)) || any;
+    return any ? solve_many(LINKS_FP64, n, gauges, x, b, prm, stats, wait_cycles, max_blocks, stream) : st;
 }

@@ -3,6 +3,7 @@
 
 #include <atomic>
 #include <map>
+#include <memory>
 #include <mutex>
 #include <shared_mutex>
 #include <string>
@@ -31,6 +32,7 @@ struct qcd_lattice {
     double *coef_host = nullptr;         // pinned staging of a solve's coefficient table (kCoefHostDoubles)
     // Named workspace buffers (staging, solver fields), grown on demand.
     mutable std::map<std::string, std::pair<void *, size_t>> ws;
+    mutable bool hop_in_captured = false;  // a caller's graph holds the fixed-point hops' input workspace
     // Instantiated CG-loop graphs keyed by solver configuration and field
     // addresses, and the stream used only to capture them.
     struct GraphEntry {
@@ -76,6 +78,8 @@ struct qcd_gauge {
     // at; UNFIT: the FP64 kernels run (also when there is no memory for it); OFF:
     // an upload was captured, whose replays change the links unseen
     enum FixState { FIX_NONE, FIX_PENDING, FIX_READY, FIX_UNFIT, FIX_OFF } fix_state = FIX_NONE;
+    bool fix_captured = false;  // a caller's graph holds the copy's address
+    std::shared_ptr<const int> fix_use = std::make_shared<const int>(0);  // shared by the calls that are using the copy
 };
 
 struct qcd_spinor {
@@ -133,12 +137,29 @@ GaugeView gauge_view(const qcd_gauge *g, int prec, int recon, cudaStream_t s, qc
 struct HopLinks {
     GaugeView form[2];
     int n;
+    std::shared_ptr<const int> use;  // keeps the fixed-point copy from being given back
+};
+enum LinkWait {
+    LINKS_QUEUE,   // for launches behind whatever writes the links
+    LINKS_SETTLE,  // one form, waiting for an upload under way (under capture: FP64)
+    LINKS_FP64     // without the fixed-point copy
 };
 // gauge_view for the Wilson hopping term: an F64 field's view carries its
 // fixed-point copy where there is one (built here on first use; left out without
 // memory for it and for links that do not fit, which the FP64 kernels take).
-// settle: one form, waiting for an upload under way (under capture: FP64).
-HopLinks hop_links(const qcd_gauge *g, int prec, int recon, cudaStream_t s, bool settle, qcd_status *st);
+HopLinks hop_links(const qcd_gauge *g, int prec, int recon, cudaStream_t s, LinkWait wait, qcd_status *st);
+// Frees what the fixed-point form holds: the field's copy, unless a caller's graph
+// or another thread's call is using it, and the lattice's workspaces of that
+// form.  False when there was nothing to free.
+bool give_back_fixed(const qcd_gauge *g, const qcd_lattice *lat, cudaStream_t s);
+// op(wait); where that finds no memory, op(LINKS_FP64) with what the fixed-point
+// form took.
+template <typename Op>
+qcd_status with_memory(const qcd_gauge *g, const qcd_lattice *lat, cudaStream_t s, LinkWait wait, const Op &op)
+{
+    const qcd_status st = op(wait);
+    return st == QCD_ERR_OOM && give_back_fixed(g, lat, s) ? op(LINKS_FP64) : st;
+}
 Reduction reduction_of(const qcd_lattice *lat);
 
 cudaError_t launch_dslash(int prec, int recon, const DslashLaunch &a, cudaStream_t s);

@@ -493,8 +493,19 @@ FieldView half_of(const FieldView &f, int k)
 // field's own); it must have the gauge field's extents, and x, b must live
 // on it.  Separate contexts let solves that share one resident gauge field
 // run concurrently on different streams.
+static qcd_status solve_with(LinkWait wait, const qcd_gauge *g, qcd_spinor *const *x, const qcd_spinor *const *b, int nrhs,
+                             const qcd_solver_params *prm, qcd_solver_stats *stats, cudaStream_t s, const qcd_lattice *ctx);
+
 qcd_status qcd::solve_impl(const qcd_gauge *g, qcd_spinor *const *x, const qcd_spinor *const *b, int nrhs,
                       const qcd_solver_params *prm, qcd_solver_stats *stats, cudaStream_t s, const qcd_lattice *ctx)
+{
+    if (!g) return fail(QCD_ERR_INVALID_ARG, "solve_cg: NULL argument");
+    return with_memory(g, ctx ? ctx : g->lat, s, LINKS_SETTLE,
+                       [&](LinkWait wait) { return solve_with(wait, g, x, b, nrhs, prm, stats, s, ctx); });
+}
+
+static qcd_status solve_with(LinkWait wait, const qcd_gauge *g, qcd_spinor *const *x, const qcd_spinor *const *b, int nrhs,
+                             const qcd_solver_params *prm, qcd_solver_stats *stats, cudaStream_t s, const qcd_lattice *ctx)
 {
     const auto t0 = std::chrono::steady_clock::now();
     if (!g || !x || !b || !prm) return fail(QCD_ERR_INVALID_ARG, "solve_cg: NULL argument");
@@ -539,7 +550,7 @@ qcd_status qcd::solve_impl(const qcd_gauge *g, qcd_spinor *const *x, const qcd_s
     // arithmetic costs more than the bytes it saves)
     const int srecon = !mixed ? g->recon : (sp == QCD_PREC_DF64 ? 18 : prm->inner_recon);
     qcd_status st;
-    HopLinks links = hop_links(g, QCD_PREC_F64, g->recon, s, true, &st);
+    const HopLinks links = hop_links(g, QCD_PREC_F64, g->recon, s, wait, &st);
     if (st != QCD_OK) return st;
     GaugeView Uh = links.form[0];
     GaugeView Us = mixed ? gauge_view(g, sp, srecon, s, &st) : Uh;

@@ -454,6 +454,7 @@ NORM2_NOALLOC_MAX = 16_777_216
 
 
 INJECT_SPINOR_CREATE = 1
+INJECT_WORKSPACE = 2
 
 
 def set_hop_threads(threads_per_site: int):
