@@ -102,6 +102,30 @@ def test_many_barrier_timeout_is_reported(q, problems):
     assert status == 0 and all(st["true_rel_residual"] <= 1e-10 for st in stats)
 
 
+def test_many_timeout_ends_systems_of_one_block(q):
+    """A system with a single block has no barrier wait to run out.  It returns
+    all the same when another system's wait does, instead of going on to
+    maxiter (its target here is out of reach: 4000 iterations take a second)."""
+    import time
+    probs = []
+    for dims, seed in (((8, 8, 8, 8), 741), ((4, 4, 4, 4), 742)):
+        lat = q.Lattice(dims, -1)
+        g = q.Gauge(lat, "f64", 18)
+        g.upload(syn.gauge_field(dims, 0.2, seed))
+        b, x = q.Spinor(lat, "full", "f64"), q.Spinor(lat, "full", "f64")
+        b.upload(syn.gaussian_spinor(dims, seed))
+        probs.append((g, x, b))
+    g, x, b = zip(*probs)
+    seconds = []
+    for _ in range(2):  # (the first call also allocates)
+        t0 = time.perf_counter()
+        status, _ = q.solve_cg_many(g, x, b, [0.13, 0.13], None, [1e-10, 1e-17], maxiter=4000, wait_cycles=1,
+                                    max_blocks=12, raise_on_error=False)  # nine blocks and one
+        seconds.append(time.perf_counter() - t0)
+        assert status == 6  # QCD_ERR_TIMEOUT
+    assert seconds[1] < 0.1
+
+
 def test_many_rejects_bad_arguments(q, problems):
     p = problems[0]
     x = q.Spinor(p["lat"], "full", "f64")
