@@ -1479,6 +1479,8 @@ qcd_status qcd_apply_dslash_multi(const qcd_gauge *g, qcd_spinor *const *out, co
         if (out[k]->prec != in[0]->prec || in[k]->prec != in[0]->prec || out[k]->parity != out[0]->parity ||
             in[k]->parity != in[0]->parity)
             return fail(QCD_ERR_INVALID_ARG, "apply_dslash_multi: fields must share precision and parity");
+        if (out[k]->ks || in[k]->ks)
+            return fail(QCD_ERR_INVALID_ARG, "apply_dslash_multi: staggered fields need qcd_apply_dslash_ks");
         if (out[k]->data == in[k]->data) return fail(QCD_ERR_INVALID_ARG, "apply_dslash_multi: out aliases in");
     }
     const bool both = out[0]->parity == QCD_PARITY_FULL && in[0]->parity == QCD_PARITY_FULL;

@@ -54,3 +54,15 @@ def test_multi_output_is_another_input(q, prec, recon):
     q.apply_dslash_multi(g, ins[1:] + ins[:1], ins)
     for k, v in enumerate(psi):
         assert F.rel_err(ins[(k + 1) % 3].download(), oracle.dhop(U, v)) <= TOL[prec], k
+
+
+@pytest.mark.parametrize("staggered", ["in", "out"])
+def test_multi_rejects_staggered_fields(q, staggered):
+    """Three complex a site instead of twelve: refused, not read past their end."""
+    lat = q.Lattice((4, 4, 2, 4), -1)
+    g = q.Gauge(lat, "f64", 18)
+    ins = [q.Spinor(lat, "odd", "f32", ks=staggered == "in" and k == 1) for k in range(2)]
+    outs = [q.Spinor(lat, "even", "f32", ks=staggered == "out" and k == 1) for k in range(2)]
+    with pytest.raises(q.QcdError) as e:
+        q.apply_dslash_multi(g, outs, ins)
+    assert e.value.status == 1
