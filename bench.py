@@ -261,8 +261,9 @@ def dslash_sweep(qcd, torch, flush, hbm, reps=20, fields=None):
     also back-to-back cold launches over three such sets."""
     from paper_1411_5219_gb300 import synthetic as syn
     out = {}
-    fmts = [("f64", 18, 1536), ("f64", 12, 1152), ("f32", 12, 576), ("f16", 12, 296), ("bf16", 12, 288),
-            ("f64", 8, 896), ("f32", 8, 448), ("f16", 8, 232), ("bf16", 8, 224)]
+    # bytes per output site (F64 reads 18 reals a link from its fixed-point copy, whatever the field holds)
+    fmts = [("f64", 18, 1536), ("f64", 12, 1536), ("f32", 12, 576), ("f16", 12, 296), ("bf16", 12, 288),
+            ("f64", 8, 1536), ("f32", 8, 448), ("f16", 8, 232), ("bf16", 8, 224)]
     for dims in syn.SWEEP_VOLUMES:
         lat = qcd.Lattice(dims, -1)
         U = syn.gauge_field(dims, 0.2, 1002)

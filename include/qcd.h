@@ -433,13 +433,16 @@ void qcd_server_destroy(qcd_server *sv);
 /* The paper's kernel classes carry the number of FLOPs each kernel performs
  * so that performance can be reported (Sec. 4), and it rates the Dslash by
  * its achieved memory bandwidth (Sec. 1, Sec. 6).  Between
- * qcd_profile_begin and qcd_profile_end every hopping-kernel launch is
+ * qcd_profile_begin and qcd_profile_end every hopping-kernel launch, with
+ * the passes that bring its fields into the form that the kernel reads, is
  * bracketed by CUDA events on its own stream, and its algorithmic traffic
  * and flops are recorded:
  *   bytes = sites * (8 links + 1 input spinor + 1 output spinor
  *                    [+ 1 spinor y of the fused epilogue]),
- *           in the storage precision (links at 18 or 12 reals; FP16
- *           spinors include their 4-byte scale);
+ *           in the storage precision (links at 18, 12 or 8 reals, in F64
+ *           at the 18 of the fixed-point copy where the kernel reads that;
+ *           FP16 spinors include their 4-byte scale; those passes add
+ *           nothing);
  *   flops = 1320 per output site (projection, two SU(3) products and the
  *           accumulation of 8 hops; the rebuilt third link row and the
  *           epilogue are not counted).

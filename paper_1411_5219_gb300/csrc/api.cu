@@ -745,8 +745,9 @@ bool fixed_hops(const qcd_lattice *lat, const GaugeView &U, int prec, int recon,
     return prec == QCD_PREC_F64 && U.fix && (tuned_tpb(lat, U, prec, recon, L, both, s) >> 16) != 8;
 }
 
-// One hopping launch, recorded with its time inside a profiling window: `sites`
-// output sites of n right-hand sides, `fields` spinors read or written each.
+// One hopping launch with the conversions of its fields, recorded with its time
+// inside a profiling window: `sites` output sites of n right-hand sides, `fields`
+// spinors read or written each.
 template <typename Launch>
 static cudaError_t profiled(int prec, int recon, double sites, int n, int fields, cudaStream_t s, const Launch &launch)
 {
@@ -809,12 +810,14 @@ static cudaError_t hop_df64(const qcd_lattice *lat, const GaugeView &U, int reco
     f.in = &in;
     f.out = &out;
     f.y = h.y ? &y : nullptr;
-    f.count_as = QCD_PREC_DF64;
-    cudaError_t e = launch_convert(in, *h.in, s);
-    if (e == cudaSuccess && h.y) e = launch_convert(y, *h.y, s);
-    if (e == cudaSuccess) e = hop(lat, U, recon, f, s);
-    if (e == cudaSuccess) e = launch_convert(*h.out, out, s);
-    return e;
+    f.counted = true;
+    return profiled(QCD_PREC_DF64, recon, lat->h * (double)nh, 1 << L, h.y ? 3 : 2, s, [&] {
+        cudaError_t e = launch_convert(in, *h.in, s);
+        if (e == cudaSuccess && h.y) e = launch_convert(y, *h.y, s);
+        if (e == cudaSuccess) e = hop(lat, U, recon, f, s);
+        if (e == cudaSuccess) e = launch_convert(*h.out, out, s);
+        return e;
+    });
 }
 
 cudaError_t hop(const qcd_lattice *lat, const GaugeView &U, int recon, const HopArgs &h, cudaStream_t s)
@@ -836,8 +839,6 @@ cudaError_t hop(const qcd_lattice *lat, const GaugeView &U, int recon, const Hop
     if (fix && in->prec != kPrecFix) {
         in_ws = fix_input_ws(lat, in->nh, in->rhs_log2);
         if (!in_ws.hv[0].data) return cudaErrorMemoryAllocation;
-        const cudaError_t e = launch_convert(in_ws, *in, s);
-        if (e != cudaSuccess) return e;
         in = &in_ws;
     }
     DslashLaunch a;
@@ -895,8 +896,14 @@ cudaError_t hop(const qcd_lattice *lat, const GaugeView &U, int recon, const Hop
     a.red_out = lat->red_out;
     a.check_status = h.check_status;
     a.run_status = h.run_status;
-    return profiled(h.count_as ? h.count_as : prec, recon, lat->h * (h.both ? 2.0 : 1.0), 1 << h.out->rhs_log2, h.y ? 3 : 2, s,
-                    [&] { return launch_dslash(prec, recon, a, s); });
+    const auto launch = [&] {
+        const cudaError_t e = in == h.in ? cudaSuccess : launch_convert(*in, *h.in, s);
+        return e == cudaSuccess ? launch_dslash(prec, recon, a, s) : e;
+    };
+    if (h.counted) return launch();
+    // (the fixed-point copy has all nine entries of a link)
+    return profiled(prec, a.U.fix && prec == QCD_PREC_F64 ? 18 : recon, lat->h * (h.both ? 2.0 : 1.0), 1 << h.out->rhs_log2,
+                    h.y ? 3 : 2, s, launch);
 }
 
 }  // namespace qcd
@@ -1553,11 +1560,10 @@ static qcd_status dslash_multi(const qcd_gauge *g, qcd_spinor *const *out, const
             a.dst[k] = static_cast<char *>(out[k]->data);
             a.dst_norm[k] = out[k]->norm;
         }
-        cudaError_t e = cudaSuccess;
+        FieldView f;
         if (prec == QCD_PREC_F64) {
             char *ws = static_cast<char *>(workspace(lat, "dm_fix", nrhs * (fd + fn)));
             if (!ws) return each_field(with_fix_input(lat, U, prec, g->recon, 0, both, s), 0);
-            FieldView f;
             f.nh = nh;
             f.h = lat->h;
             f.prec = kPrecFix;
@@ -1565,7 +1571,6 @@ static qcd_status dslash_multi(const qcd_gauge *g, qcd_spinor *const *out, const
             for (int h = 0; h < 2; ++h)
                 f.hv[h] = SpinorView{ws + (h < nh ? h : 0) * (fd / nh),
                                      reinterpret_cast<float *>(ws + nrhs * fd + (h < nh ? h : 0) * (fn / nh)), lat->stride};
-            e = launch_fix_set(f, fd, fn, pv, nrhs, s);
             for (int k = 0; k < nrhs; ++k) {
                 a.src[k] = ws + k * fd;
                 a.src_norm[k] = reinterpret_cast<const float *>(ws + nrhs * fd + k * fn);
@@ -1575,9 +1580,11 @@ static qcd_status dslash_multi(const qcd_gauge *g, qcd_spinor *const *out, const
                 a.src_norm_off[p] = both ? (1 - p) * (fn / nh) : 0;
             }
         }
-        if (e == cudaSuccess)
-            e = profiled(prec, g->recon, lat->h * (both ? 2.0 : 1.0), nrhs, 2, s,
-                         [&] { return launch_dslash_multi(prec, g->recon, a, s); });
+        const int recon = prec == QCD_PREC_F64 ? 18 : g->recon;  // (the fixed-point copy has all nine entries)
+        const cudaError_t e = profiled(prec, recon, lat->h * (both ? 2.0 : 1.0), nrhs, 2, s, [&] {
+            const cudaError_t c = prec == QCD_PREC_F64 ? launch_fix_set(f, fd, fn, pv, nrhs, s) : cudaSuccess;
+            return c == cudaSuccess ? launch_dslash_multi(prec, g->recon, a, s) : c;
+        });
         return e == cudaSuccess ? each_field(U, 1) : check_cuda(e, "apply_dslash_multi");
     }
     int L = 0;

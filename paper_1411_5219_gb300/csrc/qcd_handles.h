@@ -190,7 +190,7 @@ struct HopArgs {
     const double *coef;    // device table of cy, cd (8 doubles) read at run time, or nullptr
     const float *coef_f;   // its float image (same layout; required with coef)
     int coef_stride;       // doubles between the tables of consecutive rhs (0: shared)
-    int count_as;          // precision that a profiling window counts the launch under (0: the fields')
+    bool counted;          // part of what a profiling window counts already
     int run_status;        // with check_status: run only under this CG status (default CG_RUNNING = 0)
 };
 cudaError_t hop(const qcd_lattice *lat, const GaugeView &U, int recon, const HopArgs &h, cudaStream_t s);
