@@ -723,9 +723,11 @@ static qcd_status solve_with(LinkWait wait, const qcd_gauge *g, qcd_spinor *cons
         QCD_TRY(cudaGraphLaunch(exec, s), "solve_cg: graph launch");
         QCD_TRY(read_state(lat, s), "solve_cg: state");
         // kernels the graph ran: per trip the iteration, per reliable update
-        // its body
+        // its body (with the fixed-point hops' conversions of x and, mixed, of
+        // the field that Mhat^dag takes)
         const int op = c.eo ? 4 : 2;
-        const int per_update = split ? (c.eo ? 10 : 7) + (mid ? 1 : 0) : op + 2 + (mixed ? 1 : 0);
+        const int per_update = (split ? (c.eo ? 10 : 7) + (mid ? 1 : 0) : op + 2 + (mixed ? 1 : 0)) +
+                               (fix ? (mixed ? 2 : 1) : 0);
         note_launches((lat->state_host->trips + lat->state_host->skipped) * (op + 2) + lat->state_host->reliable_updates * per_update);
     } else {
         QCD_TRY(cg_eager(lat, F, s), "solve_cg: iterations");

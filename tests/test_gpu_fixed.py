@@ -145,3 +145,23 @@ def test_fixed_solves(q, mu, nrhs, eo):
         assert stats[k]["true_rel_residual"] <= 1e-11
         want, _ = oracle.solve_eo(U, src[k], kappa, mu, tol=1e-13)
         assert F.rel_err(xs[k].download(), want) < 1e-9
+
+
+@pytest.mark.parametrize("inner,per_update", [("f64", 1), ("f16", 2)])
+def test_launch_count_of_a_solve_holds_the_conversions(q, inner, per_update):
+    """The thread pairs convert FP64 inputs in launches of their own, the lanes do
+    not: three outside the loop (source, odd sites, residual), and per reliable
+    update x and, in mixed precision, the defect."""
+    dims = (4, 6, 4, 4)
+    lat, U, g = _gauge(q, dims)
+    b, x = q.Spinor(lat, "full", "f64"), q.Spinor(lat, "full", "f64")
+    b.upload(syn.gaussian_spinor(dims, 1520))
+    count = {}
+    for tps in (8, 1):
+        q.set_hop_threads(tps)
+        for _ in range(2):  # (the first solve builds its graph)
+            n0 = q.kernel_launches()
+            _, st = q.solve_cg(g, x, b, 0.14, 0.02, tol=1e-10, inner_prec=inner)
+            count[tps] = q.kernel_launches() - n0, st["iterations"], st["reliable_updates"]
+    assert count[1][1:] == count[8][1:]
+    assert count[1][0] - count[8][0] == 3 + per_update * count[1][2]
