@@ -1,9 +1,11 @@
-"""The FP64 reconstruct-18 hopping kernel with eight threads per output site
-(one hop direction each, summed by warp shuffles) against the FP64 oracle,
-forced through qcd_set_hop_threads(8): the even-odd and full-lattice Dslash
-of both parities with and without dagger, the Schur operator with twisted
-mass (the fused epilogues and the fused norm), and FP64 and mixed solves.
-The one-thread-per-site kernel, forced with 1, agrees to rounding.
+"""The lane hopping kernels, forced through qcd_set_hop_threads(8), against the
+FP64 oracle: one hop direction per thread, summed by warp shuffles.  The links
+here are SU(3), so sixteen threads per site run in fixed point (eight in FP64
+arithmetic for other links: test_gpu_fp64_links.py).  The even-odd and
+full-lattice Dslash of both parities with and without dagger, the Schur
+operator with twisted mass (the fused epilogues and the fused norm), and FP64
+and mixed solves.  The kernel of large lattices, forced with 1, agrees to
+rounding.
 """
 
 import numpy as np
@@ -101,7 +103,7 @@ def test_lanes8_apply_m_full_and_schur(q, lanes, kappa, mu, dagger):
 @pytest.mark.parametrize("kappa,mu", [(0.155, 0.0), (0.16, 0.01)])
 def test_lanes8_solve_matches_oracle(q, lanes, inner, kappa, mu):
     """The CG's fused operator + norm launches and the FP64 defect and
-    verification of the mixed solver all take the eight-lane kernel."""
+    verification of the mixed solver all take the lane kernel."""
     lanes(8)
     dims = (8, 8, 8, 4)
     lat, U, g = _gauge(q, dims, eps=0.2, seed=1205)
@@ -119,7 +121,7 @@ def test_lanes8_solve_matches_oracle(q, lanes, inner, kappa, mu):
 
 
 def test_lanes8_graph_and_eager_bitwise(q, lanes):
-    """A captured solve replays the eight-lane launches with the same bits."""
+    """A captured solve replays the lane launches with the same bits."""
     lanes(8)
     dims = (6, 4, 2, 8)
     lat, U, g = _gauge(q, dims, eps=0.2, seed=1207)
