@@ -369,8 +369,8 @@ cudaError_t cg_eager(const qcd_lattice *lat, const CgFields &f, cudaStream_t s)
 // (the kernels of the ones after it return at once).  The last kernel of either sets the loop condition, true while the
 // state is RUNNING (bounded by iter < maxiter and a trip cap); control kernels
 // of their own cost two launches an iteration.  Built once per
-// configuration and field addresses and cached on the lattice.
-qcd_status cg_graph(const qcd_lattice *lat, const CgFields &f, cudaGraphExec_t *out)
+// configuration, launch shapes and field addresses and cached on the lattice.
+qcd_status cg_graph(const qcd_lattice *lat, const CgFields &f, int shape_h, int shape_s, cudaGraphExec_t *out)
 {
     char key[512];
     snprintf(key, sizeof(key), "%d|%d|%p|%d|%d|%d|%p|%p|%p|%p|%p|%p|%p|%p|%p|%p|%p|%p|%p|%p|%d|%d", (int)f.c.eo,
@@ -379,8 +379,9 @@ qcd_status cg_graph(const qcd_lattice *lat, const CgFields &f, cudaGraphExec_t *
              f.rs.hv[0].data, f.ps.hv[0].data, f.qs.hv[0].data, f.ts.hv[0].data, f.ss.hv[0].data, f.xs.hv[0].data,
              (void *)f.state, f.rs.prec, f.rhs.nh);
     const size_t used = strlen(key);
-    snprintf(key + used, sizeof(key) - used, "|%p|%d|%d|%p|%d|%p|%p|%p", (void *)f.red.partials, f.rs.rhs_log2,
-             (int)f.split, f.rhs0.hv[0].data, (int)f.mid, f.Um.data, f.r_m.hv[0].data, (const void *)f.Uh.fix);
+    snprintf(key + used, sizeof(key) - used, "|%p|%d|%d|%p|%d|%p|%p|%p|%x|%x", (void *)f.red.partials, f.rs.rhs_log2,
+             (int)f.split, f.rhs0.hv[0].data, (int)f.mid, f.Um.data, f.r_m.hv[0].data, (const void *)f.Uh.fix,
+             (unsigned)shape_h, (unsigned)shape_s);
     auto it = lat->graphs.find(key);
     if (it != lat->graphs.end()) {
         it->second.last_use = ++lat->graph_clock;
@@ -711,10 +712,10 @@ static qcd_status solve_with(LinkWait wait, const qcd_gauge *g, qcd_spinor *cons
     qcd_status result = QCD_OK;
     if (!profiling_active()) {
         // choose the kernels' launch shapes before they are frozen in the graph
-        tuned_tpb(lat, Us, sp, srecon, L, !c.eo, s);
-        if (mixed) tuned_tpb(lat, Uh, QCD_PREC_F64, g->recon, L, !c.eo, s);
+        const int shape_s = tuned_tpb(lat, Us, sp, srecon, L, !c.eo, s);
+        const int shape_h = mixed ? tuned_tpb(lat, Uh, QCD_PREC_F64, g->recon, L, !c.eo, s) : shape_s;
         cudaGraphExec_t exec = nullptr;
-        if (cg_graph(lat, F, &exec) != QCD_OK) {
+        if (cg_graph(lat, F, shape_h, shape_s, &exec) != QCD_OK) {
             // the capture failed (e.g. invalidated by another thread): run
             // the same kernels eagerly instead
             QCD_TRY(cg_eager(lat, F, s), "solve_cg: iterations");

@@ -9,6 +9,7 @@ products of each component's eight neighbours, in FP64 on both sides, so the
 2-norm errors stay below a few 2^-53 of the result; double-float a few 2^-48.
 """
 
+import numpy as np
 import pytest
 
 import oracle
@@ -139,3 +140,24 @@ def test_many(q):
     for k in range(3):
         assert stats[k]["true_rel_residual"] <= 1e-11
         assert schur_residual_oracle(Us[k], vs[k], x[k].download(), kappa[k], mu[k]) <= 1.5e-11
+
+
+@pytest.mark.parametrize("first,then", [(1, 8), (8, 1)])
+def test_solve_takes_the_shape_set_last(q, first, then):
+    """A solve after qcd_set_hop_threads does not replay the graph of one before
+    it: the bits are those of a lattice that only knows the later setting."""
+    dims = (6, 4, 2, 8)
+    b = syn.gaussian_spinor(dims, 2091)
+    out = []
+    try:
+        for settings in ((first, then), (then,)):
+            lat, U, g = _gauge(q, dims, seed=2090)
+            bs, x = q.Spinor(lat, "full", "f64"), q.Spinor(lat, "full", "f64")
+            bs.upload(b)
+            for tps in settings:
+                q.set_hop_threads(tps)
+                q.solve_cg(g, x, bs, 0.14 / SCALE, 0.02 * SCALE)
+            out.append(x.download())
+    finally:
+        q.set_hop_threads(0)
+    assert np.array_equal(out[0], out[1])
