@@ -46,6 +46,14 @@
  *   - Work on handles of the same lattice must be ordered on one stream:
  *     a lattice handle owns the scratch (reductions, staging, solver
  *     fields) that these calls share.
+ *   - Operator calls may be captured into a CUDA graph of the caller.  A replay
+ *     of an F64 operator applies the links that the field holds then, uploads
+ *     after the capture included.  Captured before an eager call of its kind (or
+ *     qcd_gauge_prepare) it runs in FP64 arithmetic; so do all F64 operators on
+ *     a field whose upload was captured, since its replays change the links
+ *     unseen.  Captured double-float operators, and those of other precisions
+ *     than the field's, hold a derived copy that the next upload frees: capture
+ *     them again after it.
  */
 #ifndef QCD_H
 #define QCD_H
@@ -71,9 +79,12 @@ typedef int qcd_status;
  * real as the unevaluated sum hi + lo of two FP32 numbers (8 bytes, ~48
  * significant bits) and its kernels compute in pairs of FP32 numbers with
  * error-free transformations: FP64-accurate to ~1e-14 at FP32 instruction
- * rates, since GB300 runs FP32 58x faster than FP64.  The paper computes all
- * in double precision (Sec. 4); DF64 is this library's way to do so on
- * GB300 and is always labelled as such. */
+ * rates, since GB300 runs FP32 58x faster than FP64.  Operator calls on an F64
+ * gauge field of 18 reals a link take the fixed-point FP64 hop instead, which
+ * is faster and closer (its result rounded to DF64), except under stream
+ * capture; the solver's inner iterations keep to FP32 pairs.  The paper
+ * computes all in double precision (Sec. 4); DF64 is this library's way to do
+ * so on GB300 and is always labelled as such. */
 typedef enum { QCD_PREC_F64 = 0, QCD_PREC_F32 = 1, QCD_PREC_F16 = 2, QCD_PREC_BF16 = 3, QCD_PREC_DF64 = 4 } qcd_prec;
 /* Link storage: 18 reals (full matrix), 12 (rows 0 and 1; row 2 is
  * rebuilt as conj(row0 x row1), exact for SU(3)) or 8.  Reconstruct-8 is
@@ -132,8 +143,9 @@ void qcd_lattice_destroy(qcd_lattice *lat);
  * INVALID_ARG; OOM; CUDA. */
 qcd_status qcd_gauge_create(const qcd_lattice *lat, qcd_prec prec, qcd_recon recon, qcd_gauge **out);
 /* Copy a host gauge field (host layout above, 4*V*9 complex doubles) to
- * the device and convert it; drops derived copies.  Recon-12 and recon-8
- * assume SU(3) links.  Errors: INVALID_ARG (NULL; recon-8 links out of
+ * the device and convert it; drops derived copies, and writes the fixed-point
+ * copy of an F64 field again, where there is one, in stream order.  Recon-12
+ * and recon-8 assume SU(3) links.  Errors: INVALID_ARG (NULL; recon-8 links out of
  * reach, see qcd_recon); CUDA. */
 qcd_status qcd_gauge_upload(qcd_gauge *g, const double *host, void *stream);
 /* Build (if missing) the derived copy used by kernels of precision
@@ -189,11 +201,15 @@ qcd_status qcd_spinor_norm2(const qcd_spinor *s, double *result_device, void *st
 void qcd_spinor_destroy(qcd_spinor *s);
 
 /* out[k] = D_hop in[k] (dagger: D_hop^dagger in[k]) for k < nrhs (1..32): the
- * same parity rules as qcd_apply_dslash, all fields of one precision.  The
- * right-hand sides are gathered into one batched field (the rhs index
- * fastest inside each plane) so that a single launch reads each link once
- * for all of them; the results are scattered back.  Errors: INVALID_ARG;
- * OOM; CUDA. */
+ * same parity rules as qcd_apply_dslash, all fields of one precision.  One
+ * launch reads and writes the fields where they lie, its blocks taking the
+ * fields of the same sites one after the other so that links come from L2
+ * (F64: through fixed-point copies of the inputs, made by one more launch;
+ * under stream capture a launch per field).  Where an output overlaps another
+ * right-hand side's input, for DF64, and for F64 links outside the fixed-point
+ * form, the inputs are gathered into one batched field (the rhs index fastest
+ * inside each plane) and the results scattered back.  Errors: INVALID_ARG; OOM;
+ * CUDA. */
 qcd_status qcd_apply_dslash_multi(const qcd_gauge *g, qcd_spinor *const *out, const qcd_spinor *const *in, int nrhs,
                                   int dagger, void *stream);
 
@@ -221,10 +237,19 @@ qcd_status qcd_norm2_noalloc(const double *x_device, size_t n, double *result_de
  * (Sec. 1 and 6).  With out of parity p (EVEN or ODD) and in of parity 1-p
  * this is the block D_eo (p = EVEN) or D_oe (p = ODD); with both FULL it is
  * the hopping term on the whole lattice.  out and in share the precision
- * (F64: sums of 60-bit fixed-point products, no less exact than FP64
- * arithmetic, which links with entries above 1 and sites with extreme or
- * non-finite values take; F32/F16/BF16: FP32 arithmetic); the gauge field's
- * copy in that precision and with the gauge field's recon is used.
+ * (F64: sums of 60-bit fixed-point products, see below; F32/F16/BF16: FP32
+ * arithmetic); the gauge field's copy in that precision and with the gauge
+ * field's recon is used.
+ * F64: each real of the result is off by less than 2^-48 (measured: 2^-50.6) of
+ * the largest real in the spinors of the eight neighbouring sites.  In the
+ * 2-norm that is closer to exact than FP64 arithmetic (5e-17 of the result
+ * against 1.6e-16 on Gaussian fields), and most components are too, but not
+ * each one: a component that stays far below the others of its sites, as with
+ * unit or diagonal links, has about as many bits fewer than 56 as it lies below
+ * them, where FP64 arithmetic keeps 53 (fields whose components spread over
+ * twelve orders of magnitude: at worst 2^-34 of the component against 2^-47 with
+ * unit links, 2^-42 against 2^-46 on links exp(0.2 i H)).  Links with entries
+ * above 1 and sites with extreme or non-finite values take FP64 arithmetic.
  * Errors: INVALID_ARG (parities, lattices, precisions); CUDA. */
 qcd_status qcd_apply_dslash(const qcd_gauge *g, qcd_spinor *out, const qcd_spinor *in, int dagger, void *stream);
 
@@ -279,7 +304,9 @@ typedef struct {
  * residual and continues).  Mixed precision runs the inner iterations on
  * fields and links of `inner_prec` (FP32 arithmetic), accumulates x in FP64
  * and replaces the residual by the FP64 true residual at each reliable
- * update.  Blocks until the solve is done.  Returns OK, NOT_CONVERGED
+ * update.  The FP64 hops and, between them, the search direction of an FP64
+ * CG and the operator's temporaries are in fixed point (error bound at
+ * qcd_apply_dslash).  Blocks until the solve is done.  Returns OK, NOT_CONVERGED
  * (maxiter; x and stats written), BREAKDOWN, INVALID_ARG, OOM or CUDA. */
 qcd_status qcd_solve_cg(const qcd_gauge *g, qcd_spinor *x, const qcd_spinor *b, const qcd_solver_params *params,
                         qcd_solver_stats *stats, void *stream);
@@ -311,8 +338,8 @@ qcd_status qcd_solve_cg_batch(const qcd_gauge *g, qcd_spinor *const *x, const qc
  * field, lattice volume, hopping parameter, twisted mass and tolerance --
  * advanced together by ONE persistent cooperative kernel launch (source
  * preparation, CG, FP64 true-residual check, odd-site reconstruction and the
- * full-system residual, separated by grid-wide barriers instead of kernel
- * launches).  Meant for small lattices, where one solve cannot fill the GPU:
+ * full-system residual, separated by barriers over each system's blocks instead
+ * of kernel launches).  Meant for small lattices, where one solve cannot fill the GPU:
  * the paper's finite-temperature studies are many independent runs over
  * couplings and volumes (Sec. 1) within device memory (Sec. 2).
  * gauges[k]: F64 field; x[k], b[k]: FULL F64 spinors on one lattice with the

@@ -679,8 +679,8 @@ int tuned_tpb(const qcd_lattice *lat, const GaugeView &U, int prec, int recon, i
     const int force = g_force_tps.load();
     if (lanes8_ok && force == 8) return kLanes8;
     if (lanes8_ok && force == 1) return 64;
-    // in fixed point by size (FP64 CG, lanes against thread pairs: 12^3 x 4
-    // 1.94 against 2.33 ms, 12^3 x 8 3.05 against 2.68 ms)
+    // in fixed point by size (FP64 CG, lanes against thread pairs: 12^3 x 4, 3456
+    // output sites, 1.61 against 1.98 ms; 12^3 x 6, 5184 sites, 2.45 against 2.24)
     if (lanes8_ok && U.fix) return (both ? 2 : 1) * lat->h <= kLanesMaxSites ? kLanes8 : 64;
     const std::string key = tune_key(lat, prec, recon, L, both);
     {

@@ -24,7 +24,8 @@ __device__ __forceinline__ void copy16(int4 *dst, const int4 *src)
 // next to HBM: with direct loads the compiler keeps no hop ahead in registers
 // (250 us), so each warp copies the next hop's components and links to a
 // two-slot ring in shared memory with cp.async while it multiplies this one
-// (205 us for 1.05 GB, 76 % of HBM; the FP64 kernel took 945 us).  Three slots
+// (205 us for 1.05 GB, 76 % of HBM; the FP64 kernel took 938 us; a call with the
+// conversion of an FP64 input takes 247 us).  Three slots
 // at 12 warps per SM or two at 20 (96 registers, spills) measured slower than
 // two at 16.
 template <int kDagger, int kEpi, bool kReduce, typename Launch = DslashLaunch>

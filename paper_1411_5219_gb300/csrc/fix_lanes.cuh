@@ -2,10 +2,11 @@
 // one spin of the half spinor each, FP64 fields in and out.
 //
 // For small lattices, where a thread's chain of instructions sets the time
-// (the CG at 8^3 x 4: 1.66 ms, 2.30 ms with a thread pair per site, 2.13 ms
-// with eight FP64 lanes; from 12^3 x 8 on the pairs win): a thread converts six of its neighbour's components (the exponent is the
-// largest of the site's neighbourhood, so no sum needs a shift), does one
-// colour vector's product and joins the sums by shuffles.
+// (the CG at 8^3 x 4: 1.29 ms, 1.93 ms with a thread pair per site, 1.85 ms
+// with eight FP64 lanes; from 12^3 x 6 on the pairs win): a thread converts six
+// of its neighbour's components (the exponent is the largest of the site's
+// neighbourhood, so no sum needs a shift), does one colour vector's product and
+// joins the sums by shuffles.
 #pragma once
 
 #include "fixed.cuh"

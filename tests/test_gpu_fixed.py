@@ -2,10 +2,9 @@
 against the FP64 oracle.
 
 qcd_set_hop_threads forces the thread pair per element (1) and the sixteen
-lanes (8) whatever the lattice.  Bounds: the operator's sums round once (2^-53 of
-the result) over inputs held to 2^-56 of their site's largest component,
-far below 1e-15 norm-wise; site by site the error stays below 1e-15 of the
-largest components of the eight neighbours.
+lanes (8) whatever the lattice.  Bounds: norm-wise 1e-15, a few 2^-53 of the
+oracle's own; real by real ten units of 2^-55 of the largest real a hop, 2^-48 of
+the largest over the eight neighbours (csrc/fixed.cuh; the oracle adds about 2^-50).
 """
 
 import numpy as np
@@ -98,6 +97,31 @@ def test_fixed_unusual_values(q, case):
             assert np.all(np.abs(got - want)[fine] <= 1e-15 * bound[fine] + 1e-322)
         if case == "zeros":
             assert np.all(got[bound[:, 0, 0] == 0] == 0)
+
+
+@pytest.mark.parametrize("links", ["su3", "near unit", "unit", "diagonal"])
+@pytest.mark.parametrize("spread", [0, 3, 12])
+def test_component_bound(q, links, spread):
+    """The stated bound of each real, with components of a site spread over
+    orders of magnitude and links that keep them apart."""
+    dims = (8, 6, 4, 6)
+    lat = q.Lattice(dims, -1)
+    U = syn.gauge_field(dims, 0.01 if links == "near unit" else 0.3, 1551)
+    rng = np.random.default_rng(1552)
+    if links in ("unit", "diagonal"):
+        phase = np.zeros(U.shape[:-1]) if links == "unit" else rng.uniform(-np.pi, np.pi, U.shape[:-1])
+        phase[..., 2] = -phase[..., 0] - phase[..., 1]
+        U = np.exp(1j * phase)[..., None] * np.eye(3)
+    g = q.Gauge(lat, "f64", 18)
+    g.upload(U)
+    psi = syn.gaussian_spinor(dims, 1553)
+    psi *= 10.0 ** rng.uniform(-spread, 0, psi.shape)
+    m = np.maximum(np.abs(psi.real), np.abs(psi.imag)).max(axis=(-2, -1))
+    m = np.max([np.roll(m, s, a) for a in range(4) for s in (1, -1)], axis=0)
+    for p in (0, 1):
+        d = _apply(q, lat, g, psi, p) - oracle.dhop_eo(U, syn.to_half(psi, 1 - p), p)
+        bound = syn.to_half(np.broadcast_to(m[..., None, None], psi.shape).astype(complex), p).real
+        assert np.all(np.maximum(np.abs(d.real), np.abs(d.imag)) <= (2.0 ** -48 + 2.0 ** -50) * bound)
 
 
 def test_links_beyond_the_fixed_form_stay_fp64(q):
