@@ -43,6 +43,9 @@ METRIC = "eo-Wilson Dslash GB/s & %HBM roofline; mixed vs FP64 CG solves/s at 1e
 WORKLOAD = "24^3x8"
 TOL = 1e-10
 HBM_FALLBACK_GBS = 6800.0
+# DRAM bytes (read + write) of one fixed-point FP64 D_eo launch at 24^3 x 8 from
+# an ncu capture of the current kernel; set to None when the kernel changes.
+TRAFFIC_F64_D_24 = 77.08e6
 
 
 def workload_config():
@@ -808,8 +811,9 @@ def main():
         "gpu_launches": int(launches),
         "roofline": {"bound": "hbm", "kernel": "FP64 hop in fixed point (D_eo/D_oe with fused epilogues) in the CG",
                      "achieved": achieved, "peak": hbm, "unit": "GB/s",
-                     "frac": achieved / hbm if achieved else None, "traffic": None,
-                     "traffic_note": "achieved counts the algorithmic bytes: 8 links, input, output and epilogue "
+                     "frac": achieved / hbm if achieved else None, "traffic": TRAFFIC_F64_D_24,
+                     "traffic_note": "ncu dram read+write bytes per plain D_eo launch (cold L2; algorithmic 84.93 MB); "
+                                     "achieved counts the algorithmic bytes: 8 links, input, output and epilogue "
                                      "field per site; links and fields partly stay in L2 at this size",
                      "launches": d["launches"], "avg_us": d["ms"] / max(d["launches"], 1) * 1e3,
                      "achieved_TFLOP_s": d["flops"] / (d["ms"] * 1e-3) / 1e12 if d["ms"] > 0 else None,
