@@ -49,8 +49,10 @@
  *   - Operator calls may be captured into a CUDA graph of the caller.  A replay
  *     of an F64 operator applies the links that the field holds then, uploads
  *     after the capture included.  Captured before an eager call of its kind (or
- *     qcd_gauge_prepare) it runs in FP64 arithmetic; so do all F64 operators on
- *     a field whose upload was captured, since its replays change the links
+ *     qcd_gauge_prepare) it runs in FP64 arithmetic, and where it needs a
+ *     temporary (qcd_apply_M with eo = 1; qcd_apply_dslash_multi where it gathers)
+ *     only an eager call provides that; F64 operators on a field whose upload was
+ *     captured run in FP64 arithmetic too, since its replays change the links
  *     unseen.  Captured double-float operators, and those of other precisions
  *     than the field's, hold a derived copy that the next upload frees: capture
  *     them again after it.

@@ -690,7 +690,7 @@ int tuned_tpb(const qcd_lattice *lat, const GaugeView &U, int prec, int recon, i
         if (it != g_tune.end()) return it->second;
     }
     const int fallback = lanes8_ok ? 64 : 128;
-    if (capturing(s)) return fallback;
+    if (U.unfit || capturing(s)) return fallback;  // (a launch that may return at once says nothing)
     const FieldView ti = ws_field(lat, "tune_in", both ? 2 : 1, prec, L);
     const FieldView to = ws_field(lat, "tune_out", both ? 2 : 1, prec, L);
     if (!ti.hv[0].data || !to.hv[0].data || launch_zero(ti, s) != cudaSuccess) return fallback;

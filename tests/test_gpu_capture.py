@@ -248,11 +248,14 @@ def test_captured_upload(q, threads):
 
 
 @pytest.mark.parametrize("scale", [1.0, 4.0])
-def test_first_call_after_an_upload_does_not_wait(q, threads, scale):
+@pytest.mark.parametrize("tps", [0, 1, 8])
+def test_first_call_after_an_upload_does_not_wait(q, tps, scale):
     """Operators queued behind an upload that the GPU has not reached return
-    at once, and apply the uploaded links, in either form."""
+    at once, and apply the uploaded links, in either form and launch shape (0:
+    the library's choice, which is not made by timing such launches)."""
     import time
     import torch
+    q.set_hop_threads(tps)
     lat, U, g, psi = _setup(q, seed=1801)
     calls = [_Call(q, lat, g, psi, kind) for kind in ("half", "full", "mhat", "m")]
     ins, outs = ([q.Spinor(lat, p, "f64") for _ in range(3)] for p in ("odd", "even"))
@@ -274,6 +277,7 @@ def test_first_call_after_an_upload_does_not_wait(q, threads, scale):
         run()
     waited = time.perf_counter() - t0
     q.stream_sync()
+    q.set_hop_threads(0)
     assert waited < 0.5 * (time.perf_counter() - t0)
     for c in calls:
         assert c.error(V) < 1e-15
