@@ -375,7 +375,6 @@ __global__ void __launch_bounds__(kManyThreads, 3) many_cg_kernel(const ManySys 
     const int k = block_sys[blockIdx.x];
     const int lb = blockIdx.x - sys[k].block0;
     const int ht = hop_threads(sys[k]);
-    const bool alone = sys[k].nblocks == 1;
     ManySysState &q = st->s[k];
     int where = 0;
 #define QCD_SYNC(FIN)                                        \
@@ -405,9 +404,6 @@ __global__ void __launch_bounds__(kManyThreads, 3) many_cg_kernel(const ManySys 
     for (;;) {
         // the loop decision is read by every block after the same barrier
         const int status = __ldcg(&q.status);
-        // another system's wait ran out and the call fails: a block that waits
-        // sees it there, the only block of a system has no waits
-        if (alone && __ldcg(&st->error) != 0) return;
         if (status == MS_RUNNING && __ldcg(&q.iter) < st->maxiter) {
             // ---- one CG iteration
             hop_phase(x, k, lb, MC_OP1, 1, false, &ManySys::p, nullptr, &ManySys::t, -1);
@@ -434,6 +430,9 @@ __global__ void __launch_bounds__(kManyThreads, 3) many_cg_kernel(const ManySys 
                 const double rn = chunk_sum(x, 0, k, 12);
                 if (threadIdx.x == 0) {
                     q.iter += 1;
+                    // another system's wait ran out and the call fails: a block that
+                    // waits sees it there, the only block of a system has no waits
+                    if (x.sys[k].nblocks == 1 && *(volatile int *)&x.st->error != 0) q.status = MS_BREAKDOWN;
                     if (q.status == MS_RUNNING) {
                         if (!isfinite(rn)) {
                             q.status = MS_BREAKDOWN;
